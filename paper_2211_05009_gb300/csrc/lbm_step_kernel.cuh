@@ -7,7 +7,8 @@
 //   walls       ring nodes pull at their inner neighbour x_f instead and store
 //               f^eq(rho_f, u_w) + (1 - 1/tau)(f(x_f) - f^eq(rho_f, u_f))           Sec. 2.2 (ii)
 //               -- the non-equilibrium extrapolation rebuilt and collided in one go (the
-//               rebuilt node has moments (rho_f, u_w), so its BGK step is this closed form).
+//               rebuilt node has moments (rho_f, u_w), so its BGK step is this closed form),
+//               computed as the collided x_f plus f^eq(rho_f, u_w) - f^eq(rho_f, u_f).
 // All arithmetic runs on deviations g_j = f_j - w_j, which keeps rounding relative to the flow
 // rather than to the weights.  Every REDUCE launch (the 100th step of a checkpoint interval) also
 // forms sum(rho - 1) and the two sums of Eq. 6 against the snapshot of 100 steps before, and writes
@@ -239,46 +240,17 @@ __device__ __forceinline__ void pull_row(const S* __restrict__ p, int lane, int 
     }
 }
 
-// Deviation equilibrium g^eq_j = w_j (drho + rho A_j), A_j = 3 c.u + 9/2 (c.u)^2 - 3/2 u.u (Eq. 2).
-template <typename C>
-__device__ __forceinline__ void geq9(C drho, C rho, C ux, C uy, C (&e)[9]) {
-    const C usq = C(1.5) * (ux * ux + uy * uy);
-    const C w0 = C(4.0 / 9.0), w1 = C(1.0 / 9.0), w5 = C(1.0 / 36.0);
-    auto A = [&](C cu) { return cu * (C(3.0) + C(4.5) * cu) - usq; };
-    const C up = ux + uy, um = ux - uy;
-    e[0] = w0 * (drho - rho * usq);
-    e[1] = w1 * (drho + rho * A(ux));
-    e[2] = w1 * (drho + rho * A(uy));
-    e[3] = w1 * (drho + rho * A(-ux));
-    e[4] = w1 * (drho + rho * A(-uy));
-    e[5] = w5 * (drho + rho * A(up));
-    e[6] = w5 * (drho + rho * A(-um));
-    e[7] = w5 * (drho + rho * A(-up));
-    e[8] = w5 * (drho + rho * A(um));
-}
-
-// BGK collision of a fluid node, f*_j = g_j + omega (g^eq_j - g_j) with g^eq_j = w_j (drho + rho A_j)
-// (Eq. 1, Eq. 2), written per opposite pair (j, jbar): A = c2 +- 3 c.u with c2 = 9/2 (c.u)^2 - usq,
-// so a pair shares c2, drho + rho c2 and 3 rho c.u.  About 50 operations per node instead of the
-// 65 of forming all nine g^eq and then relaxing towards them.  ow = omega w for the three weights.
-template <typename C>
-__device__ __forceinline__ void collide_pairs(C drho, C rho, C ux, C uy, C omega, C ow0, C ow1, C ow5,
-                                              const C (&g)[9], C (&out)[9]) {
-    const C usq = C(1.5) * (ux * ux + uy * uy);
-    const C r3 = C(3.0) * rho;
-    out[0] = fma(ow0, fma(-rho, usq, drho), fma(-omega, g[0], g[0]));
-    auto pair = [&](int a, int b, C cu, C ow) {
-        const C c2 = fma(C(4.5) * cu, cu, -usq);
-        const C base = fma(rho, c2, drho);
-        const C sft = r3 * cu;
-        out[a] = fma(ow, base + sft, fma(-omega, g[a], g[a]));
-        out[b] = fma(ow, base - sft, fma(-omega, g[b], g[b]));
-    };
-    pair(1, 3, ux, ow1);
-    pair(2, 4, uy, ow1);
-    pair(5, 7, ux + uy, ow5);
-    pair(8, 6, ux - uy, ow5);
-}
+// Arithmetic with the rounding of each operation spelled out: every kernel that advances a node
+// (row step, batch, fused march) must give bitwise the same populations, so none of them may leave
+// the choice of contractions to the compiler.
+__device__ __forceinline__ float radd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float rsub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float rmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float rfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double radd(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double rsub(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ double rmul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double rfma(double a, double b, double c) { return __fma_rn(a, b, c); }
 
 template <typename C>
 __device__ __forceinline__ C rcp(C v);
@@ -291,7 +263,134 @@ template <> __device__ __forceinline__ float rcp<float>(float v) {
     const float e = fmaf(-v, r, 1.0f);
     return fmaf(r, e, r);
 }
-template <> __device__ __forceinline__ double rcp<double>(double v) { return __drcp_rn(v); }
+// FP64: hardware estimate of 1/v (relative error below 2^-20) refined by one third-order step of
+// Householder's family, r (1 + e + e^2) with e = 1 - v r: the error e^3 is below 2^-60, so three
+// FP64 operations give 1/v to the last bit or the one beside it.  Densities are near 1 here; an
+// infinity or NaN comes out as NaN, which the checkpoint reports.
+template <> __device__ __forceinline__ double rcp<double>(double v) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(v));
+    const double e = __fma_rn(-v, r, 1.0);
+    return __fma_rn(r, __fma_rn(e, e, e), r);
+}
+
+// Constants of the collision for one cavity.
+template <typename C>
+struct Relax {
+    C keep;         // 1 - omega
+    C ow0, ow1, ow5;  // omega w_j
+    C half;         // omega / 2
+};
+template <typename C>
+__device__ __forceinline__ Relax<C> make_relax(C omega) {
+    Relax<C> k;
+    k.keep = rsub(C(1.0), omega);
+    k.ow0 = rmul(omega, C(4.0 / 9.0));
+    k.ow1 = rmul(omega, C(1.0 / 9.0));
+    k.ow5 = rmul(omega, C(1.0 / 36.0));
+    k.half = rmul(omega, C(0.5));
+    return k;
+}
+
+// Moments (Eq. 3) and BGK collision (Eq. 1, Eq. 2) of a fluid node on deviations g = f - w.
+// Both forms work on the opposite pairs (j, jbar) = (1,3) (2,4) (5,7) (8,6) with sum s and
+// difference d, on the momentum j = rho u and on a = j_x u_x, b = j_y u_y, c = j_x u_y; the
+// equilibrium of a pair is w (q +- 3 c_j.j) with q = drho + 9/2 (c_j.u)(c_j.j) - 3/2 (a + b):
+// q_1 = drho + 3a - 3/2 b, q_2 = drho + 3b - 3/2 a, q_5/8 = drho + 3(a + b) +- 9c.
+//
+// FP32 arithmetic (every storage type but FP64): 68 FP32 operations.  The increment of a pair is
+// sigma +- delta, sigma = omega/2 (s^eq - s), delta = omega/2 (d^eq - d).  The differences relax
+// linearly (d^eq_5 = (j_x + j_y)/6, d^eq_8 = (j_x - j_y)/6), and delta_1, delta_2 and the rest
+// population take what makes the increment carry no momentum and no mass: in FP32 the rounding of
+// the weights otherwise shifts both by a few ulps in the same direction every step, which is what
+// dominated the velocity error (1e-5 U over 1000 steps).
+//
+// FP64: 54 FP64 operations (72.7 instructions with the equilibrium formed per direction): the pipe
+// issues 2 lanes per clock and SM, so the operation count is the run time (2048^2: 7.3 GLUPS then).
+// out = keep g + (omega g^eq) with the pair's omega g^eq from two fused multiply-adds.
+template <typename C>
+__device__ __forceinline__ void collide(const C (&g)[9], C one_ref, const Relax<C>& k, C (&out)[9], C& drho,
+                                        C& rho, C& ux, C& uy) {
+    const C s1 = radd(g[1], g[3]), d1 = rsub(g[1], g[3]);
+    const C s2 = radd(g[2], g[4]), d2 = rsub(g[2], g[4]);
+    const C s5 = radd(g[5], g[7]), d5 = rsub(g[5], g[7]);
+    const C s8 = radd(g[8], g[6]), d8 = rsub(g[8], g[6]);
+    drho = radd(radd(radd(s1, s2), radd(s5, s8)), g[0]);
+    const C jx = radd(d1, radd(d5, d8));
+    const C jy = radd(d2, rsub(d5, d8));
+    rho = radd(one_ref, drho);
+    const C inv = rcp<C>(rho);
+    ux = rmul(jx, inv);
+    uy = rmul(jy, inv);
+    const C a = rmul(jx, ux), b = rmul(jy, uy), c = rmul(jx, uy);
+    const C ab = radd(a, b);
+    const C jp = radd(jx, jy), jm = rsub(jx, jy);
+    if constexpr (sizeof(C) == 4) {
+        const C q1 = rfma(C(-1.5), b, rfma(C(3.0), a, drho));
+        const C q2 = rfma(C(-1.5), a, rfma(C(3.0), b, drho));
+        const C qd = rfma(C(3.0), ab, drho);
+        const C q5 = rfma(C(9.0), c, qd), q8 = rfma(C(-9.0), c, qd);
+        const C t1 = rfma(k.ow1, q1, -rmul(k.half, s1));
+        const C t2 = rfma(k.ow1, q2, -rmul(k.half, s2));
+        const C t5 = rfma(k.ow5, q5, -rmul(k.half, s5));
+        const C t8 = rfma(k.ow5, q8, -rmul(k.half, s8));
+        const C e5 = rmul(k.half, rfma(C(1.0 / 6.0), jp, -d5));
+        const C e8 = rmul(k.half, rfma(C(1.0 / 6.0), jm, -d8));
+        const C e1 = radd(e5, e8);  // -delta_1
+        const C e2 = rsub(e8, e5);  // delta_2
+        out[0] = rfma(C(-2.0), radd(radd(t1, t2), radd(t5, t8)), g[0]);
+        out[1] = radd(g[1], rsub(t1, e1));
+        out[3] = radd(g[3], radd(t1, e1));
+        out[2] = radd(g[2], radd(t2, e2));
+        out[4] = radd(g[4], rsub(t2, e2));
+        out[5] = radd(g[5], radd(t5, e5));
+        out[7] = radd(g[7], rsub(t5, e5));
+        out[8] = radd(g[8], radd(t8, e8));
+        out[6] = radd(g[6], rsub(t8, e8));
+    } else {
+        const C base = rfma(C(-1.5), ab, drho);
+        const C p1 = rmul(k.ow1, base);
+        const C q1 = rfma(rmul(k.ow1, C(4.5)), a, p1), q2 = rfma(rmul(k.ow1, C(4.5)), b, p1);
+        const C p5 = rmul(k.ow5, rfma(C(3.0), ab, drho));
+        const C w9 = rmul(k.ow5, C(9.0));
+        const C q5 = rfma(w9, c, p5), q8 = rfma(-w9, c, p5);
+        const C m1 = rmul(k.ow1, C(3.0)), m5 = rmul(k.ow5, C(3.0));
+        out[0] = rfma(k.keep, g[0], rmul(k.ow0, base));
+        out[1] = rfma(k.keep, g[1], rfma(m1, jx, q1));
+        out[3] = rfma(k.keep, g[3], rfma(-m1, jx, q1));
+        out[2] = rfma(k.keep, g[2], rfma(m1, jy, q2));
+        out[4] = rfma(k.keep, g[4], rfma(-m1, jy, q2));
+        out[5] = rfma(k.keep, g[5], rfma(m5, jp, q5));
+        out[7] = rfma(k.keep, g[7], rfma(-m5, jp, q5));
+        out[8] = rfma(k.keep, g[8], rfma(m5, jm, q8));
+        out[6] = rfma(k.keep, g[6], rfma(-m5, jm, q8));
+    }
+}
+
+// Wall closure of a ring node whose inner neighbour x_f collided to `out` with moments (rho, u):
+// f^eq(rho, u_w) + (1 - omega)(f(x_f) - f^eq(rho, u)) = out + f^eq(rho, u_w) - f^eq(rho, u), the
+// difference of two equilibria of equal density: w (q +- 3 c_j.j) of the differences of a, b, c
+// and j.  The walls rest or move along x with speed W.
+template <typename C>
+__device__ __forceinline__ void wall_shift(C rho, C ux, C uy, C W, C (&out)[9]) {
+    const C jx = rmul(rho, ux), jy = rmul(rho, uy), jw = rmul(rho, W);
+    const C a = rsub(rmul(jw, W), rmul(jx, ux)), b = rmul(-jy, uy), c = rmul(-jx, uy);
+    const C mx = rmul(C(3.0), rsub(jw, jx)), my = rmul(C(-3.0), jy);
+    const C ab = radd(a, b), c9 = rmul(C(9.0), c);
+    const C q1 = rfma(C(-1.5), b, rmul(C(3.0), a)), q2 = rfma(C(-1.5), a, rmul(C(3.0), b));
+    const C qd = rmul(C(3.0), ab), q5 = radd(qd, c9), q8 = rsub(qd, c9);
+    const C mp = radd(mx, my), mm = rsub(mx, my);
+    const C w1 = C(1.0 / 9.0), w5 = C(1.0 / 36.0);
+    out[0] = rfma(C(-2.0 / 3.0), ab, out[0]);  // -3/2 w_0
+    out[1] = rfma(w1, radd(q1, mx), out[1]);
+    out[3] = rfma(w1, rsub(q1, mx), out[3]);
+    out[2] = rfma(w1, radd(q2, my), out[2]);
+    out[4] = rfma(w1, rsub(q2, my), out[4]);
+    out[5] = rfma(w5, radd(q5, mp), out[5]);
+    out[7] = rfma(w5, rsub(q5, mp), out[7]);
+    out[8] = rfma(w5, radd(q8, mm), out[8]);
+    out[6] = rfma(w5, rsub(q8, mm), out[6]);
+}
 
 // Streamed populations of one row segment (V nodes) of row y, walls folded in: wall rows gather
 // at their inner row, the left/right wall nodes take the populations of x_f = 1 / nx - 2.
@@ -386,9 +485,7 @@ __device__ __forceinline__ void step_row(const S* __restrict__ src, S* __restric
     using C = typename St<S>::C;
     const int nx = cv.nx, ny = cv.ny;
     const long long pitch = cv.pitch, plane = cv.plane;
-    const C omega = cv.omega;
-    const C keep = C(1.0) - omega;  // 1 - 1/tau (wall nodes)
-    const C ow0 = omega * C(4.0 / 9.0), ow1 = omega * C(1.0 / 9.0), ow5 = omega * C(1.0 / 36.0);
+    const Relax<C> rx = make_relax<C>(cv.omega);
     C f[9][V];
     pull_segment<S, SHIFTED, V, HINT>(src, lane, x0, y, nx, ny, pitch, plane, cv.q, f);
     // LBM_Q16S works on h = g - w rho_ref: BGK and the wall closure keep their form in h with
@@ -416,52 +513,18 @@ __device__ __forceinline__ void step_row(const S* __restrict__ src, S* __restric
         C g[9];
 #pragma unroll
         for (int j = 0; j < 9; ++j) g[j] = f[j][i];
-        const C drho = ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7])) + g[8];
-        const C rho = one_ref + drho;
-        const C jx = (g[1] - g[3]) + (g[5] - g[6]) + (g[8] - g[7]);
-        const C jy = (g[2] - g[4]) + (g[5] + g[6]) - (g[7] + g[8]);
-        const C inv = rcp<C>(rho);
-        const C ux = jx * inv, uy = jy * inv;
+        C out[9], drho, rho, ux, uy;
+        collide<C>(g, one_ref, rx, out, drho, rho, ux, uy);
         const bool wall = EDGE && ((y == 0) | (y == ny - 1) | (x == 0) | (x >= nx - 1));
         C uox = ux, uoy = uy;
         if (wall) {
             const bool lid = (y == ny - 1) && (cv.corner_moving || (x > 0 && x < nx - 1));
             uox = lid ? cv.Ulid : C(0.0);
             uoy = C(0.0);
-            C e[9], ew[9];
-            geq9<C>(drho, rho, ux, uy, e);
-            geq9<C>(drho, rho, uox, uoy, ew);
-#pragma unroll
-            for (int j = 0; j < 9; ++j) f[j][i] = ew[j] + keep * (g[j] - e[j]);
-        } else if constexpr (sizeof(C) == 4 && (sizeof(S) == 4 || kIsQ16<S>)) {
-            // FP32 and LBM_Q16S storage: BGK as an increment d_j = (f^eq_j - f_j)/tau added to
-            // the pulled value.  The increment must carry no momentum; in FP32 the rounding of
-            // f^eq breaks that by a few ulps in the same direction every step, so the x and y
-            // momentum of d is removed from the (1,3) and (2,4) pairs (a rounding-level change).
-            // LBM_Q16S rounds its stores to nearest, which passes such a bias on unchanged on
-            // average, so it needs the correction as much as FP32 storage does.
-            C e[9];
-            geq9<C>(drho, rho, ux, uy, e);
-            C d[9];
-#pragma unroll
-            for (int j = 0; j < 9; ++j) d[j] = omega * (e[j] - g[j]);
-            const C mx = (d[1] - d[3]) + (d[5] - d[6]) + (d[8] - d[7]);
-            const C my = (d[2] - d[4]) + (d[5] + d[6]) - (d[7] + d[8]);
-            d[1] -= C(0.5) * mx;
-            d[3] += C(0.5) * mx;
-            d[2] -= C(0.5) * my;
-            d[4] += C(0.5) * my;
-#pragma unroll
-            for (int j = 0; j < 9; ++j) f[j][i] = g[j] + d[j];
-        } else {
-            // FP64 storage (bound by the FP64 pipe) and binary16 / bfloat16 storage (bound by
-            // instruction issue; their stored rounding swamps an FP32 bias): the pairwise form
-            // with fewer operations.
-            C out[9];
-            collide_pairs<C>(drho, rho, ux, uy, omega, ow0, ow1, ow5, g, out);
-#pragma unroll
-            for (int j = 0; j < 9; ++j) f[j][i] = out[j];
+            wall_shift<C>(rho, ux, uy, uox, out);
         }
+#pragma unroll
+        for (int j = 0; j < 9; ++j) f[j][i] = out[j];
         if (EDGE && x >= nx) {
 #pragma unroll
             for (int j = 0; j < 9; ++j) f[j][i] = C(0.0);
@@ -547,14 +610,13 @@ __device__ __forceinline__ void block_partials(C a0, C a1, C a2, double* partial
     }
 }
 
-// Resident blocks per SM the register budget is sized for.  binary16 / bfloat16 storage: 32 warps
-// per SM (64 registers, a few spilled to L1).  Left to itself the compiler takes 80 and leaves 24
-// warps, and these kernels wait on memory latency: f16s 163 -> 170 GLUPS at 4096^2 (bf16s 161 ->
-// 168).  0 (no bound) for the rest -- a bound of 1 is not the same as none, it lets the compiler
+// Resident blocks per SM the register budget is sized for.  binary16 / bfloat16 storage: 28 warps
+// per SM (72 registers).  These kernels wait on memory latency, and 4096^2 measures 169 GLUPS with
+// 24 warps, 176 with 28 and 172 with 32 (64 registers, which spill; bf16s 165, 173, 170).  0 (no bound) for the rest -- a bound of 1 is not the same as none, it lets the compiler
 // take more registers; LBM_Q16S, bound by its integer code conversions, lost 4 % at 2048^2 under
 // the same cap.
 template <typename S, int BY>
-inline constexpr int kStepMinBlocks = (sizeof(S) == 2 && !kIsQ16<S>) ? 32 / BY : 0;
+inline constexpr int kStepMinBlocks = (sizeof(S) == 2 && !kIsQ16<S>) ? 28 / BY : 0;
 
 template <typename S, bool SHIFTED, bool REDUCE, int V, int R, int BY, int HINT>
 __global__ void __launch_bounds__(32 * BY, (kStepMinBlocks<S, BY>)) k_step(const StepArgs a) {
