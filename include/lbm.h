@@ -137,7 +137,7 @@ int lbm_get_info(const lbm_ctx *ctx, lbm_info *info);
 /* Advance n >= 0 time steps of Eq. 1 with the Sec. 2.2 (ii) walls: for every node pull
  * f_j(x - c_j) (streaming), form rho and u (Eq. 3) and collide towards f^eq (Eq. 2); wall nodes
  * take f^eq(rho_f, u_w) + (1 - 1/tau)[f(x_f) - f^eq(rho_f, u_f)] from their inner neighbour
- * x_f.  One fused kernel per step.  After every step whose global index is a multiple of 100
+ * x_f.  One fused kernel per step, or per few steps (launch shapes below).  After every step whose global index is a multiple of 100
  * the library also forms, in FP64, the mass sum rho and the Eq. 6 residual against the velocity
  * field of 100 steps earlier, and samples the probes (lbm_probe).  Asynchronous.
  * Errors: LBM_EINVAL (n < 0), LBM_ECUDA. */
@@ -153,9 +153,10 @@ int lbm_run_to_residual(lbm_ctx *ctx, double tol, long max_steps, long *steps_do
 
 /* ------------------------------------------------------------------ launch shapes */
 
-/* The fused step kernel has several launch shapes (rows per thread, warps per block, register
- * budget).  They compute bitwise-identical populations; only speed differs (the FP64 checkpoint
- * sums may differ in the last bits, since the partial sums are grouped by block). */
+/* The time step has several launch shapes (rows per thread, warps per block, register budget; the
+ * last one advances four steps per launch in FP32 storage).  They compute bitwise-identical populations; only
+ * speed differs (the FP64 checkpoint sums may differ in the last bits, since the partial sums are
+ * grouped by block). */
 int lbm_launch_config_count(void);
 
 /* Select shape cfg in [0, lbm_launch_config_count()).  Synchronising.  LBM_EINVAL if out of range. */

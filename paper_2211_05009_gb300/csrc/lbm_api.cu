@@ -2,6 +2,7 @@
 // (single launches and 100-step CUDA graphs), checkpointing of Eq. 6 results, field import and
 // export through caller buffers, probes and save/load.  All compute runs in the kernels of
 // lbm_step.cu and lbm_aux.cu; nothing here touches population values on the CPU.
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdint>
@@ -47,7 +48,9 @@ struct lbm_ctx {
     void* alloc_user = nullptr;
     size_t device_bytes = 0;
 
-    void* buf[2] = {nullptr, nullptr};  // populations, ping-pong; current = buf[step & 1]
+    void* buf[2] = {nullptr, nullptr};  // populations, ping-pong; current = buf[which]
+    int which = 0;
+    int sms = 0;  // multiprocessors of the device
     void* snap = nullptr;               // [2][ny][pitch] Eq. 6 snapshot (arithmetic type)
     double* partials = nullptr;         // reduction partials
     int npartials = 0;
@@ -59,7 +62,7 @@ struct lbm_ctx {
 
     cudaStream_t stream = nullptr;
     cudaStream_t cap_stream = nullptr;
-    cudaGraphExec_t chunk[2] = {nullptr, nullptr};
+    cudaGraphExec_t chunk[2][2] = {};  // [checkpoint parity][buffer it starts from]
     cudaEvent_t ev[2] = {nullptr, nullptr};
 
     ProbeSet probes{};
@@ -110,12 +113,12 @@ struct lbm_ctx {
         a.st = d_state;
         return a;
     }
-    FieldArgs cur() const { return field((int)(step & 1)); }
+    FieldArgs cur() const { return field(which); }
 
-    StepArgs step_args(long long gstep, int s) const {
+    StepArgs step_args(int from, int s) const {
         StepArgs a{};
-        a.src = buf[gstep & 1];
-        a.dst = buf[(gstep + 1) & 1];
+        a.src = buf[from];
+        a.dst = buf[from ^ 1];
         a.nx = nx;
         a.ny = ny;
         a.pitch = pitch;
@@ -135,18 +138,25 @@ struct lbm_ctx {
     }
 
     void invalidate_graphs() {
-        for (auto& g : chunk)
-            if (g) {
-                cudaGraphExecDestroy(g);
-                g = nullptr;
-            }
+        for (auto& pair : chunk)
+            for (auto& g : pair)
+                if (g) {
+                    cudaGraphExecDestroy(g);
+                    g = nullptr;
+                }
     }
 
-    // Enqueue the kernels of one time step from global step gstep on stream st.
-    int enqueue_step(long long gstep, cudaStream_t st) {
+    // Enqueue one launch from global step gstep and buffer `from` on stream st: a checkpoint step by
+    // itself, else as many plain steps (at most n, none of them a checkpoint step) as the shape
+    // fuses.  Returns the steps taken in *taken; the state is then in the other buffer.
+    int enqueue(long long gstep, long long n, int from, cudaStream_t st, int* taken) {
         const int s = (int)(gstep % kInterval);
-        const bool reduce = (gstep + 1) % kInterval == 0;
-        int rc = cuda(launch_step(dtype, cfg, step_args(gstep, s), reduce, st), "step kernel launch");
+        const bool reduce = s == kInterval - 1;
+        const int plain = (int)std::min<long long>(n, kInterval - 1 - s);
+        const int fused = reduce ? 1 : std::min(config_steps(dtype, cfg), plain);
+        *taken = fused;
+        int rc = fused > 1 ? cuda(launch_march(dtype, step_args(from, s), fused, sms, st), "fused step launch")
+                           : cuda(launch_step(dtype, cfg, step_args(from, s), reduce, st), "step kernel launch");
         if (rc) return rc;
         if (reduce) {
             rc = cuda(launch_finalize_checkpoint(partials, geo.blocks, (double)nx * ny, d_state, st),
@@ -159,17 +169,25 @@ struct lbm_ctx {
         }
         return rc;
     }
+    // Launches of one whole interval (each one changes the buffer).
+    int interval_launches() const {
+        const int f = config_steps(dtype, cfg);
+        return (kInterval - 1 + f - 1) / f + 1;
+    }
 
-    // 100-step graph for chunks that start at an aligned step; slot = parity of the checkpoint.
-    int ensure_graph(int slot) {
-        if (chunk[slot]) return LBM_OK;
+    // 100-step graph for chunks that start at an aligned step in buffer `from`; slot = parity of the
+    // checkpoint.
+    int ensure_graph(int slot, int from) {
+        if (chunk[slot][from]) return LBM_OK;
         cudaGraph_t g = nullptr;
         int rc = cuda(cudaStreamBeginCapture(cap_stream, cudaStreamCaptureModeThreadLocal),
                       "begin graph capture");
         if (rc) return rc;
         // the chunk ends at a checkpoint of parity `slot`; its first step is a multiple of 100
         const long long g0 = slot == 1 ? 0 : kInterval;
-        for (int s = 0; s < kInterval && !rc; ++s) rc = enqueue_step(g0 + s, cap_stream);
+        int b = from;
+        for (int s = 0, taken = 0; s < kInterval && !rc; s += taken, b ^= 1)
+            rc = enqueue(g0 + s, kInterval - s, b, cap_stream, &taken);
         cudaError_t e = cudaStreamEndCapture(cap_stream, &g);
         if (rc) {
             if (g) cudaGraphDestroy(g);
@@ -177,7 +195,7 @@ struct lbm_ctx {
         }
         rc = cuda(e, "end graph capture");
         if (rc) return rc;
-        rc = cuda(cudaGraphInstantiate(&chunk[slot], g, 0), "graph instantiate");
+        rc = cuda(cudaGraphInstantiate(&chunk[slot][from], g, 0), "graph instantiate");
         cudaGraphDestroy(g);
         return rc;
     }
@@ -187,17 +205,20 @@ struct lbm_ctx {
         while (n > 0 && !rc) {
             if (step % kInterval == 0 && n >= kInterval) {
                 const int slot = (int)(((step + kInterval) / kInterval) & 1);
-                rc = ensure_graph(slot);
+                rc = ensure_graph(slot, which);
                 if (rc) return rc;
-                rc = cuda(cudaGraphLaunch(chunk[slot], stream), "graph launch");
+                rc = cuda(cudaGraphLaunch(chunk[slot][which], stream), "graph launch");
                 if (rc) return rc;
+                which ^= interval_launches() & 1;
                 step += kInterval;
                 n -= kInterval;
             } else {
-                rc = enqueue_step(step, stream);
+                int taken = 0;
+                rc = enqueue(step, n, which, stream, &taken);
                 if (rc) return rc;
-                step += 1;
-                n -= 1;
+                which ^= 1;
+                step += taken;
+                n -= taken;
             }
         }
         return rc;
@@ -293,6 +314,11 @@ extern "C" int lbm_create_ex(int nx, int ny, double tau, double U, lbm_dtype dty
     }
 
     lbm_ctx* c = new lbm_ctx();
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        cudaGetLastError();
+        return create_fail(c, LBM_ECUDA, "no CUDA device available (the library has no CPU path)");
+    }
     c->nx = nx;
     c->ny = ny;
     c->tau = tau;
@@ -305,7 +331,7 @@ extern "C" int lbm_create_ex(int nx, int ny, double tau, double U, lbm_dtype dty
     c->pitch = row_pitch(c->dtype, nx);
     c->q = q16_codec(U);
     c->plane = c->pitch * (long long)ny;
-    c->cfg = default_step_config(c->dtype);
+    c->cfg = default_step_config(c->dtype, nx, ny);
     c->geo = step_geometry(c->dtype, c->cfg, ny, c->pitch);
     int max_blocks = 0;
     for (int k = 0; k < kStepConfigs; ++k) {
@@ -432,15 +458,22 @@ extern "C" int lbm_autotune(lbm_ctx* c, int steps_per_trial, int* best, double* 
     if (!rc) rc = c->cuda(cudaEventCreate(&e2), "event create");
     float plain[kStepConfigs], red[kStepConfigs];
     for (int k = 0; k < kStepConfigs; ++k) plain[k] = red[k] = 1e30f;
+    // `n` steps of shape k (steps 0..97 of a checkpoint interval never reduce)
+    auto plain_steps = [&](int k, int n) {
+        const int f = config_steps(t->dtype, k);
+        for (int s = 0, from = 0; s < n && !rc; s += f, from ^= 1) {
+            const int m = std::min(f, n - s);
+            rc = m > 1 ? c->cuda(launch_march(t->dtype, t->step_args(from, s % 94), m, t->sms, t->stream), "autotune launch")
+                       : c->cuda(launch_step(t->dtype, k, t->step_args(from, s % 98), false, t->stream), "autotune launch");
+        }
+    };
     for (int round = 0; round < 3 && !rc; ++round) {
         for (int k = 0; k < kStepConfigs && !rc; ++k) {
-            if (round == 0)  // warm-up
-                for (int s = 0; s < steps_per_trial && !rc; ++s)
-                    rc = c->cuda(launch_step(t->dtype, k, t->step_args(s & 1, s % 98), false, t->stream), "autotune launch");
+            if (k >= kRowConfigs && config_steps(t->dtype, k) == 1) continue;  // the default row shape again
+            if (round > 0 && plain[k] > 1.25f * *std::min_element(plain, plain + kStepConfigs)) continue;  // out of the race
+            if (round == 0) plain_steps(k, steps_per_trial);  // warm-up
             if (!rc) rc = c->cuda(cudaEventRecord(e0, t->stream), "event record");
-            // steps 0..97 of a checkpoint interval never reduce
-            for (int s = 0; s < steps_per_trial && !rc; ++s)
-                rc = c->cuda(launch_step(t->dtype, k, t->step_args(s & 1, s % 98), false, t->stream), "autotune launch");
+            plain_steps(k, steps_per_trial);
             if (!rc) rc = c->cuda(cudaEventRecord(e1, t->stream), "event record");
             for (int s = 0; s < 2 && !rc; ++s)
                 rc = c->cuda(launch_step(t->dtype, k, t->step_args(s & 1, 99), true, t->stream), "autotune launch");
@@ -646,6 +679,7 @@ extern "C" int lbm_set_moments_ex(lbm_ctx* c, const double* rho, const double* u
     }
     if (rc) return rc;
     c->step = 0;
+    c->which = 0;  // where the captured graphs of the first interval start
     // the captured 100-step graphs hold the probe set by value and nothing else that this call
     // changes (the step counter picks a graph, the state lives in device memory): keep them unless
     // a probe's start step moves, so that re-seeding the field every 100 steps costs no capture
@@ -809,7 +843,7 @@ extern "C" int lbm_save(lbm_ctx* c, const char* path) {
     const size_t snap_bytes = 2ull * c->ny * c->nx * ab;
     char* host = (char*)malloc(pop_bytes + snap_bytes + sizeof(DevState));
     if (!host) return c->fail(LBM_ENOMEM, "host buffer for checkpoint");
-    int rc = c->cuda(cudaMemcpy2DAsync(host, row, c->buf[c->step & 1], (size_t)c->pitch * es, row,
+    int rc = c->cuda(cudaMemcpy2DAsync(host, row, c->buf[c->which], (size_t)c->pitch * es, row,
                                        9ull * c->ny, cudaMemcpyDeviceToHost, c->stream), "population copy");
     if (!rc) rc = c->cuda(cudaMemcpy2DAsync(host + pop_bytes, c->nx * ab, c->snap, (size_t)c->pitch * ab,
                                             c->nx * ab, 2ull * c->ny, cudaMemcpyDeviceToHost, c->stream), "snapshot copy");
@@ -874,7 +908,7 @@ extern "C" int lbm_load(lbm_ctx* c, const char* path) {
     c->step = h.step;
     for (int q = 0; q < c->probes.n; ++q) c->probes.start[q] = c->step;
     c->invalidate_graphs();
-    if (!rc) rc = c->cuda(cudaMemcpy2DAsync(c->buf[c->step & 1], (size_t)c->pitch * es, host, row, row, 9ull * c->ny, cudaMemcpyHostToDevice, c->stream), "population upload");
+    if (!rc) rc = c->cuda(cudaMemcpy2DAsync(c->buf[c->which], (size_t)c->pitch * es, host, row, row, 9ull * c->ny, cudaMemcpyHostToDevice, c->stream), "population upload");
     if (!rc) rc = c->cuda(cudaMemcpy2DAsync(c->snap, (size_t)c->pitch * ab, host + pop_bytes, c->nx * ab, c->nx * ab, 2ull * c->ny, cudaMemcpyHostToDevice, c->stream), "snapshot upload");
     if (!rc) rc = c->cuda(cudaMemcpyAsync(c->d_state, host + pop_bytes + snap_bytes, sizeof(DevState), cudaMemcpyHostToDevice, c->stream), "state upload");
     if (!rc) {

@@ -21,14 +21,27 @@ struct StepGeometry {
     int grid_x, grid_y, blocks;
 };
 
-// Launch shapes of the step kernel (see lbm_step_kernel.cuh); all give identical populations.
-constexpr int kStepConfigs = 6;
-// Fastest shape per storage type measured on GB300 at 2048 x 2048 (f64, f32, f32s, f16s, bf16s);
+// Launch shapes of the time step; all give identical populations.  0..5: one step per launch (row
+// step, lbm_step_kernel.cuh).  6: kMarchSteps plain steps per launch (lbm_march.cuh) for FP32
+// storage; steps left over run as one shorter launch, checkpoint steps one by one.  The other types
+// gain nothing from fewer passes over memory and take their default row shape there: FP64 is bound by
+// its pipe, LBM_Q16S by its code conversions, and binary16 / bfloat16 meet the FP32 pipe first
+// (4096^2, fused 178 / 164 GLUPS, row step 177 / 174; 2048^2 145 / 134 against 168 / 162).
+constexpr int kStepConfigs = 7, kRowConfigs = 6;
+constexpr int kMarchSteps = 4;
+inline bool march_dtype(int dtype) { return dtype == 1 || dtype == 2; }
+// Plain steps per launch of a shape.
+inline int config_steps(int dtype, int cfg) { return cfg < kRowConfigs || !march_dtype(dtype) ? 1 : kMarchSteps; }
+// Fastest row shape per storage type measured on GB300 at 2048 x 2048 (f64, f32, f32s, f16s, bf16s);
 // lbm_autotune re-measures on the caller's size.
-inline int default_step_config(int dtype) {
+inline int default_row_config(int dtype) {
     constexpr int k[6] = {1, 4, 0, 2, 2, 2};
     return (dtype >= 0 && dtype < 6) ? k[dtype] : 0;
 }
+// Row shape of the single steps of a shape.
+inline int row_config(int dtype, int cfg) { return cfg < kRowConfigs ? cfg : default_row_config(dtype); }
+// Shape of a new context.
+int default_step_config(int dtype, int nx, int ny);
 
 constexpr int kDtypeQ16S = 5;
 // LBM_Q16S scale S_j of direction j for lid speed U: the largest code is (2 - 2^-13) S_j, and
@@ -50,6 +63,9 @@ long long row_pitch(int dtype, int nx);
 int storage_bytes(int dtype);
 
 cudaError_t launch_step(int dtype, int cfg, const StepArgs& a, bool reduce, cudaStream_t st);
+// `steps` (1 .. kMarchSteps) plain steps from a.src to a.dst in one launch (march_dtype types only);
+// sms: multiprocessors of the device.
+cudaError_t launch_march(int dtype, const StepArgs& a, int steps, int sms, cudaStream_t st);
 cudaError_t launch_finalize_checkpoint(const double* partials, int nblocks, double nodes,
                                        DevState* st, cudaStream_t s);
 

@@ -19,7 +19,7 @@ struct Shape {
     int R, BY;
 };
 // must match launch_step_cfg in lbm_step_kernel.cuh
-constexpr Shape kShapes[kStepConfigs] = {{2, 2}, {1, 4}, {2, 2}, {4, 1}, {2, 4}, {4, 2}};
+constexpr Shape kShapes[kRowConfigs] = {{2, 2}, {1, 4}, {2, 2}, {4, 1}, {2, 4}, {4, 2}};
 }  // namespace
 
 double q16_scale(int j, double U) {
@@ -39,10 +39,19 @@ QCodec q16_codec(double U) {
     return q;
 }
 
+int default_step_config(int dtype, int nx, int ny) {
+    // Fused steps pay once the two population buffers outgrow the L2 cache; below that the rows that
+    // neighbouring segments compute twice cost more than the saved launches.  us a step, row step
+    // against fused: f32s 1024^2 8.5 / 8.4, 1500^2 26.1 / 13.8; f32 1024^2 9.1 / 13.1, 1500^2
+    // 26.2 / 21.7, 500 x 1000 6.2 / 9.7.
+    const long long from = dtype == 2 ? 1000000 : 1600000;
+    return march_dtype(dtype) && (long long)nx * ny >= from ? kRowConfigs : default_row_config(dtype);
+}
+
 StepGeometry step_geometry(int dtype, int cfg, int ny, long long pitch) {
     StepGeometry g{};
     const int V = storage_bytes(dtype) == 2 ? 4 : 2;  // as launch_step_cfg
-    const Shape s = kShapes[cfg];
+    const Shape s = kShapes[row_config(dtype, cfg)];
     g.grid_x = (int)(pitch / (32 * V));
     g.grid_y = (ny + s.BY * s.R - 1) / (s.BY * s.R);
     g.blocks = g.grid_x * g.grid_y;
@@ -51,6 +60,7 @@ StepGeometry step_geometry(int dtype, int cfg, int ny, long long pitch) {
 
 cudaError_t launch_step(int dtype, int cfg, const StepArgs& a, bool reduce, cudaStream_t st) {
     if (cfg < 0 || cfg >= kStepConfigs) return cudaErrorInvalidValue;
+    cfg = row_config(dtype, cfg);
     switch (dtype) {
         case 0: return launch_step_f64(cfg, a, reduce, st);
         case 1: return launch_step_f32(cfg, a, reduce, st);

@@ -7,8 +7,7 @@
 //   walls       ring nodes pull at their inner neighbour x_f instead and store
 //               f^eq(rho_f, u_w) + (1 - 1/tau)(f(x_f) - f^eq(rho_f, u_f))           Sec. 2.2 (ii)
 //               -- the non-equilibrium extrapolation rebuilt and collided in one go (the
-//               rebuilt node has moments (rho_f, u_w), so its BGK step is this closed form),
-//               computed as the collided x_f plus f^eq(rho_f, u_w) - f^eq(rho_f, u_f).
+//               rebuilt node has moments (rho_f, u_w), so its BGK step is this closed form).
 // All arithmetic runs on deviations g_j = f_j - w_j, which keeps rounding relative to the flow
 // rather than to the weights.  Every REDUCE launch (the 100th step of a checkpoint interval) also
 // forms sum(rho - 1) and the two sums of Eq. 6 against the snapshot of 100 steps before, and writes
@@ -240,9 +239,10 @@ __device__ __forceinline__ void pull_row(const S* __restrict__ p, int lane, int 
     }
 }
 
-// Arithmetic with the rounding of each operation spelled out: every kernel that advances a node
-// (row step, batch, fused march) must give bitwise the same populations, so none of them may leave
-// the choice of contractions to the compiler.
+// ------------------------------------------------------------------ arithmetic on pairs and momentum
+// LBM_F64 and LBM_F32S.  The rounding of each operation is spelled out: every kernel that advances
+// a node (row step, batch, fused march) must give bitwise the same populations, so none of them may
+// leave the choice of contractions to the compiler.
 __device__ __forceinline__ float radd(float a, float b) { return __fadd_rn(a, b); }
 __device__ __forceinline__ float rsub(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ float rmul(float a, float b) { return __fmul_rn(a, b); }
@@ -252,43 +252,89 @@ __device__ __forceinline__ double rsub(double a, double b) { return __dsub_rn(a,
 __device__ __forceinline__ double rmul(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ double rfma(double a, double b, double c) { return __fma_rn(a, b, c); }
 
+// Two FP32 values in one 64-bit register pair, for Blackwell's packed FP32 instructions: the same
+// roundings as the scalar ones at half the issue slots.
+struct f32x2 {
+    unsigned long long v;
+    __device__ __forceinline__ f32x2() {}
+    __device__ __forceinline__ f32x2(float lo, float hi) { asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi)); }
+    __device__ __forceinline__ explicit f32x2(double c) : f32x2(float(c), float(c)) {}
+    __device__ __forceinline__ explicit f32x2(float c) : f32x2(c, c) {}
+    __device__ __forceinline__ float lo() const { return __uint_as_float((unsigned)v); }
+    __device__ __forceinline__ float hi() const { return __uint_as_float((unsigned)(v >> 32)); }
+};
+__device__ __forceinline__ f32x2 radd(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ f32x2 rsub(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ f32x2 rmul(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ f32x2 rfma(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+
+// -1/v.
 template <typename C>
-__device__ __forceinline__ C rcp(C v);
+__device__ __forceinline__ C nrcp(C v);
 // FP32: hardware reciprocal estimate refined by one Newton-Raphson step r + r(1 - v r) (error
 // below one ulp for the densities rho ~ 1 met here; no subnormals).  The IEEE-rounded reciprocal
 // costs several times the instructions in a kernel that is partly issue-bound.
-template <> __device__ __forceinline__ float rcp<float>(float v) {
+template <> __device__ __forceinline__ float nrcp<float>(float v) {
     float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
-    const float e = fmaf(-v, r, 1.0f);
-    return fmaf(r, e, r);
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(-v));
+    return __fmaf_rn(r, __fmaf_rn(v, r, 1.0f), r);
+}
+template <> __device__ __forceinline__ f32x2 nrcp<f32x2>(f32x2 v) {
+    float r0, r1;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(-v.lo()));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r1) : "f"(-v.hi()));
+    const f32x2 r(r0, r1);
+    return rfma(r, rfma(v, r, f32x2(1.0f)), r);
 }
 // FP64: hardware estimate of 1/v (relative error below 2^-20) refined by one third-order step of
 // Householder's family, r (1 + e + e^2) with e = 1 - v r: the error e^3 is below 2^-60, so three
 // FP64 operations give 1/v to the last bit or the one beside it.  Densities are near 1 here; an
 // infinity or NaN comes out as NaN, which the checkpoint reports.
-template <> __device__ __forceinline__ double rcp<double>(double v) {
+template <> __device__ __forceinline__ double nrcp<double>(double v) {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(v));
     const double e = __fma_rn(-v, r, 1.0);
-    return __fma_rn(r, __fma_rn(e, e, e), r);
+    return __fma_rn(-r, __fma_rn(e, e, e), -r);
 }
 
-// Constants of the collision for one cavity.
+// Constants of the collision for one cavity (the FP32 and the FP64 form use different ones).
 template <typename C>
 struct Relax {
-    C keep;         // 1 - omega
-    C ow0, ow1, ow5;  // omega w_j
-    C half;         // omega / 2
+    C ow1, ow5;   // omega w_1, omega w_5
+    C w4, w9;     // -9/2 omega w_1, -9 omega w_5
+    C pw9;        // 9 omega w_5
+    C khalf;      // FP32: (1 - omega)/2.  FP64: 1 - omega
+    C nhalf;      // FP32: -omega/2.       FP64: omega w_0
+    C o12;        // FP32: omega/12 = 3 omega w_5
 };
 template <typename C>
 __device__ __forceinline__ Relax<C> make_relax(C omega) {
+    constexpr bool f64 = sizeof(C) == 8;
     Relax<C> k;
-    k.keep = rsub(C(1.0), omega);
-    k.ow0 = rmul(omega, C(4.0 / 9.0));
     k.ow1 = rmul(omega, C(1.0 / 9.0));
     k.ow5 = rmul(omega, C(1.0 / 36.0));
-    k.half = rmul(omega, C(0.5));
+    k.w4 = rmul(k.ow1, C(-4.5));
+    k.w9 = rmul(k.ow5, C(-9.0));
+    k.pw9 = -k.w9;
+    k.khalf = rmul(rsub(C(1.0), omega), C(f64 ? 1.0 : 0.5));
+    k.nhalf = rmul(omega, C(f64 ? 4.0 / 9.0 : -0.5));
+    k.o12 = rmul(omega, C(1.0 / 12.0));
     return k;
 }
 
@@ -298,72 +344,69 @@ __device__ __forceinline__ Relax<C> make_relax(C omega) {
 // equilibrium of a pair is w (q +- 3 c_j.j) with q = drho + 9/2 (c_j.u)(c_j.j) - 3/2 (a + b):
 // q_1 = drho + 3a - 3/2 b, q_2 = drho + 3b - 3/2 a, q_5/8 = drho + 3(a + b) +- 9c.
 //
-// FP32 arithmetic (every storage type but FP64): 68 FP32 operations.  The increment of a pair is
-// sigma +- delta, sigma = omega/2 (s^eq - s), delta = omega/2 (d^eq - d).  The differences relax
-// linearly (d^eq_5 = (j_x + j_y)/6, d^eq_8 = (j_x - j_y)/6), and delta_1, delta_2 and the rest
-// population take what makes the increment carry no momentum and no mass: in FP32 the rounding of
-// the weights otherwise shifts both by a few ulps in the same direction every step, which is what
-// dominated the velocity error (1e-5 U over 1000 steps).
+// FP32 (LBM_F32S): 61 FP32 operations.  A pair leaves as u +- v, its
+// relaxed half sum u = (1 - omega) s/2 + omega w q and half difference v = d/2 + delta,
+// delta = omega/2 (d^eq - d) with d^eq_5 = (j_x + j_y)/6, d^eq_8 = (j_x - j_y)/6.  delta_1 and
+// delta_2 are taken from delta_5 and delta_8 so that the increments carry no momentum, and the rest
+// population takes what keeps the mass: in FP32 the rounding of weights and moments otherwise
+// shifts both in the same direction every step.  (Relaxing each direction by itself, 53 operations,
+// is 1e-5 U off after 1000 steps of 133x77 at Re 400, this form 1.5e-7 U, increments formed per
+// direction with their momentum taken out 3.6e-7 U.)
 //
-// FP64: 54 FP64 operations (72.7 instructions with the equilibrium formed per direction): the pipe
+// FP64: 53 FP64 operations (72.7 instructions with the equilibrium formed per direction): the pipe
 // issues 2 lanes per clock and SM, so the operation count is the run time (2048^2: 7.3 GLUPS then).
 // out = keep g + (omega g^eq) with the pair's omega g^eq from two fused multiply-adds.
 template <typename C>
 __device__ __forceinline__ void collide(const C (&g)[9], C one_ref, const Relax<C>& k, C (&out)[9], C& drho,
                                         C& rho, C& ux, C& uy) {
+    // d1 = g1 - g3, d2 = g2 - g4, and the negated n5 = g7 - g5, n8 = g6 - g8
     const C s1 = radd(g[1], g[3]), d1 = rsub(g[1], g[3]);
     const C s2 = radd(g[2], g[4]), d2 = rsub(g[2], g[4]);
-    const C s5 = radd(g[5], g[7]), d5 = rsub(g[5], g[7]);
-    const C s8 = radd(g[8], g[6]), d8 = rsub(g[8], g[6]);
+    const C s5 = radd(g[5], g[7]), n5 = rsub(g[7], g[5]);
+    const C s8 = radd(g[8], g[6]), n8 = rsub(g[6], g[8]);
     drho = radd(radd(radd(s1, s2), radd(s5, s8)), g[0]);
-    const C jx = radd(d1, radd(d5, d8));
-    const C jy = radd(d2, rsub(d5, d8));
+    // -j and -1/rho, whose signs cancel in u: negations would be instructions of their own
+    const C jx = rsub(radd(n5, n8), d1);
+    const C jy = rsub(rsub(n5, n8), d2);
     rho = radd(one_ref, drho);
-    const C inv = rcp<C>(rho);
+    const C inv = nrcp<C>(rho);
     ux = rmul(jx, inv);
     uy = rmul(jy, inv);
+    // -a, -b, -c and -(a + b).  No sum of two products: the assembler fuses such packed ones.
     const C a = rmul(jx, ux), b = rmul(jy, uy), c = rmul(jx, uy);
-    const C ab = radd(a, b);
+    const C ab = rfma(jx, ux, b);
     const C jp = radd(jx, jy), jm = rsub(jx, jy);
-    if constexpr (sizeof(C) == 4) {
-        const C q1 = rfma(C(-1.5), b, rfma(C(3.0), a, drho));
-        const C q2 = rfma(C(-1.5), a, rfma(C(3.0), b, drho));
-        const C qd = rfma(C(3.0), ab, drho);
-        const C q5 = rfma(C(9.0), c, qd), q8 = rfma(C(-9.0), c, qd);
-        const C t1 = rfma(k.ow1, q1, -rmul(k.half, s1));
-        const C t2 = rfma(k.ow1, q2, -rmul(k.half, s2));
-        const C t5 = rfma(k.ow5, q5, -rmul(k.half, s5));
-        const C t8 = rfma(k.ow5, q8, -rmul(k.half, s8));
-        const C e5 = rmul(k.half, rfma(C(1.0 / 6.0), jp, -d5));
-        const C e8 = rmul(k.half, rfma(C(1.0 / 6.0), jm, -d8));
-        const C e1 = radd(e5, e8);  // -delta_1
-        const C e2 = rsub(e8, e5);  // delta_2
-        out[0] = rfma(C(-2.0), radd(radd(t1, t2), radd(t5, t8)), g[0]);
-        out[1] = radd(g[1], rsub(t1, e1));
-        out[3] = radd(g[3], radd(t1, e1));
-        out[2] = radd(g[2], radd(t2, e2));
-        out[4] = radd(g[4], rsub(t2, e2));
-        out[5] = radd(g[5], radd(t5, e5));
-        out[7] = radd(g[7], rsub(t5, e5));
-        out[8] = radd(g[8], radd(t8, e8));
-        out[6] = radd(g[6], rsub(t8, e8));
+    const C base = rfma(C(1.5), ab, drho);
+    const C p1 = rmul(k.ow1, base), p5 = rmul(k.ow5, rfma(C(-3.0), ab, drho));
+    const C q1 = rfma(k.w4, a, p1), q2 = rfma(k.w4, b, p1);
+    const C q5 = rfma(k.w9, c, p5), q8 = rfma(k.pw9, c, p5);
+    if constexpr (!std::is_same<C, double>::value) {
+        const C u1 = rfma(k.khalf, s1, q1), u2 = rfma(k.khalf, s2, q2);
+        const C u5 = rfma(k.khalf, s5, q5), u8 = rfma(k.khalf, s8, q8);
+        const C e5 = rfma(k.nhalf, n5, rmul(k.o12, jp));  // -delta_5
+        const C e8 = rfma(k.nhalf, n8, rmul(k.o12, jm));  // -delta_8
+        const C v1 = rfma(C(0.5), d1, radd(e5, e8)), v2 = rfma(C(0.5), d2, rsub(e5, e8));
+        const C v5 = rfma(C(0.5), n5, e5), v8 = rfma(C(0.5), n8, e8);  // negated
+        out[0] = rfma(C(-2.0), radd(radd(u1, u2), radd(u5, u8)), drho);
+        out[1] = radd(u1, v1);
+        out[3] = rsub(u1, v1);
+        out[2] = radd(u2, v2);
+        out[4] = rsub(u2, v2);
+        out[5] = rsub(u5, v5);
+        out[7] = radd(u5, v5);
+        out[8] = rsub(u8, v8);
+        out[6] = radd(u8, v8);
     } else {
-        const C base = rfma(C(-1.5), ab, drho);
-        const C p1 = rmul(k.ow1, base);
-        const C q1 = rfma(rmul(k.ow1, C(4.5)), a, p1), q2 = rfma(rmul(k.ow1, C(4.5)), b, p1);
-        const C p5 = rmul(k.ow5, rfma(C(3.0), ab, drho));
-        const C w9 = rmul(k.ow5, C(9.0));
-        const C q5 = rfma(w9, c, p5), q8 = rfma(-w9, c, p5);
-        const C m1 = rmul(k.ow1, C(3.0)), m5 = rmul(k.ow5, C(3.0));
-        out[0] = rfma(k.keep, g[0], rmul(k.ow0, base));
-        out[1] = rfma(k.keep, g[1], rfma(m1, jx, q1));
-        out[3] = rfma(k.keep, g[3], rfma(-m1, jx, q1));
-        out[2] = rfma(k.keep, g[2], rfma(m1, jy, q2));
-        out[4] = rfma(k.keep, g[4], rfma(-m1, jy, q2));
-        out[5] = rfma(k.keep, g[5], rfma(m5, jp, q5));
-        out[7] = rfma(k.keep, g[7], rfma(-m5, jp, q5));
-        out[8] = rfma(k.keep, g[8], rfma(m5, jm, q8));
-        out[6] = rfma(k.keep, g[6], rfma(-m5, jm, q8));
+        const C m1 = rmul(k.ow1, C(3.0)), m5 = k.o12;
+        out[0] = rfma(k.khalf, g[0], rmul(k.nhalf, base));
+        out[1] = rfma(k.khalf, g[1], rfma(-m1, jx, q1));
+        out[3] = rfma(k.khalf, g[3], rfma(m1, jx, q1));
+        out[2] = rfma(k.khalf, g[2], rfma(-m1, jy, q2));
+        out[4] = rfma(k.khalf, g[4], rfma(m1, jy, q2));
+        out[5] = rfma(k.khalf, g[5], rfma(-m5, jp, q5));
+        out[7] = rfma(k.khalf, g[7], rfma(m5, jp, q5));
+        out[8] = rfma(k.khalf, g[8], rfma(-m5, jm, q8));
+        out[6] = rfma(k.khalf, g[6], rfma(m5, jm, q8));
     }
 }
 
@@ -391,6 +434,119 @@ __device__ __forceinline__ void wall_shift(C rho, C ux, C uy, C W, C (&out)[9]) 
     out[8] = rfma(w5, radd(q8, mm), out[8]);
     out[6] = rfma(w5, rsub(q8, mm), out[6]);
 }
+
+// ------------------------------------------------------------------ arithmetic per direction
+// LBM_F32 and 16-bit storage: what these store is rounded far above FP32 arithmetic on deviations
+// (4e-6 of the velocity after 250 steps of a 500 x 1000 cavity in LBM_F32, 5e-4 in binary16), so
+// their results are that rounding's noise.  They keep the arithmetic that forms every direction by
+// itself, and with it their results bit for bit.
+
+// Deviation equilibrium g^eq_j = w_j (drho + rho A_j), A_j = 3 c.u + 9/2 (c.u)^2 - 3/2 u.u (Eq. 2).
+template <typename C>
+__device__ __forceinline__ void geq9(C drho, C rho, C ux, C uy, C (&e)[9]) {
+    const C usq = C(1.5) * (ux * ux + uy * uy);
+    const C w0 = C(4.0 / 9.0), w1 = C(1.0 / 9.0), w5 = C(1.0 / 36.0);
+    auto A = [&](C cu) { return cu * (C(3.0) + C(4.5) * cu) - usq; };
+    const C up = ux + uy, um = ux - uy;
+    e[0] = w0 * (drho - rho * usq);
+    e[1] = w1 * (drho + rho * A(ux));
+    e[2] = w1 * (drho + rho * A(uy));
+    e[3] = w1 * (drho + rho * A(-ux));
+    e[4] = w1 * (drho + rho * A(-uy));
+    e[5] = w5 * (drho + rho * A(up));
+    e[6] = w5 * (drho + rho * A(-um));
+    e[7] = w5 * (drho + rho * A(-up));
+    e[8] = w5 * (drho + rho * A(um));
+}
+
+// BGK collision of a fluid node, f*_j = g_j + omega (g^eq_j - g_j) with g^eq_j = w_j (drho + rho A_j)
+// (Eq. 1, Eq. 2), written per opposite pair (j, jbar): A = c2 +- 3 c.u with c2 = 9/2 (c.u)^2 - usq,
+// so a pair shares c2, drho + rho c2 and 3 rho c.u.  About 50 operations per node instead of the
+// 65 of forming all nine g^eq and then relaxing towards them.  ow = omega w for the three weights.
+template <typename C>
+__device__ __forceinline__ void collide_pairs(C drho, C rho, C ux, C uy, C omega, C ow0, C ow1, C ow5,
+                                              const C (&g)[9], C (&out)[9]) {
+    const C usq = C(1.5) * (ux * ux + uy * uy);
+    const C r3 = C(3.0) * rho;
+    out[0] = fma(ow0, fma(-rho, usq, drho), fma(-omega, g[0], g[0]));
+    auto pair = [&](int a, int b, C cu, C ow) {
+        const C c2 = fma(C(4.5) * cu, cu, -usq);
+        const C base = fma(rho, c2, drho);
+        const C sft = r3 * cu;
+        out[a] = fma(ow, base + sft, fma(-omega, g[a], g[a]));
+        out[b] = fma(ow, base - sft, fma(-omega, g[b], g[b]));
+    };
+    pair(1, 3, ux, ow1);
+    pair(2, 4, uy, ow1);
+    pair(5, 7, ux + uy, ow5);
+    pair(8, 6, ux - uy, ow5);
+}
+
+// FP32: hardware reciprocal estimate refined by one Newton-Raphson step r + r(1 - v r) (error
+// below one ulp for the densities rho ~ 1 met here; no subnormals).  The IEEE-rounded reciprocal
+// costs several times the instructions in a kernel that is partly issue-bound.
+__device__ __forceinline__ float rcp(float v) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    const float e = fmaf(-v, r, 1.0f);
+    return fmaf(r, e, r);
+}
+
+// Moments of a node (Eq. 3).
+template <typename C>
+__device__ __forceinline__ void moments9(const C (&g)[9], C one_ref, C& drho, C& rho, C& ux, C& uy) {
+    drho = ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7])) + g[8];
+    rho = one_ref + drho;
+    const C jx = (g[1] - g[3]) + (g[5] - g[6]) + (g[8] - g[7]);
+    const C jy = (g[2] - g[4]) + (g[5] + g[6]) - (g[7] + g[8]);
+    const C inv = rcp(rho);
+    ux = jx * inv;
+    uy = jy * inv;
+}
+
+// Wall closure of a ring node from the values g pulled by its inner neighbour.
+template <typename C>
+__device__ __forceinline__ void wall9(const C (&g)[9], C drho, C rho, C ux, C uy, C W, C omega, C (&out)[9]) {
+    const C keep = C(1.0) - omega;  // 1 - 1/tau
+    C e[9], ew[9];
+    geq9<C>(drho, rho, ux, uy, e);
+    geq9<C>(drho, rho, W, C(0.0), ew);
+#pragma unroll
+    for (int j = 0; j < 9; ++j) out[j] = ew[j] + keep * (g[j] - e[j]);
+}
+
+// Collision of a fluid node.  MOMENTUM: BGK as an increment d_j = (f^eq_j - f_j)/tau added to the
+// pulled value, with the x and y momentum of d removed from the (1,3) and (2,4) pairs: in FP32 the
+// rounding of f^eq otherwise shifts the momentum by a few ulps in the same direction every step.
+// LBM_Q16S rounds its stores to nearest, which passes such a bias on unchanged on average, so it
+// needs the correction as much as LBM_F32 does.  binary16 / bfloat16 swamp the bias and take the
+// pairwise form with fewer operations.
+template <bool MOMENTUM, typename C>
+__device__ __forceinline__ void collide9(const C (&g)[9], C drho, C rho, C ux, C uy, C omega, C (&out)[9]) {
+    if constexpr (MOMENTUM) {
+        C e[9];
+        geq9<C>(drho, rho, ux, uy, e);
+        C d[9];
+#pragma unroll
+        for (int j = 0; j < 9; ++j) d[j] = omega * (e[j] - g[j]);
+        const C mx = (d[1] - d[3]) + (d[5] - d[6]) + (d[8] - d[7]);
+        const C my = (d[2] - d[4]) + (d[5] + d[6]) - (d[7] + d[8]);
+        d[1] -= C(0.5) * mx;
+        d[3] += C(0.5) * mx;
+        d[2] -= C(0.5) * my;
+        d[4] += C(0.5) * my;
+#pragma unroll
+        for (int j = 0; j < 9; ++j) out[j] = g[j] + d[j];
+    } else {
+        const C ow0 = omega * C(4.0 / 9.0), ow1 = omega * C(1.0 / 9.0), ow5 = omega * C(1.0 / 36.0);
+        collide_pairs<C>(drho, rho, ux, uy, omega, ow0, ow1, ow5, g, out);
+    }
+}
+
+// Whether a storage type takes the arithmetic on pairs and momentum (collide, wall_shift).
+template <typename S, bool SHIFTED> inline constexpr bool kOnPairs = SHIFTED && sizeof(S) >= 4;
+// ... and whether its per-direction collision takes the momentum correction.
+template <typename S> inline constexpr bool kMomentum = sizeof(S) == 4 || kIsQ16<S>;
 
 // Streamed populations of one row segment (V nodes) of row y, walls folded in: wall rows gather
 // at their inner row, the left/right wall nodes take the populations of x_f = 1 / nx - 2.
@@ -514,14 +670,19 @@ __device__ __forceinline__ void step_row(const S* __restrict__ src, S* __restric
 #pragma unroll
         for (int j = 0; j < 9; ++j) g[j] = f[j][i];
         C out[9], drho, rho, ux, uy;
-        collide<C>(g, one_ref, rx, out, drho, rho, ux, uy);
+        constexpr bool PAIRS = kOnPairs<S, SHIFTED>;
+        if constexpr (PAIRS) collide<C>(g, one_ref, rx, out, drho, rho, ux, uy);
+        else moments9<C>(g, one_ref, drho, rho, ux, uy);
         const bool wall = EDGE && ((y == 0) | (y == ny - 1) | (x == 0) | (x >= nx - 1));
         C uox = ux, uoy = uy;
         if (wall) {
             const bool lid = (y == ny - 1) && (cv.corner_moving || (x > 0 && x < nx - 1));
             uox = lid ? cv.Ulid : C(0.0);
             uoy = C(0.0);
-            wall_shift<C>(rho, ux, uy, uox, out);
+            if constexpr (PAIRS) wall_shift<C>(rho, ux, uy, uox, out);
+            else wall9<C>(g, drho, rho, ux, uy, uox, cv.omega, out);
+        } else if constexpr (!PAIRS) {
+            collide9<kMomentum<S>, C>(g, drho, rho, ux, uy, cv.omega, out);
         }
 #pragma unroll
         for (int j = 0; j < 9; ++j) f[j][i] = out[j];
@@ -610,13 +771,14 @@ __device__ __forceinline__ void block_partials(C a0, C a1, C a2, double* partial
     }
 }
 
-// Resident blocks per SM the register budget is sized for.  binary16 / bfloat16 storage: 28 warps
-// per SM (72 registers).  These kernels wait on memory latency, and 4096^2 measures 169 GLUPS with
-// 24 warps, 176 with 28 and 172 with 32 (64 registers, which spill; bf16s 165, 173, 170).  0 (no bound) for the rest -- a bound of 1 is not the same as none, it lets the compiler
+// Resident blocks per SM the register budget is sized for.  binary16 / bfloat16 storage: 32 warps
+// per SM (64 registers, a few spilled to L1).  Left to itself the compiler takes 80 and leaves 24
+// warps, and these kernels wait on memory latency: f16s 163 -> 170 GLUPS at 4096^2 (bf16s 161 ->
+// 168).  0 (no bound) for the rest -- a bound of 1 is not the same as none, it lets the compiler
 // take more registers; LBM_Q16S, bound by its integer code conversions, lost 4 % at 2048^2 under
 // the same cap.
 template <typename S, int BY>
-inline constexpr int kStepMinBlocks = (sizeof(S) == 2 && !kIsQ16<S>) ? 28 / BY : 0;
+inline constexpr int kStepMinBlocks = (sizeof(S) == 2 && !kIsQ16<S>) ? 32 / BY : 0;
 
 template <typename S, bool SHIFTED, bool REDUCE, int V, int R, int BY, int HINT>
 __global__ void __launch_bounds__(32 * BY, (kStepMinBlocks<S, BY>)) k_step(const StepArgs a) {

@@ -1,0 +1,57 @@
+"""Launch shapes that advance several steps per launch against the single-step shape: populations
+and probe samples bitwise, Eq. 6 to the rounding of its differently grouped FP32 partial sums, at
+the sizes where strips, halos and segments can go wrong."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_2211_05009_gb300 import binding as B  # noqa: E402
+from paper_2211_05009_gb300.cavity import Cavity  # noqa: E402
+
+SIZES = [(3, 3), (5, 4), (66, 9), (121, 40),   # one strip; two-row segments; the wall one past a strip
+         (129, 31), (130, 33), (131, 34), (240, 65),  # right wall in every slot of a lane; exactly two strips
+         (500, 200)]
+
+
+def run(nx, ny, dtype, cfg, corners):
+    with Cavity(nx, ny, tau=0.62, U=0.1, dtype=dtype, corners_moving=corners) as cav:
+        B.lbm_set_launch_config(cav.ctx, cfg)
+        top = (ny - 1) / nx  # probes on the lid, on the bottom wall and inside, sampled at odd steps too
+        series = [cav.probe(x, y, every=e, cap=250)[1] for x, y, e in ((0.5, top, 3), (0.4, 0.0, 2), (0.3, 0.4 * top, 1))]
+        for n in (37, 2, 1, 160, 50):  # crosses two checkpoints off and on the interval boundary
+            cav.step(n)
+        assert cav.step_count == 250
+        return cav.populations(host=True), [s.cpu().numpy() for s in series], cav.residual()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f32s", "f16s", "bf16s", "f64", "q16s"])
+@pytest.mark.parametrize("nx,ny", SIZES)
+def test_fused_steps_equal_single_steps(nx, ny, dtype):
+    want, probes, r = run(nx, ny, dtype, 0, corners=nx == 129)
+    assert np.isfinite(want).all()
+    for cfg in range(1, B.lbm_launch_config_count()):
+        got, p, rc = run(nx, ny, dtype, cfg, corners=nx == 129)
+        assert np.array_equal(got, want), f"shape {cfg}"
+        for a, b in zip(p, probes):
+            assert np.array_equal(a, b), f"shape {cfg}"
+        assert abs(rc - r) <= (1e-12 if dtype == "f64" else 2e-6) * r, f"shape {cfg}"
+
+
+def test_state_moves_between_shapes():
+    """A shape changed between calls, a re-seed and a checkpoint file continue from the current state."""
+    out = []
+    for shapes in ((0, 0, 0), (6, 6, 0), (1, 6, 6)):
+        with Cavity(150, 70, Re=300.0, U=0.1, dtype="f32s") as cav:
+            for cfg, n in zip(shapes, (153, 100, 47)):
+                B.lbm_set_launch_config(cav.ctx, cfg)
+                cav.step(n)
+            fields = cav.moments()
+            first = cav.populations(host=True)
+            cav.set_moments(*fields)
+            cav.step(200)
+            out.append((first, cav.populations(host=True), cav.residual()))
+    for first, second, r in out[1:]:
+        assert np.array_equal(first, out[0][0]) and np.array_equal(second, out[0][1])
+        assert abs(r - out[0][2]) <= 2e-6 * r
