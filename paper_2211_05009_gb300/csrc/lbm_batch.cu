@@ -17,6 +17,7 @@
 // the read-only path: they are either L2 loads (ld.global.cg) or weak L1-cached loads, which are
 // coherent here because every read of a pool follows the grid barrier after its last write.
 //
+// FP32 batches large enough take their plain steps three per pass instead (k_batch_march).
 // Tile shape: rows per work item (1, 2, 4) x load path (L2 / L1); lbm_batch_autotune times each
 // on the batch's own state and keeps the fastest.  Whole checkpoint intervals (the plain launch
 // and the checkpoint launch) are captured once in a CUDA graph and replayed.
@@ -32,6 +33,7 @@
 
 #include "lbm.h"
 #include "lbm_internal.h"
+#include "lbm_march.cuh"
 #include "lbm_step_kernel.cuh"
 
 namespace lbm {
@@ -289,6 +291,159 @@ __global__ void __launch_bounds__(kBatchThreads, MINB) k_batch(const BatchArgs a
     }
 }
 
+// ------------------------------------------------------------------ fused plain steps
+// kBatchFuse plain steps per pass over memory for FP32 storage (lbm_march.cuh): one item is a strip of
+// columns of one cavity over a segment of its rows, and a grid barrier separates passes instead of
+// steps.  Three and not four steps: each pass changes the pool, so the pool of a state stays its
+// step's parity.  Segments are sized so that one item per warp covers the batch: rows of a warp =
+// strip-rows of the active cavities / warps, an eighth less in strips with a wall column, whose warps
+// take longer.  45 cavities 500 wide (13.5M nodes), f32s: 156 us a step taken by itself (HBM bound
+// at 0.92 of the copy rate), 90 us in fused passes (FP32 pipe; 500 columns fill 5 strips to 83 %).
+// Rows a warp from which plain steps are fused: a pass computes kBatchFuse - 1 rows of a segment
+// twice on average, and the row kernel spreads few rows over more warps.
+constexpr int kBatchFuseRows = 8;
+constexpr int kBatchFuse = 3, kBatchFuseV = 4, kBatchFuseBlocks = 3;
+using BatchStrips = StripGeometry<kBatchFuseV, kBatchFuse>;
+
+// Segments of one cavity at `rows` rows an inner item.
+__device__ __forceinline__ MarchGrid batch_grid(const BatchCav& c, int rows) {
+    MarchGrid g;
+    g.strips = BatchStrips::strips(c.nx);
+    const int side = max(2, rows - rows / 8), most = c.ny / 2;
+    g.segs = max(1, min((c.ny + rows - 1) / rows, most));
+    g.esegs = max(1, min((c.ny + side - 1) / side, most));
+    return g;
+}
+
+// a.nsteps plain steps, a multiple of kBatchFuse.
+template <typename S, bool SHIFTED>
+__global__ void __launch_bounds__(kBatchThreads, kBatchFuseBlocks) k_batch_march(const BatchArgs a) {
+    extern __shared__ __align__(16) unsigned char march_smem[];
+    __shared__ int s_active[LBM_BATCH_MAX];
+    __shared__ int s_prefix[LBM_BATCH_MAX + 1];
+    __shared__ int s_sum[kBatchThreads / 32];
+    BatchState* st = a.st;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int W = kBatchThreads / 32;
+    const int nwarps = gridDim.x * W;
+    const long long step0 = __ldcg(&st->step);
+    const int n = __ldcg(&st->n_active);
+    for (int k = threadIdx.x; k < n; k += blockDim.x) s_active[k] = __ldcg(&st->active[k]);
+    __syncthreads();
+    auto block_sum = [&](int v) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+        __syncthreads();
+        if (lane == 0) s_sum[warp] = v;
+        __syncthreads();
+        int t = 0;
+#pragma unroll
+        for (int w = 0; w < W; ++w) t += s_sum[w];
+        return t;
+    };
+    int v = 0;
+    for (int k = threadIdx.x; k < n; k += blockDim.x) {
+        const BatchCav& c = a.cavs[s_active[k]];
+        v += BatchStrips::strips(c.nx) * c.ny;
+    }
+    int rows = max(4, (block_sum(v) + nwarps - 1) / nwarps), items = 0;
+    for (int t = 0; t < 64; ++t) {  // until one item per warp covers the batch (ragged ends)
+        v = 0;
+        for (int k = threadIdx.x; k < n; k += blockDim.x) v += batch_grid(a.cavs[s_active[k]], rows).warps();
+        items = block_sum(v);
+        if (items <= nwarps) break;
+        rows += max(1, rows / 32);
+    }
+    if (warp == 0) {  // exclusive prefix of the items
+        int base = 0;
+        for (int k0 = 0; k0 < n; k0 += 32) {
+            const int own = k0 + lane < n ? batch_grid(a.cavs[s_active[k0 + lane]], rows).warps() : 0;
+            int inc = own;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int up = __shfl_up_sync(kFull, inc, o);
+                if (lane >= o) inc += up;
+            }
+            if (k0 + lane < n) s_prefix[k0 + lane] = base + inc - own;
+            base += __shfl_sync(kFull, inc, 31);
+        }
+        if (lane == 0) s_prefix[n] = base;
+    }
+    __syncthreads();
+
+    void* ring = march_smem + warp * march_ring_bytes<S, kBatchFuseV, kBatchFuse>();
+    for (int s = 0; s < a.nsteps; s += kBatchFuse) {
+        const long long step = step0 + s;
+        const bool odd = (step & 1) != 0;
+        const S* src_pool = static_cast<const S*>(odd ? a.pool[1] : a.pool[0]);
+        S* dst_pool = static_cast<S*>(odd ? a.pool[0] : a.pool[1]);
+        for (int item = blockIdx.x * W + warp; item < items; item += nwarps) {
+            int lo = 0, hi = n - 1;  // largest k with prefix[k] <= item
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (s_prefix[mid] <= item) lo = mid; else hi = mid - 1;
+            }
+            const BatchCav& cd = a.cavs[s_active[lo]];
+            CavityView<float> cv;
+            cv.nx = cd.nx;
+            cv.ny = cd.ny;
+            cv.pitch = cd.pitch;
+            cv.plane = cd.plane;
+            cv.omega = cd.omega_f;
+            cv.Ulid = cd.U_f;
+            cv.corner_moving = cd.corner_moving;
+            cv.sref = cv.sref_w = 0.0f;
+            ProbeOne pr;
+            pr.n_ = (cd.series && !a.no_probe) ? 1 : 0;
+            pr.px_ = cd.px;
+            pr.py_ = cd.py;
+            pr.every_ = cd.every > 0 ? cd.every : 1;
+            pr.start_ = cd.series ? __ldcg(&st->probe_start[s_active[lo]]) : 0;
+            pr.cap_ = cd.cap > 0 ? cd.cap : 1;
+            pr.series_ = cd.series;
+            int strip, y0, y1;
+            batch_grid(cd, rows).place(item - s_prefix[lo], cd.ny, strip, y0, y1);
+            march<S, SHIFTED, kBatchFuseV, kBatchFuse, true, 2>(src_pool + cd.off, dst_pool + cd.off, cv, lane,
+                                                                BatchStrips::begin(strip, cd.nx), y0, y1, kBatchFuse,
+                                                                pr, step, ring);
+        }
+        if (a.absent_block == (int)blockIdx.x && s == 0) return;  // test hook: never arrives
+        if (!grid_barrier(st, a.spin_limit)) return;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) st->step = step0 + a.nsteps;
+}
+
+template <typename S, bool SHIFTED>
+constexpr int batch_march_smem() { return kBatchThreads / 32 * march_ring_bytes<S, kBatchFuseV, kBatchFuse>(); }
+
+static cudaError_t launch_batch_march(int dtype, const BatchArgs& a, int blocks, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(kBatchThreads);
+    cfg.dynamicSmemBytes = batch_march_smem<float, true>();
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return dtype == 1 ? cudaLaunchKernelEx(&cfg, k_batch_march<float, false>, a) : cudaLaunchKernelEx(&cfg, k_batch_march<float, true>, a);
+}
+
+// Blocks of the cooperative fused launch on the current device (0: the query failed).
+static int batch_march_blocks(int dtype) {
+    const void* k = dtype == 1 ? (const void*)k_batch_march<float, false> : (const void*)k_batch_march<float, true>;
+    constexpr int smem = batch_march_smem<float, true>();
+    int dev = 0, sms = 0, per = 0;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+        cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, kBatchThreads, smem) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return per * sms;
+}
+
 template <typename S, bool SHIFTED, int HINT, int MINB>
 static cudaError_t launch_batch_h(const BatchArgs& a, bool reduce, int blocks, cudaStream_t st) {
     constexpr int V = sizeof(S) == 8 ? 2 : 4;
@@ -390,6 +545,8 @@ struct lbm_batch {
     DevState* h_ext = nullptr;  // pinned
     int shape = 0;              // index into kBatchShapes
     int blocks = 0;
+    int march_blocks = 0;       // blocks of the fused launch (0: none for this storage type)
+    bool fuse_slower = false;   // lbm_batch_autotune measured the fused passes slower
     long long step = 0;  // host mirror of the active step
     double spin_limit_s = 2.0;
     int absent_block = -1;
@@ -466,6 +623,33 @@ struct lbm_batch {
         return launch_batch(dtype, kBatchShapes[shape], a, reduce, blocks, st);
     }
 
+    // Whether plain steps run fused: FP32 storage while every warp has enough rows that the few a
+    // segment computes twice stay cheap.  Follows the active list as of the last pull_state.
+    bool fuses() const {
+        if (march_blocks <= 0 || fuse_slower) return false;
+        long long rows = 0;
+        for (int k = 0; k < h_state->n_active; ++k) {
+            const BatchCav& c = cavs[h_state->active[k]];
+            rows += (long long)BatchStrips::strips(c.nx) * c.ny;
+        }
+        return rows >= (long long)kBatchFuseRows * march_blocks * (kBatchThreads / 32);
+    }
+    // Enqueue a.nsteps plain steps.
+    cudaError_t launch_plain(BatchArgs a, bool fuse, cudaStream_t st) const {
+        const int all = a.nsteps, fused = fuse ? all / kBatchFuse * kBatchFuse : 0;
+        cudaError_t e = cudaSuccess;
+        if (fused > 0) {
+            a.nsteps = fused;
+            e = launch_batch_march(dtype, a, march_blocks, st);
+            a.absent_block = -1;
+        }
+        if (e == cudaSuccess && all > fused) {
+            a.nsteps = all - fused;
+            e = launch(a, false, st);
+        }
+        return e;
+    }
+
     // Cut every cavity into items of the shape's row count and rebuild the prefix of the active
     // list.  Needs a current h_state (after pull_state); leaves the upload queued on the stream.
     int relayout(int s) {
@@ -512,7 +696,8 @@ struct lbm_batch {
     // captured once per tile shape and barrier limit.  A capture the driver refuses leaves
     // graph_broken set and the intervals are launched directly.
     int ensure_graph() {
-        const long long key = shape * 1000003LL + (long long)(spin_limit_s * 1e6);
+        const bool fuse = fuses();
+        const long long key = (2 * shape + (fuse ? 1 : 0)) * 1000003LL + (long long)(spin_limit_s * 1e6);
         if (gexec && key == graph_key) return LBM_OK;
         if (gexec) cudaGraphExecDestroy(gexec);
         gexec = nullptr;
@@ -523,7 +708,7 @@ struct lbm_batch {
         cudaGraph_t g = nullptr;
         cudaError_t e = cudaStreamBeginCapture(cap_stream, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
-            cudaError_t e1 = launch(a, false, cap_stream);
+            cudaError_t e1 = launch_plain(a, fuse, cap_stream);
             a.nsteps = 1;
             if (e1 == cudaSuccess) e1 = launch(a, true, cap_stream);
             e = cudaStreamEndCapture(cap_stream, &g);
@@ -566,7 +751,7 @@ struct lbm_batch {
             const long long plain = ends_on_checkpoint ? chunk - 1 : chunk;
             if (plain > 0) {
                 a.nsteps = (int)plain;
-                rc = cuda(launch(a, false, stream), "batch kernel launch");
+                rc = cuda(launch_plain(a, fuses(), stream), "batch kernel launch");
                 if (rc) return rc;
                 a.absent_block = -1;
             }
@@ -657,6 +842,25 @@ struct lbm_batch {
                 if (rs < rp || (rs == rp && ms[s] < ms[pick])) pick = s;
             }
             best = pick;
+        }
+        // the fused passes against the chosen shape's single steps
+        if (!rc && best >= 0 && march_blocks > 0) {
+            fuse_slower = false;
+            if (fuses()) {
+                BatchArgs a = args(kBatchFuse);
+                a.no_probe = 1;
+                float t = 0.f;
+                const int m = (steps + kBatchFuse - 1) / kBatchFuse * kBatchFuse;
+                rc = cuda(launch_batch_march(dtype, a, march_blocks, stream), "autotune warm-up");
+                a.nsteps = m;
+                if (!rc) rc = cuda(cudaEventRecord(e0, stream), "event");
+                if (!rc) rc = cuda(launch_batch_march(dtype, a, march_blocks, stream), "autotune trial");
+                if (!rc) rc = cuda(cudaEventRecord(e1, stream), "event");
+                if (!rc) rc = sync();
+                if (!rc) rc = cuda(cudaEventElapsedTime(&t, e0, e1), "event time");
+                if (!rc) rc = pull_state();
+                if (!rc) fuse_slower = t / m > ms[best] / steps;
+            }
         }
         // restore: populations, the step counter, the chosen layout
         int rc2 = cuda(cudaMemcpyAsync(live, backup, pool_bytes, cudaMemcpyDeviceToDevice, stream), "population restore");
@@ -786,6 +990,7 @@ extern "C" int lbm_batch_create(int n, const int* nx, const int* ny, const doubl
     if (!rc) rc = b->sync();
     if (!rc) rc = b->relayout(0);
     if (rc) return fail(rc, "");
+    if (march_dtype(b->dtype)) b->march_blocks = batch_march_blocks(b->dtype);
     *out = b;
     return LBM_OK;
 }

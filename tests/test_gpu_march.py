@@ -55,3 +55,38 @@ def test_state_moves_between_shapes():
     for first, second, r in out[1:]:
         assert np.array_equal(first, out[0][0]) and np.array_equal(second, out[0][1])
         assert abs(r - out[0][2]) <= 2e-6 * r
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f32s"])
+def test_fused_batch_equals_single_cavities(dtype):
+    """A batch with rows enough to fuse its plain steps (uneven cavities, the smallest grid and one
+    whose right wall is alone in its strip among them), with probes, over graph replays, leftover
+    steps, a tile-shape trial in between and retirement."""
+    cases = [(130, 900 + 17 * i, 300.0 + 50 * i, 0.1) for i in range(8)] + [(3, 5, 10.0, 0.1), (121, 40, 200.0, 0.1), (241, 333, 500.0, 0.1)]
+    every, cap, n = 3, 200, len(cases)
+    nx, ny, re, u = zip(*cases)
+    b = B.lbm_batch_create(nx, ny, re, u, dtype)
+    B.lbm_batch_set_stream(b, torch.cuda.current_stream().cuda_stream)
+    series = torch.zeros((n, cap, 2), dtype=torch.float64, device="cuda")
+    try:
+        B.lbm_batch_probe(b, [0.5] * n, [0.3] * n, every, series, cap)
+        B.lbm_batch_step(b, 100)
+        B.lbm_batch_step(b, 37)
+        B.lbm_batch_autotune(b, 7)
+        B.lbm_batch_step(b, 214)
+        r, status = B.lbm_batch_residual(b, n)
+        assert (status == 0).all()
+        for i, (x, y, e, v) in enumerate(cases):
+            with Cavity(x, y, Re=e, U=v, dtype=dtype) as cav:
+                B.lbm_set_launch_config(cav.ctx, 0)
+                ser = cav.probe(0.5, 0.3, every=every, cap=cap)[1]
+                cav.step(351)
+                got = torch.empty((9, y, x), dtype=torch.float64, device="cuda")
+                B.lbm_batch_get_populations(b, i, got)
+                assert torch.equal(got, cav.populations()), f"cavity {i}"
+                assert torch.equal(series[i, :351 // every], ser[:351 // every]), f"cavity {i}"
+                assert abs(r[i] - cav.residual()) <= 2e-6 * r[i]
+        rc, done = B.lbm_batch_run_to_residual(b, n, 10.0, 200)  # everything retires at the next checkpoint
+        assert rc == B.LBM_OK and (done == 49).all()
+    finally:
+        B.lbm_batch_destroy(b)
