@@ -18,6 +18,7 @@
 #include <cstring>
 #include <random>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "lbm.h"
@@ -27,68 +28,59 @@
 namespace lbm {
 namespace nn {
 
-constexpr float kLeak = 0.1f;
+__device__ __forceinline__ __nv_bfloat16 as_bf16(float v) { return __float2bfloat16_rn(v); }
+__device__ __forceinline__ __nv_bfloat16 as_bf16(__nv_bfloat16 v) { return v; }
 
-__global__ void k_im2col_pk(const float* __restrict__ x1, int c1, const float* __restrict__ x2, int c2,
-                            int H, int W, int Kp, __nv_bfloat16* __restrict__ out) {
-    // out[p][k], k = ci*9 + ky*3 + kx over the channels of x1 then x2; zeros past C*9 and outside
-    const long long P = (long long)H * W;
+// out[p][k], k = ci*9 + ky*3 + kx over the channels of x1 then x2; zeros past C*9 and outside: eight
+// values and one 16-byte store per thread (Kp is a multiple of 8)
+template <typename X>
+__global__ void __launch_bounds__(256) k_im2col_pk(const X* __restrict__ x1, int c1, const X* __restrict__ x2, int c2, int H,
+                                                   int W, int Kp, __nv_bfloat16* __restrict__ out) {
+    const int P = H * W, octets = Kp / 8;
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= P * Kp) return;
-    const int k = (int)(idx % Kp);
-    const long long p = idx / Kp;
-    const int C = c1 + c2;
-    float v = 0.f;
-    if (k < C * 9) {
-        const int ci = k / 9, r = k % 9, ky = r / 3, kx = r % 3;
-        const int y = (int)(p / W) + ky - 1, x = (int)(p % W) + kx - 1;
-        if (y >= 0 && y < H && x >= 0 && x < W)
-            v = ci < c1 ? x1[((long long)ci * H + y) * W + x] : x2[((long long)(ci - c1) * H + y) * W + x];
+    if (idx >= (long long)P * octets) return;
+    const int p = (int)(idx / octets), k0 = (int)(idx - (long long)p * octets) * 8;
+    const int py = p / W, px = p - py * W;
+    __nv_bfloat16 v[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const int k = k0 + j, ci = k / 9, r = k - ci * 9, y = py + r / 3 - 1, x = px + r % 3 - 1;
+        v[j] = as_bf16(0.f);
+        if (ci < c1 + c2 && y >= 0 && y < H && x >= 0 && x < W)
+            v[j] = as_bf16(ci < c1 ? x1[((long long)ci * H + y) * W + x] : x2[((long long)(ci - c1) * H + y) * W + x]);
     }
-    out[idx] = __float2bfloat16_rn(v);
+    *reinterpret_cast<uint4*>(out + (long long)p * Kp + k0) = *reinterpret_cast<const uint4*>(v);
 }
 
-__global__ void k_im2col_kp(const float* __restrict__ x1, int c1, const float* __restrict__ x2, int c2,
-                            int H, int W, int Kp, __nv_bfloat16* __restrict__ out) {
-    // out[k][p]
-    const long long P = (long long)H * W;
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= P * Kp) return;
-    const long long p = idx % P;
-    const int k = (int)(idx / P);
-    const int C = c1 + c2;
-    float v = 0.f;
-    if (k < C * 9) {
-        const int ci = k / 9, r = k % 9, ky = r / 3, kx = r % 3;
-        const int y = (int)(p / W) + ky - 1, x = (int)(p % W) + kx - 1;
-        if (y >= 0 && y < H && x >= 0 && x < W)
-            v = ci < c1 ? x1[((long long)ci * H + y) * W + x] : x2[((long long)(ci - c1) * H + y) * W + x];
+// out[k][p], eight pixels and one 16-byte store per thread (P is a multiple of 8)
+__global__ void __launch_bounds__(256) k_im2col_kp(const float* __restrict__ x1, int c1, const float* __restrict__ x2,
+                                                   int c2, int H, int W, __nv_bfloat16* __restrict__ out) {
+    const int P = H * W, p0 = (blockIdx.x * blockDim.x + threadIdx.x) * 8;
+    if (p0 >= P) return;
+    const int k = blockIdx.y, ci = k / 9, tap = k - ci * 9, ky = tap / 3 - 1, kx = tap % 3 - 1;
+    __nv_bfloat16 v[8];
+    if (ci < c1 + c2) {
+        const float* __restrict__ x = ci < c1 ? x1 + (long long)ci * P : x2 + (long long)(ci - c1) * P;
+        int yy = p0 / W + ky, xx = p0 % W + kx;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const bool in = yy >= 0 && yy < H && xx >= 0 && xx < W;
+            v[j] = __float2bfloat16_rn(in ? x[yy * W + xx] : 0.f);
+            if (++xx == W + kx) {
+                xx = kx;
+                ++yy;
+            }
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = __float2bfloat16_rn(0.f);
     }
-    out[idx] = __float2bfloat16_rn(v);
+    *reinterpret_cast<uint4*>(out + (long long)k * P + p0) = *reinterpret_cast<const uint4*>(v);
 }
 
 __global__ void k_to_bf16(const float* __restrict__ x, long long n, __nv_bfloat16* __restrict__ y) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) y[i] = __float2bfloat16_rn(x[i]);
-}
-
-// wq[co][Kp] = w[co][k] (k < ci*9), wf[ci][Kp2] with wf[ci][co*9 + (8 - r)] = w[co][ci*9 + r]
-__global__ void k_prep_weights(const float* __restrict__ w, int ci, int co, int Kp, int Kp2,
-                               __nv_bfloat16* __restrict__ wq, __nv_bfloat16* __restrict__ wf) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx < co * Kp) {
-        const int o = idx / Kp, k = idx % Kp;
-        wq[idx] = __float2bfloat16_rn(k < ci * 9 ? w[o * ci * 9 + k] : 0.f);
-    }
-    if (idx < ci * Kp2) {
-        const int i = idx / Kp2, k = idx % Kp2;
-        float v = 0.f;
-        if (k < co * 9) {
-            const int o = k / 9, r = 8 - k % 9;
-            v = w[(o * ci + i) * 9 + r];
-        }
-        wf[idx] = __float2bfloat16_rn(v);
-    }
 }
 
 __global__ void k_bias_act(float* __restrict__ y, const float* __restrict__ b, int C, long long P, int act) {
@@ -121,6 +113,108 @@ __global__ void k_act_back(const float* __restrict__ y, const float* __restrict_
     if (threadIdx.x == 0) db[c] += sh[0];
 }
 
+// ------------------------------------------------------------------ channels-last operands
+// Input of a convolution as BF16, channels-last [pixel][Cp], zero padded: one pixel and 8 channels per
+// thread.  MODE 0: x1 ++ x2.  MODE 1: the 2x2 average of x1 (an image of twice the size).  MODE 2: the
+// nearest x2 upsampling of x1 (half the size) ++ x2.  In modes 1 and 2 the c1 channels also go to y in
+// FP32, which the weight gradient reads.
+template <int MODE>
+__global__ void __launch_bounds__(256) k_to_channels_last(const float* __restrict__ x1, int c1, const float* __restrict__ x2,
+                                                          int c2, int H, int W, int Cp, float* __restrict__ y,
+                                                          __nv_bfloat16* __restrict__ X) {
+    const int P = H * W, p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= P) return;
+    const int cg = blockIdx.y * 8, yy = p / W, xx = p - yy * W;
+    __nv_bfloat16 b[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const int c = cg + j;
+        float v = 0.f;
+        if (c < c1) {
+            if constexpr (MODE == 0) {
+                v = x1[(long long)c * P + p];
+            } else if constexpr (MODE == 1) {
+                const float* s = x1 + ((long long)c * 2 * H + 2 * yy) * 2 * W + 2 * xx;
+                const float2 u = *reinterpret_cast<const float2*>(s), w = *reinterpret_cast<const float2*>(s + 2 * W);
+                v = 0.25f * ((u.x + u.y) + (w.x + w.y));
+            } else {
+                v = x1[((long long)c * (H / 2) + yy / 2) * (W / 2) + xx / 2];
+            }
+            if constexpr (MODE != 0) y[(long long)c * P + p] = v;
+        } else if (c < c1 + c2) {
+            v = x2[(long long)(c - c1) * P + p];
+        }
+        b[j] = __float2bfloat16_rn(v);
+    }
+    *reinterpret_cast<uint4*>(X + (long long)p * Cp + cg) = *reinterpret_cast<const uint4*>(b);
+}
+
+// dz = dy act'(y) in BF16, channel-major [co][P] (the weight gradient's operand) and channels-last
+// [P][Cp] (the data gradient's input), and db[c] += sum_p dz in FP32: one pixel and 8 channels per
+// thread.
+__global__ void __launch_bounds__(256) k_act_back_cl(const float* __restrict__ y, const float* __restrict__ dy, int C, int P,
+                                                     int Cp, int act, float* __restrict__ db, __nv_bfloat16* __restrict__ dzq,
+                                                     __nv_bfloat16* __restrict__ X) {
+    __shared__ float sh[8][8];
+    const int p = blockIdx.x * blockDim.x + threadIdx.x, cg = blockIdx.y * 8;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    __nv_bfloat16 b[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const int c = cg + j;
+        float g = 0.f;
+        if (c < C && p < P) {
+            const long long i = (long long)c * P + p;
+            g = dy[i];
+            if (act && y[i] <= 0.f) g *= kLeak;
+            dzq[i] = __float2bfloat16_rn(g);
+        }
+        b[j] = __float2bfloat16_rn(g);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+        if (lane == 0) sh[warp][j] = g;
+    }
+    if (p < P) *reinterpret_cast<uint4*>(X + (long long)p * Cp + cg) = *reinterpret_cast<const uint4*>(b);
+    __syncthreads();
+    if (threadIdx.x < 8 && cg + threadIdx.x < C) {
+        float s = 0.f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) s += sh[w][threadIdx.x];
+        atomicAdd(db + cg + threadIdx.x, s);
+    }
+}
+
+// Weights of every convolution as BF16 from the FP32 parameters, one launch per change of them.
+// wq[o][Kp]: k = i*9 + tap; wf[i][Kp2]: k = o*9 + tap with the taps flipped (the data gradient's).
+// The same tap-major and zero padded: wt[o][tap][cpi], wb[i][tap][cpo].
+struct ConvDev {
+    int ci, co, Kp, Kp2, cpi, cpo;
+    long long woff, wq, wf, wt, wb;
+};
+__global__ void __launch_bounds__(256) k_prep_weights(const ConvDev* __restrict__ convs, const float* __restrict__ params,
+                                                      __nv_bfloat16* __restrict__ wq, __nv_bfloat16* __restrict__ wf,
+                                                      __nv_bfloat16* __restrict__ taps) {
+    const ConvDev c = convs[blockIdx.y];
+    const float* __restrict__ w = params + c.woff;
+    const int stride = gridDim.x * blockDim.x, first = blockIdx.x * blockDim.x + threadIdx.x;
+    for (int i = first; i < c.co * c.Kp; i += stride) {
+        const int o = i / c.Kp, k = i - o * c.Kp;
+        wq[c.wq + i] = __float2bfloat16_rn(k < c.ci * 9 ? w[o * c.ci * 9 + k] : 0.f);
+    }
+    for (int i = first; i < c.ci * c.Kp2; i += stride) {
+        const int ch = i / c.Kp2, k = i - ch * c.Kp2, o = k / 9;
+        wf[c.wf + i] = __float2bfloat16_rn(o < c.co ? w[(o * c.ci + ch) * 9 + 8 - (k - o * 9)] : 0.f);
+    }
+    for (int i = first; i < c.co * 9 * c.cpi; i += stride) {
+        const int o = i / (9 * c.cpi), r = i - o * 9 * c.cpi, tap = r / c.cpi, ch = r - tap * c.cpi;
+        taps[c.wt + i] = __float2bfloat16_rn(ch < c.ci ? w[(o * c.ci + ch) * 9 + tap] : 0.f);
+    }
+    for (int i = first; i < c.ci * 9 * c.cpo; i += stride) {
+        const int ch = i / (9 * c.cpo), r = i - ch * 9 * c.cpo, tap = r / c.cpo, o = r - tap * c.cpo;
+        taps[c.wb + i] = __float2bfloat16_rn(o < c.co ? w[(o * c.ci + ch) * 9 + 8 - tap] : 0.f);
+    }
+}
+
 __global__ void k_pool2(const float* __restrict__ x, int C, int H, int W, float* __restrict__ y) {
     const int h = H / 2, w = W / 2;
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -145,21 +239,24 @@ __global__ void k_up2(const float* __restrict__ x, int C, int h, int w, float* _
     y[i] = x[((long long)c * h + yy / 2) * w + xx / 2];
 }
 
+template <bool STORE>
 __global__ void k_up2_back(const float* __restrict__ dy, int C, int h, int w, float* __restrict__ dx) {
     const int W = 2 * w;
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (long long)C * h * w) return;
     const int xx = (int)(i % w), yy = (int)((i / w) % h), c = (int)(i / ((long long)w * h));
     const float* s = dy + ((long long)c * 2 * h + 2 * yy) * W + 2 * xx;
-    dx[i] += (s[0] + s[1]) + (s[W] + s[W + 1]);
+    const float v = (s[0] + s[1]) + (s[W] + s[W + 1]);
+    dx[i] = STORE ? v : dx[i] + v;
 }
 
 // Number of valid pixels (mask is 0/1) into cnt[0].
 // stats[0] = sum mask (the count n); stats[2] = sum mask (base + out - target)_0 / n, the mean
 // density-channel error, which the loss ignores (one block, fixed order).
-__global__ void k_mask_stats(const float* __restrict__ mask, const float* __restrict__ out, const float* __restrict__ base,
-                             const float* __restrict__ tgt, long long P, double* stats) {
-    __shared__ double sh[2][256];
+__global__ void __launch_bounds__(1024) k_mask_stats(const float* __restrict__ mask, const float* __restrict__ out,
+                                                     const float* __restrict__ base, const float* __restrict__ tgt,
+                                                     long long P, double* stats) {
+    __shared__ double sh[2][1024];
     double s = 0.0, e = 0.0;
     for (long long i = threadIdx.x; i < P; i += blockDim.x) {
         s += mask[i];
@@ -168,7 +265,7 @@ __global__ void k_mask_stats(const float* __restrict__ mask, const float* __rest
     sh[0][threadIdx.x] = s;
     sh[1][threadIdx.x] = e;
     __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
+    for (int o = 512; o > 0; o >>= 1) {
         if (threadIdx.x < o) {
             sh[0][threadIdx.x] += sh[0][threadIdx.x + o];
             sh[1][threadIdx.x] += sh[1][threadIdx.x + o];
@@ -207,12 +304,18 @@ __global__ void k_mse(const float* __restrict__ out, const float* __restrict__ b
     if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
 }
 
-// loss[1] = sum(part) / (3 loss[0])
-__global__ void k_sum_parts(const double* part, int n, double* loss) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// loss[1] = sum(part) / (3 loss[0]) (one block, fixed order)
+__global__ void __launch_bounds__(256) k_sum_parts(const double* part, int n, double* loss) {
+    __shared__ double sh[256];
     double s = 0.0;
-    for (int i = 0; i < n; ++i) s += part[i];
-    loss[1] = s / (3.0 * loss[0]);
+    for (int i = threadIdx.x; i < n; i += 256) s += part[i];
+    sh[threadIdx.x] = s;
+    __syncthreads();
+    for (int o = 128; o > 0; o >>= 1) {
+        if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) loss[1] = sh[0] / (3.0 * loss[0]);
 }
 
 __global__ void k_adam(float* __restrict__ w, const float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
@@ -347,7 +450,12 @@ struct lbm_net {
     std::vector<long long> act_size;
     __nv_bfloat16* col = nullptr;  // im2col scratch (backend 3: the channels-last BF16 input)
     long long col_elems = 0;
-    __nv_bfloat16* wtap = nullptr;  // backend 3: the current conv's weights, tap-major
+    // backend 3: two channels-last inputs (a convolution reads one and writes the next one's), and the
+    // weights of every convolution tap-major, laid out once per change of the parameters
+    __nv_bfloat16* cl[2] = {nullptr, nullptr};
+    __nv_bfloat16* taps = nullptr;
+    ConvDev* d_convs = nullptr;
+    std::vector<ConvDev> devs;
     float* dz = nullptr;            // dZ scratch (largest tensor)
     __nv_bfloat16* dzq = nullptr;   // dZ in BF16
     double* parts = nullptr;
@@ -432,11 +540,13 @@ int ensure_buffers(lbm_net* n, int H, int W) {
     n->gact.clear();
     n->act_size.clear();
     cudaFree(n->col);
-    cudaFree(n->wtap);
+    for (auto& p : n->cl) {
+        cudaFree(p);
+        p = nullptr;
+    }
     cudaFree(n->dz);
     cudaFree(n->dzq);
     n->col = nullptr;
-    n->wtap = nullptr;
     n->dz = nullptr;
     n->dzq = nullptr;
     Graph g = make_graph(n->ch);
@@ -453,13 +563,8 @@ int ensure_buffers(lbm_net* n, int H, int W) {
         n->act_size.push_back(sz);
         maxt = std::max(maxt, sz);
     }
-    long long maxcol = 0;
-    for (auto& c : n->convs) {
-        // find the level of this conv from its output tensor is not tracked: bound by level 0
-        maxcol = std::max(maxcol, (long long)std::max(c.Kp, c.Kp2));
-    }
     // im2col scratch: largest (pixels at the conv's level) x (Kp or Kp2); bound generously
-    long long need = 0;
+    long long need = 0, cl = 0;
     {
         std::vector<std::pair<int, int>> io;
         conv_list(n->ch, io);
@@ -468,14 +573,12 @@ int ensure_buffers(lbm_net* n, int H, int W) {
             const ConvSpec& c = n->convs[i];
             const long long P = (long long)(H >> lv[i]) * (W >> lv[i]);
             need = std::max(need, P * (long long)std::max(c.Kp, c.Kp2));
-            need = std::max(need, P * (long long)std::max(conv_cp(c.ci), conv_cp(c.co)));  // channels-last inputs
+            cl = std::max(cl, P * (long long)std::max(conv_cp(c.ci), conv_cp(c.co)));
         }
     }
-    long long wtap_elems = 0;
-    for (auto& c : n->convs)
-        wtap_elems = std::max(wtap_elems, 9ll * std::max((long long)c.co * conv_cp(c.ci), (long long)c.ci * conv_cp(c.co)));
     n->col_elems = need;
-    if (cudaMalloc(&n->col, need * 2) != cudaSuccess || cudaMalloc(&n->wtap, wtap_elems * 2) != cudaSuccess ||
+    if (cudaMalloc(&n->col, need * 2) != cudaSuccess || cudaMalloc(&n->cl[0], cl * 2) != cudaSuccess ||
+        cudaMalloc(&n->cl[1], cl * 2) != cudaSuccess ||
         cudaMalloc(&n->dz, maxt * 4) != cudaSuccess || cudaMalloc(&n->dzq, maxt * 2) != cudaSuccess) {
         cudaGetLastError();
         return n->fail(LBM_ENOMEM, "network scratch buffers");
@@ -487,36 +590,53 @@ int ensure_buffers(lbm_net* n, int H, int W) {
 
 int prep_weights(lbm_net* n) {
     if (!n->weights_dirty) return LBM_OK;
-    for (auto& c : n->convs) {
-        const int cnt = std::max(c.co * c.Kp, c.ci * c.Kp2);
-        k_prep_weights<<<nblk(cnt), 256, 0, n->stream>>>(n->params + c.woff, c.ci, c.co, c.Kp, c.Kp2, n->wq + c.wq_off,
-                                                         n->wf + c.wf_off);
-    }
+    k_prep_weights<<<dim3(64, (unsigned)n->convs.size()), 256, 0, n->stream>>>(n->d_convs, n->params, n->wq, n->wf, n->taps);
     n->weights_dirty = false;
     return n->cuda(cudaGetLastError(), "weight preparation");
+}
+
+// Backend 3: cl[to] = channels-last input of a convolution (k_to_channels_last).
+template <int MODE>
+int channels_last(lbm_net* n, int to, const float* x1, int c1, const float* x2, int c2, int H, int W, float* y) {
+    const int Cp = conv_cp(c1 + c2);
+    k_to_channels_last<MODE><<<dim3(nblk((long long)H * W), (unsigned)(Cp / 8)), 256, 0, n->stream>>>(x1, c1, x2, c2, H, W, Cp, y,
+                                                                                                   n->cl[to]);
+    return n->cuda(cudaGetLastError(), "channels-last input");
+}
+
+// Backend 3: y = act(conv(cl[from]) + b) in one kernel; chain: the result also becomes cl[from ^ 1].
+int conv_cl(lbm_net* n, int ci, int from, int H, int W, float* y, bool chain) {
+    const ConvSpec& c = n->convs[ci];
+    return n->cuda(conv3x3_channels_last(n->cl[from], c.ci, H, W, n->taps + n->devs[ci].wt, c.co, y, n->params + c.boff,
+                                         c.act != 0, nullptr, 0, chain ? n->cl[from ^ 1] : nullptr, n->d_err, n->stream),
+                   "conv (tcgen05, TMA boxes)");
+}
+
+// Backend 3, images that the channels-last convolution does not take (deep levels of ragged heights,
+// widths like 192): the explicit im2col, with the layer's epilogue in the product all the same.
+int conv_im2col(lbm_net* n, int ci, const float* x1, int c1, const float* x2, int c2, int H, int W, float* y) {
+    const ConvSpec& c = n->convs[ci];
+    const int P = H * W;
+    k_im2col_pk<float><<<nblk((long long)P * c.Kp / 8), 256, 0, n->stream>>>(x1, c1, x2, c2, H, W, c.Kp, n->col);
+    int rc = n->cuda(cudaGetLastError(), "im2col");
+    if (!rc) rc = n->cuda(gemm_bf16_nt_umma_layer(P, c.co, c.Kp, n->col, n->wq + c.wq_off, y, n->params + c.boff, c.act != 0, nullptr, 0,
+                                                  n->d_err, n->stream), "conv gemm (tcgen05)");
+    return rc;
 }
 
 // y (tensor) = act(conv(x1 ++ x2) + b)
 int conv_fwd(lbm_net* n, const ConvSpec& c, const float* x1, int c1, const float* x2, int c2, int H, int W, float* y) {
     const long long P = (long long)H * W;
     int rc = LBM_OK;
-    bool implicit = n->backend == 2 || n->backend == 3;
-    if (n->backend == 2) {  // implicit GEMM: the im2col rows are gathered inside the tensor-core kernel
+    bool implicit = n->backend == 2;
+    if (implicit) {  // implicit GEMM: the im2col rows are gathered inside the tensor-core kernel
         const cudaError_t e = conv3x3_bf16_umma(x1, c1, x2, c2, H, W, c.Kp, n->wq + c.wq_off, c.co, y, (int)P, kStore,
                                                 true, n->d_err, n->stream);
         if (e == cudaErrorInvalidValue) implicit = false;  // shape it does not take: explicit im2col below
         else rc = n->cuda(e, "conv (tcgen05 implicit)");
-    } else if (n->backend == 3) {  // implicit GEMM over the channels-last input, A tiles by TMA boxes
-        rc = n->cuda(weights_tap_major(n->wq + c.wq_off, c.Kp, c1 + c2, c.co, n->wtap, n->stream), "tap-major weights");
-        if (!rc) {
-            const cudaError_t e = conv3x3_bf16_tma(x1, c1, x2, c2, H, W, n->wtap, c.co, y, (int)P, kStore, true, n->col,
-                                                   n->d_err, n->stream);
-            if (e == cudaErrorInvalidValue) implicit = false;  // shape it does not take: explicit im2col below
-            else rc = n->cuda(e, "conv (tcgen05, TMA boxes)");
-        }
     }
     if (!implicit) {
-        k_im2col_pk<<<nblk(P * c.Kp), 256, 0, n->stream>>>(x1, c1, x2, c2, H, W, c.Kp, n->col);
+        k_im2col_pk<float><<<nblk(P * c.Kp / 8), 256, 0, n->stream>>>(x1, c1, x2, c2, H, W, c.Kp, n->col);
         rc = n->cuda(cudaGetLastError(), "im2col");
     }
     if (!rc && !implicit) {
@@ -534,6 +654,39 @@ int conv_fwd(lbm_net* n, const ConvSpec& c, const float* x1, int c1, const float
     return rc;
 }
 
+int im2col_kp(lbm_net* n, const ConvSpec& c, const float* x1, int c1, const float* x2, int c2, int H, int W) {
+    k_im2col_kp<<<dim3(nblk((long long)H * W / 8), (unsigned)c.Kp), 256, 0, n->stream>>>(x1, c1, x2, c2, H, W, n->col);
+    return n->cuda(cudaGetLastError(), "im2col (k-major)");
+}
+
+// Backend 3: given dL/dy (gy) and y, accumulate dW and db and store dL/dx (gx1: c1 channels, gx2: c2).
+// The weight gradient is split over the pixels until its tiles fill the GPU, down to four K steps each:
+// with one slice per 4096 pixels a 128-wide level-0 layer ran on 8 CTAs.
+int conv_bwd_cl(lbm_net* n, int ci, const float* x1, int c1, const float* x2, int c2, int H, int W, const float* y,
+                const float* gy, float* gx1, float* gx2) {
+    const ConvSpec& c = n->convs[ci];
+    const int P = H * W, cp = conv_cp(c.co);
+    k_act_back_cl<<<dim3(nblk(P), (unsigned)(cp / 8)), 256, 0, n->stream>>>(y, gy, c.co, P, cp, c.act, n->grads + c.boff, n->dzq,
+                                                                         n->cl[0]);
+    int rc = n->cuda(cudaGetLastError(), "activation backward");
+    if (!rc) rc = im2col_kp(n, c, x1, c1, x2, c2, H, W);
+    if (!rc) {
+        const int tiles = (c.ci * 9 + 127) / 128, split = std::max(1, std::min(152 / tiles, P / 256));
+        rc = n->cuda(gemm_bf16_nt_umma(c.ci * 9, c.co, P, n->col, P, n->dzq, P, n->grads + c.woff, c.ci * 9, kAtomicAdd, true, split,
+                                       n->d_err, n->stream), "weight-gradient gemm (tcgen05)");
+    }
+    if (rc || !gx1) return rc;
+    const int rows = c1 + (gx2 ? c2 : 0);
+    if (conv_tma_takes(H, W))
+        return n->cuda(conv3x3_channels_last(n->cl[0], c.co, H, W, n->taps + n->devs[ci].wb, rows, gx1, nullptr, false, gx2, c1, nullptr,
+                                             n->d_err, n->stream), "data-gradient conv (tcgen05, TMA boxes)");
+    k_im2col_pk<__nv_bfloat16><<<nblk((long long)P * c.Kp2 / 8), 256, 0, n->stream>>>(n->dzq, c.co, nullptr, 0, H, W, c.Kp2, n->col);
+    rc = n->cuda(cudaGetLastError(), "im2col of dZ");
+    if (!rc) rc = n->cuda(gemm_bf16_nt_umma_layer(P, rows, c.Kp2, n->col, n->wf + c.wf_off, gx1, nullptr, false, gx2, c1, n->d_err,
+                                                  n->stream), "data-gradient gemm (tcgen05)");
+    return rc;
+}
+
 // given dL/dy (gy) and y: accumulate dW, db; accumulate dL/dx into gx1 (c1 channels), gx2 (c2)
 int conv_bwd(lbm_net* n, const ConvSpec& c, const float* x1, int c1, const float* x2, int c2, int H, int W,
              const float* y, const float* gy, float* gx1, float* gx2) {
@@ -544,8 +697,7 @@ int conv_bwd(lbm_net* n, const ConvSpec& c, const float* x1, int c1, const float
     // weight gradient: dW[co][k] += sum_p dZ[co][p] XcT[k][p]; accumulate in a scratch of Kp
     // columns is not needed: the GEMM writes only k < ci*9 when N = ci*9 (ldc = ci*9)
     if (!rc) {
-        k_im2col_kp<<<nblk(P * c.Kp), 256, 0, n->stream>>>(x1, c1, x2, c2, H, W, c.Kp, n->col);
-        rc = n->cuda(cudaGetLastError(), "im2col (k-major)");
+        rc = im2col_kp(n, c, x1, c1, x2, c2, H, W);
     }
     if (!rc) {
         const int split = P >= 16384 ? (int)std::min<long long>(32, P / 4096) : 1;
@@ -560,23 +712,8 @@ int conv_bwd(lbm_net* n, const ConvSpec& c, const float* x1, int c1, const float
     if (!rc && (gx1 || gx2)) {
         const __nv_bfloat16* wf1 = n->wf + c.wf_off;
         const __nv_bfloat16* wf2 = wf1 + (long long)c1 * c.Kp2;
-        bool implicit = n->backend == 2 || n->backend == 3;
-        if (n->backend == 3) {  // over dZ (co channels) with the flipped weights, tap-major
-            bool first = true;
-            for (int part = 0; part < 2 && !rc && implicit; ++part) {
-                float* gx = part == 0 ? gx1 : gx2;
-                if (!gx) continue;
-                const int rows = part == 0 ? c1 : c2;
-                rc = n->cuda(weights_tap_major(part == 0 ? wf1 : wf2, c.Kp2, c.co, rows, n->wtap, n->stream),
-                             "tap-major weights");
-                if (rc) break;
-                const cudaError_t e = conv3x3_bf16_tma(n->dz, c.co, nullptr, 0, H, W, n->wtap, rows, gx, (int)P, kAccumulate,
-                                                       true, n->col, n->d_err, n->stream);
-                if (e == cudaErrorInvalidValue && first) implicit = false;  // explicit im2col below
-                else rc = n->cuda(e, "data-gradient conv (tcgen05, TMA boxes)");
-                first = false;
-            }
-        } else if (implicit) {  // implicit GEMM over dZ (co channels) with the flipped weights
+        bool implicit = n->backend == 2;
+        if (implicit) {  // implicit GEMM over dZ (co channels) with the flipped weights
             bool first = true;  // a shape the kernel does not take is refused before anything launches
             for (int part = 0; part < 2 && !rc && implicit; ++part) {
                 float* gx = part == 0 ? gx1 : gx2;
@@ -590,7 +727,7 @@ int conv_bwd(lbm_net* n, const ConvSpec& c, const float* x1, int c1, const float
             }
         }
         if (!implicit) {
-            k_im2col_pk<<<nblk(P * c.Kp2), 256, 0, n->stream>>>(n->dz, c.co, nullptr, 0, H, W, c.Kp2, n->col);
+            k_im2col_pk<float><<<nblk(P * c.Kp2 / 8), 256, 0, n->stream>>>(n->dz, c.co, nullptr, 0, H, W, c.Kp2, n->col);
             rc = n->cuda(cudaGetLastError(), "im2col of dZ");
         }
         if (!implicit && n->backend != 0) {
@@ -612,12 +749,51 @@ int conv_bwd(lbm_net* n, const ConvSpec& c, const float* x1, int c1, const float
     return rc;
 }
 
+// Backend 3: one kernel per convolution and one for the input of each that does not simply follow
+// another convolution.
+int forward_cl(lbm_net* n, const Graph& g, int H, int W) {
+    auto A = [&](int t) { return n->act[t]; };
+    int rc = LBM_OK, ci = 0;
+    // the two convolutions of a stage: MODE x1 (++ x2) -> mid -> out; up: x1's FP32 image (MODE 1, 2)
+    auto stage = [&](auto mode, const float* x1, int c1, const float* x2, int c2, int h, int w, float* up, float* mid, int cm,
+                     float* out, bool chain) {
+        constexpr int MODE = decltype(mode)::value;
+        if (conv_tma_takes(h, w)) {
+            rc = channels_last<MODE>(n, 0, x1, c1, x2, c2, h, w, up);
+            if (!rc) rc = conv_cl(n, ci, 0, h, w, mid, true);
+            if (!rc) rc = conv_cl(n, ci + 1, 1, h, w, out, chain);
+        } else {
+            const long long P = (long long)c1 * h * w;
+            if (MODE == 1) k_pool2<<<nblk(P), 256, 0, n->stream>>>(x1, c1, 2 * h, 2 * w, up);
+            if (MODE == 2) k_up2<<<nblk(P), 256, 0, n->stream>>>(x1, c1, h / 2, w / 2, up);
+            rc = n->cuda(cudaGetLastError(), "pool / upsample");
+            if (!rc) rc = conv_im2col(n, ci, MODE ? up : x1, c1, x2, c2, h, w, mid);
+            if (!rc) rc = conv_im2col(n, ci + 1, mid, cm, nullptr, 0, h, w, out);
+        }
+        ci += 2;
+    };
+    stage(std::integral_constant<int, 0>{}, A(g.input), 7, nullptr, 0, H, W, nullptr, A(g.a[0]), n->ch[0], A(g.e[0]), false);
+    for (int l = 1; l < 5 && !rc; ++l)
+        stage(std::integral_constant<int, 1>{}, A(g.e[l - 1]), n->ch[l - 1], nullptr, 0, H >> l, W >> l, A(g.p[l]), A(g.a[l]),
+              n->ch[l], A(g.e[l]), false);
+    for (int l = 3; l >= 0 && !rc; --l)
+        stage(std::integral_constant<int, 2>{}, A(l == 3 ? g.e[4] : g.d[l + 1]), n->ch[l + 1], A(g.e[l]), n->ch[l], H >> l, W >> l,
+              A(g.u[l]), A(g.b[l]), n->ch[l], A(g.d[l]), l == 0);
+    if (rc) return rc;
+    return conv_tma_takes(H, W) ? conv_cl(n, ci, 0, H, W, A(g.out), false)
+                                : conv_im2col(n, ci, A(g.d[0]), n->ch[0], nullptr, 0, H, W, A(g.out));
+}
+
 int forward(lbm_net* n, const float* in, int H, int W) {
     int rc = ensure_buffers(n, H, W);
     if (!rc) rc = prep_weights(n);
     if (rc) return rc;
     Graph g = make_graph(n->ch);
     auto A = [&](int t) { return n->act[t]; };
+    if (n->backend == 3) {
+        rc = n->cuda(cudaMemcpyAsync(A(g.input), in, n->act_size[g.input] * 4, cudaMemcpyDeviceToDevice, n->stream), "input copy");
+        return rc ? rc : forward_cl(n, g, H, W);
+    }
     rc = n->cuda(cudaMemcpyAsync(A(g.input), in, n->act_size[g.input] * 4, cudaMemcpyDeviceToDevice, n->stream), "input copy");
     int ci = 0;  // conv index
     for (int l = 0; l < 5 && !rc; ++l) {
@@ -643,11 +819,42 @@ int forward(lbm_net* n, const float* in, int H, int W) {
     return rc;
 }
 
+// Backend 3.  Every gradient tensor but e[0..3] has one contribution and is stored, not accumulated;
+// e[l] gets the skip's first (decoder) and the pooling's added (encoder).
+int backward_cl(lbm_net* n, const Graph& g, int H, int W, const float* gout) {
+    auto A = [&](int t) { return n->act[t]; };
+    auto G = [&](int t) { return n->gact[t]; };
+    int ci = (int)n->convs.size() - 1;
+    int rc = conv_bwd_cl(n, ci--, A(g.d[0]), n->ch[0], nullptr, 0, H, W, A(g.out), gout, G(g.d[0]), nullptr);
+    for (int l = 0; l <= 3 && !rc; ++l) {
+        const int h = H >> l, w = W >> l;
+        rc = conv_bwd_cl(n, ci--, A(g.b[l]), n->ch[l], nullptr, 0, h, w, A(g.d[l]), G(g.d[l]), G(g.b[l]), nullptr);
+        if (!rc) rc = conv_bwd_cl(n, ci--, A(g.u[l]), n->ch[l + 1], A(g.e[l]), n->ch[l], h, w, A(g.b[l]), G(g.b[l]), G(g.u[l]), G(g.e[l]));
+        const int below = l == 3 ? g.e[4] : g.d[l + 1];
+        if (!rc) {
+            k_up2_back<true><<<nblk((long long)n->ch[l + 1] * (h / 2) * (w / 2)), 256, 0, n->stream>>>(G(g.u[l]), n->ch[l + 1], h / 2, w / 2, G(below));
+            rc = n->cuda(cudaGetLastError(), "upsample backward");
+        }
+    }
+    for (int l = 4; l >= 0 && !rc; --l) {
+        const int h = H >> l, w = W >> l;
+        rc = conv_bwd_cl(n, ci--, A(g.a[l]), n->ch[l], nullptr, 0, h, w, A(g.e[l]), G(g.e[l]), G(g.a[l]), nullptr);
+        if (!rc) rc = conv_bwd_cl(n, ci--, l ? A(g.p[l]) : A(g.input), l ? n->ch[l - 1] : 7, nullptr, 0, h, w, A(g.a[l]), G(g.a[l]),
+                                  l ? G(g.p[l]) : nullptr, nullptr);
+        if (!rc && l) {
+            k_pool2_back<<<nblk(n->act_size[g.e[l - 1]]), 256, 0, n->stream>>>(G(g.p[l]), n->ch[l - 1], h * 2, w * 2, G(g.e[l - 1]));
+            rc = n->cuda(cudaGetLastError(), "pool backward");
+        }
+    }
+    return rc;
+}
+
 int backward(lbm_net* n, int H, int W, const float* gout) {
     Graph g = make_graph(n->ch);
     auto A = [&](int t) { return n->act[t]; };
     auto G = [&](int t) { return n->gact[t]; };
     int rc = LBM_OK;
+    if (n->backend == 3) return backward_cl(n, g, H, W, gout);
     for (size_t t = 0; t < n->gact.size() && !rc; ++t)
         rc = n->cuda(cudaMemsetAsync(n->gact[t], 0, n->act_size[t] * 4, n->stream), "gradient reset");
     if (!rc) rc = n->cuda(cudaMemcpyAsync(G(g.out), gout, n->act_size[g.out] * 4, cudaMemcpyDeviceToDevice, n->stream), "gradient copy");
@@ -659,7 +866,7 @@ int backward(lbm_net* n, int H, int W, const float* gout) {
         if (!rc) rc = conv_bwd(n, n->convs[ci--], A(g.u[l]), n->ch[l + 1], A(g.e[l]), n->ch[l], h, w, A(g.b[l]), G(g.b[l]), G(g.u[l]), G(g.e[l]));
         const int below = l == 3 ? g.e[4] : g.d[l + 1];
         if (!rc) {
-            k_up2_back<<<nblk((long long)n->ch[l + 1] * (h / 2) * (w / 2)), 256, 0, n->stream>>>(G(g.u[l]), n->ch[l + 1], h / 2, w / 2, G(below));
+            k_up2_back<false><<<nblk((long long)n->ch[l + 1] * (h / 2) * (w / 2)), 256, 0, n->stream>>>(G(g.u[l]), n->ch[l + 1], h / 2, w / 2, G(below));
             rc = n->cuda(cudaGetLastError(), "upsample backward");
         }
     }
@@ -712,6 +919,15 @@ extern "C" int lbm_net_create(int width, unsigned long long seed, lbm_net** out)
         f += (long long)c.ci * c.Kp2;
         n->convs.push_back(c);
     }
+    long long taps = 0;
+    for (auto& c : n->convs) {
+        ConvDev t{c.ci, c.co, c.Kp, c.Kp2, conv_cp(c.ci), conv_cp(c.co), c.woff, c.wq_off, c.wf_off, 0, 0};
+        t.wt = taps;
+        taps += 9ll * c.co * t.cpi;
+        t.wb = taps;
+        taps += 9ll * c.ci * t.cpo;
+        n->devs.push_back(t);
+    }
     n->nparams = off;
     n->nwq = q;
     n->nwf = f;
@@ -722,6 +938,8 @@ extern "C" int lbm_net_create(int width, unsigned long long seed, lbm_net** out)
     };
     if (cudaMalloc(&n->params, off * 4) != cudaSuccess || cudaMalloc(&n->grads, off * 4) != cudaSuccess ||
         cudaMalloc(&n->adam_m, off * 4) != cudaSuccess || cudaMalloc(&n->adam_v, off * 4) != cudaSuccess ||
+        cudaMalloc(&n->taps, taps * 2) != cudaSuccess ||
+        cudaMalloc(&n->d_convs, n->devs.size() * sizeof(ConvDev)) != cudaSuccess ||
         cudaMalloc(&n->wq, q * 2) != cudaSuccess || cudaMalloc(&n->wf, f * 2) != cudaSuccess ||
         cudaMalloc(&n->parts, 1024 * sizeof(double)) != cudaSuccess || cudaMalloc(&n->d_loss, 3 * sizeof(double)) != cudaSuccess ||
         cudaMalloc(&n->d_err, sizeof(int)) != cudaSuccess ||
@@ -738,6 +956,7 @@ extern "C" int lbm_net_create(int width, unsigned long long seed, lbm_net** out)
         for (long long k = 0; k < (long long)c.ci * c.co * 9; ++k) h[c.woff + k] = U(rng);
     }
     if (cudaMemcpy(n->params, h.data(), off * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(n->d_convs, n->devs.data(), n->devs.size() * sizeof(ConvDev), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemset(n->grads, 0, off * 4) != cudaSuccess || cudaMemset(n->adam_m, 0, off * 4) != cudaSuccess ||
         cudaMemset(n->adam_v, 0, off * 4) != cudaSuccess || cudaMemset(n->d_err, 0, sizeof(int)) != cudaSuccess) {
         cudaGetLastError();
@@ -753,7 +972,7 @@ extern "C" void lbm_net_destroy(lbm_net* n) {
     for (float* p : n->act) cudaFree(p);
     for (float* p : n->gact) cudaFree(p);
     for (void* p : {(void*)n->params, (void*)n->grads, (void*)n->adam_m, (void*)n->adam_v, (void*)n->wq, (void*)n->wf,
-                    (void*)n->col, (void*)n->wtap, (void*)n->dz, (void*)n->dzq, (void*)n->parts, (void*)n->d_loss,
+                    (void*)n->col, (void*)n->cl[0], (void*)n->cl[1], (void*)n->taps, (void*)n->d_convs, (void*)n->dz, (void*)n->dzq, (void*)n->parts, (void*)n->d_loss,
                     (void*)n->d_err})
         if (p) cudaFree(p);
     if (n->h_loss) cudaFreeHost(n->h_loss);
@@ -839,9 +1058,9 @@ extern "C" int lbm_net_backward(lbm_net* n, const float* in, const float* base, 
     const long long P = (long long)H * W;
     const int nb = 512;
     // loss and dL/d(out) (into the dZ scratch, which backward copies before reusing it)
-    k_mask_stats<<<1, 256, 0, n->stream>>>(mask, n->act[g.out], base, target, P, n->d_loss);
+    k_mask_stats<<<1, 1024, 0, n->stream>>>(mask, n->act[g.out], base, target, P, n->d_loss);
     k_mse<<<nb, 256, 0, n->stream>>>(n->act[g.out], base, target, mask, P, n->d_loss, n->dz, n->parts);
-    k_sum_parts<<<1, 32, 0, n->stream>>>(n->parts, nb, n->d_loss);
+    k_sum_parts<<<1, 256, 0, n->stream>>>(n->parts, nb, n->d_loss);
     rc = n->cuda(cudaGetLastError(), "loss");
     if (!rc) rc = backward(n, H, W, n->dz);
     if (!rc) rc = n->cuda(cudaMemcpyAsync(n->h_loss, n->d_loss + 1, sizeof(double), cudaMemcpyDeviceToHost, n->stream), "loss copy");

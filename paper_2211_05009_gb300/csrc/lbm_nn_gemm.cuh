@@ -17,6 +17,8 @@
 namespace lbm {
 namespace nn {
 
+constexpr float kLeak = 0.1f;  // leaky ReLU slope
+
 enum GemmOp { kStore = 0, kAccumulate = 1, kAtomicAdd = 2 };
 
 cudaError_t gemm_bf16_nt(int M, int N, int K, const __nv_bfloat16* A, int lda,
@@ -50,6 +52,18 @@ cudaError_t weights_tap_major(const __nv_bfloat16* Wt, int ldk, int C, int N, __
 cudaError_t conv3x3_bf16_tma(const float* x1, int c1, const float* x2, int c2, int H, int W, const __nv_bfloat16* Wtap,
                              int N, float* C, int ldc, GemmOp op, bool trans_c, __nv_bfloat16* xs, int* err,
                              cudaStream_t st);
+
+// Whether the convolutions over channels-last inputs take an H x W image.
+bool conv_tma_takes(int H, int W);
+// y[n][p] = conv(xs)[n][p] with xs [H][W][conv_cp(C_in)] BF16 channels-last: plus bias[n] and leaky ReLU
+// if given; output channels from n2 on go to y2 (if given) instead; y_cl (if given) also receives the
+// values as BF16, channels-last [pixel][conv_cp(N)], zero padded.
+cudaError_t conv3x3_channels_last(const __nv_bfloat16* xs, int C_in, int H, int W, const __nv_bfloat16* Wtap, int N, float* y,
+                                  const float* bias, bool act, float* y2, int n2, __nv_bfloat16* y_cl, int* err,
+                                  cudaStream_t st);
+// The same layer as a product with an explicit im2col A [M][K], B [N][K]: y[n][m].
+cudaError_t gemm_bf16_nt_umma_layer(int M, int N, int K, const __nv_bfloat16* A, const __nv_bfloat16* B, float* y, const float* bias,
+                                    bool act, float* y2, int n2, int* err, cudaStream_t st);
 
 }  // namespace nn
 }  // namespace lbm

@@ -33,6 +33,8 @@ namespace {
 constexpr int TM = 128, TK = 64;
 constexpr int kTileA = TM * TK * 2;           // 16 KB
 constexpr int kSmemBudget = 110 * 1024;       // per CTA: two CTAs per SM
+constexpr int kSmemWhole = 210 * 1024;        // per CTA when it has an SM to itself
+constexpr int kFewCtas = 152;                 // CTAs of such a launch: one per SM
 constexpr int kSmemExtra = 1024 + 256;        // 1024-byte alignment slack + barriers / TMEM slot
 constexpr long long kWaitCycles = 2000000000ll;  // ~1 s
 
@@ -53,6 +55,27 @@ Plan plan_for(int N) {
     return p;
 }
 
+// The plan for few row tiles (deep levels of the network: 1 .. 32 tiles, 27 .. 45 K steps).  A CTA's K
+// steps are a chain whose pace is the copies' latency over the stages in flight, so while a wave has
+// SMs to spare the columns are cut into narrower tiles (down to 32) and a CTA takes the shared memory
+// of a whole SM: 160 -> 160 channels at 16 x 16, one of 2 CTAs with 3 stages against 10 with 9.  The
+// sums of an element do not depend on the cut.
+Plan plan_for(int N, long long row_tiles) {
+    Plan p = plan_for(N);
+    if (row_tiles * p.tiles_n * 2 > kFewCtas) return p;
+    const int most = (int)(kFewCtas / row_tiles), wanted = (N + 31) / 32;
+    p.tiles_n = wanted < most ? wanted : most;
+    p.tn = ((N + p.tiles_n - 1) / p.tiles_n + 15) / 16 * 16;
+    p.tiles_n = (N + p.tn - 1) / p.tn;
+    p.cols = 32;
+    while (p.cols < p.tn) p.cols <<= 1;
+    const int stage = kTileA + p.tn * TK * 2;
+    p.stages = (kSmemWhole - kSmemExtra) / stage;
+    if (p.stages > 10) p.stages = 10;
+    p.smem = p.stages * stage + kSmemExtra;
+    return p;
+}
+
 __device__ __forceinline__ uint32_t sa(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
 
 // tcgen05 shared-memory descriptor, K-major operand in the 128-byte swizzle layout: start >> 4,
@@ -66,6 +89,11 @@ __device__ __forceinline__ uint64_t desc_sw128(uint32_t addr) {
     d |= (uint64_t)1 << 46;
     d |= (uint64_t)2 << 61;
     return d;
+}
+
+__device__ __forceinline__ uint32_t bf16x2(float lo, float hi) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t*>(&v);
 }
 
 __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
@@ -107,6 +135,20 @@ struct ConvGeo {
     int W, cb;
 };
 
+// What the epilogue does with C[m][n].  bias, act: leaky ReLU(c + bias[n]) with kStore.  C2: columns
+// from n2 on go there (column n - n2).  cl: the stored value also as BF16, channels-last
+// [pixel][cp], zeros in columns N .. cp - 1 -- the input of a following convolution.
+struct Epilogue {
+    float* C;
+    int ldc, op, trans_c;
+    const float* bias;
+    int act;
+    float* C2;
+    int n2;
+    __nv_bfloat16* cl;
+    int cp;
+};
+
 // CONV = false: the GEMM above.  CONV = true: A is a 3x3, padding-1 convolution input stored
 // channels-last in BF16 ([H][W][Cp], Cp = cb * 64) and K is ordered tap-major (k = tap * Cp + c,
 // tap = ky * 3 + kx).  The 128 pixels of an M tile are 128 consecutive pixels of one row (W a
@@ -117,8 +159,7 @@ struct ConvGeo {
 template <bool CONV>
 __global__ void __launch_bounds__(128, 1)
     k_gemm_tc05(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int M, int N, int K,
-                float* __restrict__ C, int ldc, int op, int trans_c, int k_per_split, int tn, int cols, int stages,
-                int* err, ConvGeo geo) {
+                const Epilogue ep, int k_per_split, int tn, int cols, int stages, int* err, ConvGeo geo) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* base = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const int stage_bytes = kTileA + tn * TK * 2;
@@ -211,31 +252,66 @@ __global__ void __launch_bounds__(128, 1)
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::);
     if (ok && !abort_flag && nk > 0) {
         const int row = m0 + warp * 32 + lane;
+        // a convolution's last column tile also writes the channels-last padding
+        const int cend = CONV && ep.cl && n0 + tn >= N ? ep.cp - n0 : tn;
 #pragma unroll 1
-        for (int c0 = 0; c0 < tn; c0 += 16) {
-            uint32_t v[16];
-            const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0;
-            asm volatile(
-                "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
-                "%14, %15}, [%16];\n"
-                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                  "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-                : "r"(taddr));
-            asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::);
-            if (row < M) {
+        for (int c0 = 0; c0 < cend; c0 += 16) {
+            float f[16];
+            if (c0 < tn) {
+                uint32_t v[16];
+                const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0;
+                asm volatile(
+                    "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
+                    "%14, %15}, [%16];\n"
+                    : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+                      "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+                    : "r"(taddr));
+                asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::);
+#pragma unroll
+                for (int j = 0; j < 16; ++j) f[j] = __uint_as_float(v[j]);
+            } else {
+#pragma unroll
+                for (int j = 0; j < 16; ++j) f[j] = 0.f;
+            }
+            if (row >= M) continue;
+            const int n = n0 + c0;
+            auto at = [&](int j) {
+                float* c = ep.C;
+                int m = n + j;
+                if (ep.C2 && m >= ep.n2) {
+                    c = ep.C2;
+                    m -= ep.n2;
+                }
+                return ep.trans_c ? c + (long long)m * ep.ldc + row : c + (long long)row * ep.ldc + m;
+            };
+            if (ep.op == kAtomicAdd) {
+#pragma unroll
+                for (int j = 0; j < 16; ++j)
+                    if (n + j < N) atomicAdd(at(j), f[j]);
+                continue;
+            }
+            if (ep.op == kAccumulate) {  // all 16 old values in flight before the first store
+                float old[16];
+#pragma unroll
+                for (int j = 0; j < 16; ++j) old[j] = n + j < N ? *at(j) : 0.f;
+#pragma unroll
+                for (int j = 0; j < 16; ++j) f[j] += old[j];
+            }
+            if (ep.bias) {
 #pragma unroll
                 for (int j = 0; j < 16; ++j) {
-                    const int n = n0 + c0 + j;
-                    if (n < N) {
-                        float* c = trans_c ? C + (long long)n * ldc + row : C + (long long)row * ldc + n;
-                        const float f = __uint_as_float(v[j]);
-                        if (op == kAtomicAdd)
-                            atomicAdd(c, f);
-                        else if (op == kAccumulate)
-                            *c += f;
-                        else
-                            *c = f;
-                    }
+                    f[j] = n + j < N ? f[j] + __ldg(ep.bias + n + j) : 0.f;
+                    if (ep.act && f[j] < 0.f) f[j] *= kLeak;
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+                if (n + j < N) *at(j) = f[j];
+            if constexpr (CONV) {
+                if (ep.cl) {
+                    uint4* q = reinterpret_cast<uint4*>(ep.cl + (long long)row * ep.cp + n);
+                    q[0] = make_uint4(bf16x2(f[0], f[1]), bf16x2(f[2], f[3]), bf16x2(f[4], f[5]), bf16x2(f[6], f[7]));
+                    q[1] = make_uint4(bf16x2(f[8], f[9]), bf16x2(f[10], f[11]), bf16x2(f[12], f[13]), bf16x2(f[14], f[15]));
                 }
             }
         }
@@ -266,11 +342,6 @@ struct ConvIn {
 };
 
 constexpr int kWinCh = 8;  // channels a 64-wide K range can touch (ceil(64 / 9) + 1)
-
-__device__ __forceinline__ uint32_t bf16x2(float lo, float hi) {
-    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-    return *reinterpret_cast<const uint32_t*>(&v);
-}
 
 // Window geometry of the tile starting at pixel m0: rows wy0 .. wy0+R-1, columns wx0 .. wx0+WC-1.
 __host__ __device__ inline void conv_window(int m0, int M, int W, int TMr, int& wy0, int& R, int& wx0, int& WC) {
@@ -463,6 +534,12 @@ __global__ void __launch_bounds__(kConvThreads, 2)
                 : "r"(taddr));
             asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::);
             if (row < M) {
+                float old[16];
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    const int n = n0 + c0 + j;
+                    old[j] = op == kAccumulate && n < N ? (trans_c ? C[(long long)n * ldc + row] : C[(long long)row * ldc + n]) : 0.f;
+                }
 #pragma unroll
                 for (int j = 0; j < 16; ++j) {
                     const int n = n0 + c0 + j;
@@ -472,7 +549,7 @@ __global__ void __launch_bounds__(kConvThreads, 2)
                         if (op == kAtomicAdd)
                             atomicAdd(c, f);
                         else if (op == kAccumulate)
-                            *c += f;
+                            *c = old[j] + f;
                         else
                             *c = f;
                     }
@@ -560,40 +637,71 @@ __global__ void k_weights_tap_major(const __nv_bfloat16* __restrict__ Wt, int ld
     Wtap[i] = c < C ? Wt[(long long)n * ldk + c * 9 + tap] : __float2bfloat16_rn(0.f);
 }
 
+// Opt in to a plan's dynamic shared memory: the attribute belongs to the current device, so the
+// largest size set so far is kept per device (thread-safe).
+template <bool CONV>
+cudaError_t opt_in(int smem) {
+    static std::mutex mu;
+    static int opted[64] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lock(mu);
+    if (dev >= 64 || smem > opted[dev]) {
+        e = cudaFuncSetAttribute(k_gemm_tc05<CONV>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        if (dev < 64) opted[dev] = smem;
+    }
+    return cudaSuccess;
+}
+
+// The convolution GEMM over a channels-last input xs [H][W][Cp].
+cudaError_t conv_gemm(const __nv_bfloat16* xs, int Cp, int H, int W, const __nv_bfloat16* Wtap, int N, const Epilogue& ep,
+                      int* err, cudaStream_t st) {
+    const int bw = W < TM ? W : TM;
+    const long long tiles = (long long)H * W / TM;
+    const int K = 9 * Cp;
+    const Plan p = plan_for(N, tiles);
+    CUtensorMap ma, mb;
+    if (!make_act_map(&ma, xs, H, W, Cp, bw, TM / bw) || !make_map(&mb, Wtap, N, K, K, p.tn)) return cudaErrorInvalidValue;
+    const cudaError_t e = opt_in<true>(p.smem);
+    if (e != cudaSuccess) return e;
+    k_gemm_tc05<true><<<dim3(p.tiles_n, (unsigned)tiles, 1), 128, p.smem, st>>>(ma, mb, H * W, N, K, ep, K, p.tn, p.cols, p.stages,
+                                                                               err, ConvGeo{W, Cp / TK});
+    return cudaGetLastError();
+}
+
 }  // namespace
 
-cudaError_t gemm_bf16_nt_umma(int M, int N, int K, const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb,
-                              float* C, int ldc, GemmOp op, bool trans_c, int split_k, int* err, cudaStream_t st) {
+static cudaError_t gemm_ep(int M, int N, int K, const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb,
+                           const Epilogue& ep, int split_k, int* err, cudaStream_t st) {
     if (M <= 0 || N <= 0) return cudaSuccess;
     if ((K & 7) || (lda & 7) || (ldb & 7) || K <= 0 || !err) return cudaErrorInvalidValue;
     if (((uintptr_t)A & 15) || ((uintptr_t)B & 15)) return cudaErrorInvalidValue;  // TMA: 16-byte aligned bases
     if (split_k < 1) split_k = 1;
-    if (split_k > 1 && op != kAtomicAdd) return cudaErrorInvalidValue;
-    const Plan p = plan_for(N);
-    CUtensorMap ma, mb;
-    if (!make_map(&ma, A, M, K, lda, TM) || !make_map(&mb, B, N, K, ldb, p.tn)) return cudaErrorInvalidValue;
-    {
-        // opt in to the plan's dynamic shared memory: the attribute belongs to the current device,
-        // so the largest size set so far is kept per device (thread-safe)
-        static std::mutex mu;
-        static int opted[64] = {};
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e != cudaSuccess) return e;
-        std::lock_guard<std::mutex> lock(mu);
-        if (dev >= 64 || p.smem > opted[dev]) {
-            e = cudaFuncSetAttribute(k_gemm_tc05<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
-            if (e != cudaSuccess) return e;
-            if (dev < 64) opted[dev] = p.smem;
-        }
-    }
+    if (split_k > 1 && ep.op != kAtomicAdd) return cudaErrorInvalidValue;
     int kps = (K + split_k - 1) / split_k;
     kps = (kps + TK - 1) / TK * TK;
     split_k = (K + kps - 1) / kps;
+    const Plan p = plan_for(N, (long long)((M + TM - 1) / TM) * split_k);
+    CUtensorMap ma, mb;
+    if (!make_map(&ma, A, M, K, lda, TM) || !make_map(&mb, B, N, K, ldb, p.tn)) return cudaErrorInvalidValue;
+    const cudaError_t e = opt_in<false>(p.smem);
+    if (e != cudaSuccess) return e;
     const dim3 grid(p.tiles_n, (M + TM - 1) / TM, split_k);
-    k_gemm_tc05<false><<<grid, 128, p.smem, st>>>(ma, mb, M, N, K, C, ldc, (int)op, trans_c ? 1 : 0, kps, p.tn, p.cols,
-                                                   p.stages, err, ConvGeo{0, 0});
+    k_gemm_tc05<false><<<grid, 128, p.smem, st>>>(ma, mb, M, N, K, ep, kps, p.tn, p.cols, p.stages, err, ConvGeo{});
     return cudaGetLastError();
+}
+
+cudaError_t gemm_bf16_nt_umma(int M, int N, int K, const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb,
+                              float* C, int ldc, GemmOp op, bool trans_c, int split_k, int* err, cudaStream_t st) {
+    return gemm_ep(M, N, K, A, lda, B, ldb, Epilogue{C, ldc, (int)op, trans_c ? 1 : 0, nullptr, 0, nullptr, 0, nullptr, 0}, split_k,
+                   err, st);
+}
+
+cudaError_t gemm_bf16_nt_umma_layer(int M, int N, int K, const __nv_bfloat16* A, const __nv_bfloat16* B, float* y, const float* bias,
+                                    bool act, float* y2, int n2, int* err, cudaStream_t st) {
+    return gemm_ep(M, N, K, A, K, B, K, Epilogue{y, M, kStore, 1, bias, act ? 1 : 0, y2, n2, nullptr, 0}, 1, err, st);
 }
 
 cudaError_t conv3x3_bf16_umma(const float* x1, int c1, const float* x2, int c2, int H, int W, int K,
@@ -649,6 +757,11 @@ namespace nn {
 
 int conv_cp(int c) { return (c + TK - 1) / TK * TK; }
 
+// Tiles of 128 pixels: part of one row, or whole rows; the box's dimensions stay <= 256.
+bool conv_tma_takes(int H, int W) {
+    return H > 0 && W > 0 && (long long)H * W % TM == 0 && (W % TM == 0 || TM % W == 0) && H <= 0x7fffffff / W;
+}
+
 cudaError_t weights_tap_major(const __nv_bfloat16* Wt, int ldk, int C, int N, __nv_bfloat16* Wtap, cudaStream_t st) {
     if (N <= 0 || C <= 0) return cudaSuccess;
     if (!Wt || !Wtap || ldk < 9 * C) return cudaErrorInvalidValue;
@@ -663,34 +776,22 @@ cudaError_t conv3x3_bf16_tma(const float* x1, int c1, const float* x2, int c2, i
     const long long P = (long long)H * W;
     if (P <= 0 || N <= 0) return cudaSuccess;
     if (!x1 || c1 < 1 || c2 < 0 || (c2 > 0 && !x2) || !Wtap || !xs || !err) return cudaErrorInvalidValue;
-    // tiles of 128 pixels: part of one row, or whole rows; the box's dimensions stay <= 256
-    if (P % TM || !(W % TM == 0 || TM % W == 0) || H > 0x7fffffff / W) return cudaErrorInvalidValue;
+    if (!conv_tma_takes(H, W)) return cudaErrorInvalidValue;
     if (((uintptr_t)Wtap & 15) || ((uintptr_t)xs & 15)) return cudaErrorInvalidValue;
-    const int Cp = conv_cp(c1 + c2), K = 9 * Cp;
-    const Plan p = plan_for(N);
-    CUtensorMap ma, mb;
-    const int bw = W < TM ? W : TM;
-    if (!make_act_map(&ma, xs, H, W, Cp, bw, TM / bw) || !make_map(&mb, Wtap, N, K, K, p.tn)) return cudaErrorInvalidValue;
-    {
-        static std::mutex mu;
-        static int opted[64] = {};
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e != cudaSuccess) return e;
-        std::lock_guard<std::mutex> lock(mu);
-        if (dev >= 64 || p.smem > opted[dev]) {
-            e = cudaFuncSetAttribute(k_gemm_tc05<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
-            if (e != cudaSuccess) return e;
-            if (dev < 64) opted[dev] = p.smem;
-        }
-    }
+    const int Cp = conv_cp(c1 + c2);
     k_channels_last_bf16<<<dim3((unsigned)((P + 255) / 256), (unsigned)(Cp / 8)), 256, 0, st>>>(x1, c1, x2, c2, P, Cp, xs);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const dim3 grid(p.tiles_n, (unsigned)(P / TM), 1);
-    k_gemm_tc05<true><<<grid, 128, p.smem, st>>>(ma, mb, (int)P, N, K, C, ldc, (int)op, trans_c ? 1 : 0, K, p.tn, p.cols,
-                                                  p.stages, err, ConvGeo{W, Cp / TK});
-    return cudaGetLastError();
+    return conv_gemm(xs, Cp, H, W, Wtap, N, Epilogue{C, ldc, (int)op, trans_c ? 1 : 0, nullptr, 0, nullptr, 0, nullptr, 0}, err, st);
+}
+
+cudaError_t conv3x3_channels_last(const __nv_bfloat16* xs, int C_in, int H, int W, const __nv_bfloat16* Wtap, int N, float* y,
+                                  const float* bias, bool act, float* y2, int n2, __nv_bfloat16* y_cl, int* err,
+                                  cudaStream_t st) {
+    const long long P = (long long)H * W;
+    if (N < 1 || C_in < 1 || !conv_tma_takes(H, W)) return cudaErrorInvalidValue;
+    return conv_gemm(xs, conv_cp(C_in), H, W, Wtap, N, Epilogue{y, (int)P, kStore, 1, bias, act ? 1 : 0, y2, n2, y_cl, y_cl ? conv_cp(N) : 0},
+                     err, st);
 }
 
 }  // namespace nn
