@@ -12,6 +12,7 @@
 // Operands are rounded to BF16 where they enter the GEMM (weights, im2col columns, dZ); the FP32
 // master weights are updated by Adam.  Activation: leaky ReLU (slope 0.1) after every conv but
 // the output head.  Down: 2x2 average pool; up: nearest x2; skips by channel concatenation.
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -159,17 +160,20 @@ __global__ void __launch_bounds__(256) k_act_back_cl(const float* __restrict__ y
     const int p = blockIdx.x * blockDim.x + threadIdx.x, cg = blockIdx.y * 8;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     __nv_bfloat16 b[8];
+    float gv[8], yv[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {  // all loads in flight before the first use
+        const bool in = cg + j < C && p < P;
+        const long long i = in ? (long long)(cg + j) * P + p : 0;
+        gv[j] = in ? dy[i] : 0.f;
+        yv[j] = in && act ? y[i] : 1.f;
+    }
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-        const int c = cg + j;
-        float g = 0.f;
-        if (c < C && p < P) {
-            const long long i = (long long)c * P + p;
-            g = dy[i];
-            if (act && y[i] <= 0.f) g *= kLeak;
-            dzq[i] = __float2bfloat16_rn(g);
-        }
+        float g = gv[j];
+        if (yv[j] <= 0.f) g *= kLeak;
         b[j] = __float2bfloat16_rn(g);
+        if (cg + j < C && p < P) dzq[(long long)(cg + j) * P + p] = b[j];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
         if (lane == 0) sh[warp][j] = g;
@@ -251,43 +255,58 @@ __global__ void k_up2_back(const float* __restrict__ dy, int C, int h, int w, fl
 }
 
 // Number of valid pixels (mask is 0/1) into cnt[0].
-// stats[0] = sum mask (the count n); stats[2] = sum mask (base + out - target)_0 / n, the mean
-// density-channel error, which the loss ignores (one block, fixed order).
-__global__ void __launch_bounds__(1024) k_mask_stats(const float* __restrict__ mask, const float* __restrict__ out,
-                                                     const float* __restrict__ base, const float* __restrict__ tgt,
-                                                     long long P, double* stats) {
-    __shared__ double sh[2][1024];
+// Partial sums of mask and of mask (base + out - target)_0 per block: the count n and, over n, the
+// mean density-channel error, which the loss ignores.
+constexpr int kStatBlocks = 64;
+__global__ void __launch_bounds__(256) k_mask_stats(const float* __restrict__ mask, const float* __restrict__ out,
+                                                    const float* __restrict__ base, const float* __restrict__ tgt,
+                                                    long long P, double* __restrict__ part) {
+    __shared__ double sh[2][256];
     double s = 0.0, e = 0.0;
-    for (long long i = threadIdx.x; i < P; i += blockDim.x) {
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < P; i += (long long)gridDim.x * blockDim.x) {
         s += mask[i];
         e += (double)(mask[i] * (base[i] + out[i] - tgt[i]));
     }
     sh[0][threadIdx.x] = s;
     sh[1][threadIdx.x] = e;
     __syncthreads();
-    for (int o = 512; o > 0; o >>= 1) {
+    for (int o = 128; o > 0; o >>= 1) {
         if (threadIdx.x < o) {
             sh[0][threadIdx.x] += sh[0][threadIdx.x + o];
             sh[1][threadIdx.x] += sh[1][threadIdx.x + o];
         }
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        stats[0] = sh[0][0];
-        stats[2] = sh[0][0] > 0.0 ? sh[1][0] / sh[0][0] : 0.0;
-    }
+    if (threadIdx.x < 2) part[2 * blockIdx.x + threadIdx.x] = sh[threadIdx.x][0];
 }
 
 // loss = sum mask (e - [c = 0] mean_0)^2 / (3 n), e = base + out - target per channel c: the
 // density channel is compared up to a constant (the level of a steady density field only records
 // how long the wall scheme's mass loss acted; a uniform offset does not change the flow).
-// dout = d loss / d out (the mean's own derivative cancels).  Partial sums per block.
-__global__ void k_mse(const float* __restrict__ out, const float* __restrict__ base, const float* __restrict__ tgt,
-                      const float* __restrict__ mask, long long P, const double* __restrict__ stats,
-                      float* __restrict__ dout, double* __restrict__ part) {
+// dout = d loss / d out (the mean's own derivative cancels).  Partial sums per block; every block
+// forms the count and the mean from k_mask_stats' partials in the same order.
+__global__ void __launch_bounds__(256) k_mse(const float* __restrict__ out, const float* __restrict__ base,
+                                             const float* __restrict__ tgt, const float* __restrict__ mask, long long P,
+                                             const double* __restrict__ stat_part, double* __restrict__ stats,
+                                             float* __restrict__ dout, double* __restrict__ part) {
     __shared__ double sh[256];
-    const float inv_n = (float)(1.0 / (3.0 * stats[0]));
-    const float mean0 = (float)stats[2];
+    __shared__ double st[2];
+    if (threadIdx.x < 64) {
+        static_assert(kStatBlocks == 64, "two warps sum the partials");
+        const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        double v = stat_part[2 * lane + q] + stat_part[2 * (lane + 32) + q];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) st[q] = v;
+    }
+    __syncthreads();
+    const double cnt = st[0], mean = cnt > 0.0 ? st[1] / cnt : 0.0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        stats[0] = cnt;
+        stats[2] = mean;
+    }
+    const float inv_n = (float)(1.0 / (3.0 * cnt));
+    const float mean0 = (float)mean;
     double s = 0.0;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < 3 * P; i += (long long)gridDim.x * blockDim.x) {
         const float m = mask[i % P];
@@ -435,6 +454,13 @@ struct ConvSpec {
     long long wq_off, wf_off;  // offsets into the BF16 weight arrays
 };
 
+struct NetGraph {
+    int H, W;
+    bool seen[2];
+    cudaGraphExec_t exec[2];
+};
+constexpr size_t kMaxNetGraphs = 16;
+
 struct lbm_net {
     int width = 0;
     int ch[5];
@@ -444,12 +470,17 @@ struct lbm_net {
     __nv_bfloat16 *wq = nullptr, *wf = nullptr;
     long long adam_t = 0;
     bool weights_dirty = true;
-    // activations and gradients for one sample size
+    // activations and gradients for one sample size, laid out in the arena
     int H = 0, W = 0;
+    void* arena = nullptr;
+    size_t arena_bytes = 0;
+    // captured launches of the default back end per sample size (exec[0] forward, exec[1] backward),
+    // most recently used first
+    std::vector<NetGraph> graphs;
+    cudaStream_t cap_stream = nullptr;
     std::vector<float*> act, gact;  // per tensor
     std::vector<long long> act_size;
     __nv_bfloat16* col = nullptr;  // im2col scratch (backend 3: the channels-last BF16 input)
-    long long col_elems = 0;
     // backend 3: two channels-last inputs (a convolution reads one and writes the next one's), and the
     // weights of every convolution tap-major, laid out once per change of the parameters
     __nv_bfloat16* cl[2] = {nullptr, nullptr};
@@ -531,57 +562,63 @@ void conv_list(const int* ch, std::vector<std::pair<int, int>>& io) {
     io.push_back({ch[0], 3});
 }
 
+void drop_graphs(lbm_net* n) {
+    for (auto& g : n->graphs)
+        for (auto& e : g.exec)
+            if (e) cudaGraphExecDestroy(e);
+    n->graphs.clear();
+}
+
+// Lays the tensors of an H x W sample out in the arena, which is one allocation that only grows: a
+// mini-batch of uneven heights otherwise freed and allocated some 80 buffers per sample (half of the
+// time of a training step).
 int ensure_buffers(lbm_net* n, int H, int W) {
     if (n->H == H && n->W == W) return LBM_OK;
-    cudaStreamSynchronize(n->stream);
-    for (float* p : n->act) cudaFree(p);
-    for (float* p : n->gact) cudaFree(p);
-    n->act.clear();
-    n->gact.clear();
-    n->act_size.clear();
-    cudaFree(n->col);
-    for (auto& p : n->cl) {
-        cudaFree(p);
-        p = nullptr;
-    }
-    cudaFree(n->dz);
-    cudaFree(n->dzq);
-    n->col = nullptr;
-    n->dz = nullptr;
-    n->dzq = nullptr;
     Graph g = make_graph(n->ch);
-    long long maxt = 0;
-    for (auto& ts : g.t) {
-        const long long sz = (long long)ts.c * (H >> ts.level) * (W >> ts.level);
-        float *a = nullptr, *ga = nullptr;
-        if (cudaMalloc(&a, sz * 4) != cudaSuccess || cudaMalloc(&ga, sz * 4) != cudaSuccess) {
-            cudaGetLastError();
-            return n->fail(LBM_ENOMEM, "network activation buffers");
-        }
-        n->act.push_back(a);
-        n->gact.push_back(ga);
-        n->act_size.push_back(sz);
-        maxt = std::max(maxt, sz);
+    // im2col scratch and channels-last inputs: the largest over the convolutions
+    long long maxt = 0, col = 0, cl = 0;
+    for (auto& ts : g.t) maxt = std::max(maxt, (long long)ts.c * (H >> ts.level) * (W >> ts.level));
+    const int lv[19] = {0, 0, 1, 1, 2, 2, 3, 3, 4, 4, 3, 3, 2, 2, 1, 1, 0, 0, 0};
+    for (int i = 0; i < 19; ++i) {
+        const ConvSpec& c = n->convs[i];
+        const long long P = (long long)(H >> lv[i]) * (W >> lv[i]);
+        col = std::max(col, P * (long long)std::max(c.Kp, c.Kp2));
+        cl = std::max(cl, P * (long long)std::max(conv_cp(c.ci), conv_cp(c.co)));
     }
-    // im2col scratch: largest (pixels at the conv's level) x (Kp or Kp2); bound generously
-    long long need = 0, cl = 0;
-    {
-        std::vector<std::pair<int, int>> io;
-        conv_list(n->ch, io);
-        const int lv[19] = {0, 0, 1, 1, 2, 2, 3, 3, 4, 4, 3, 3, 2, 2, 1, 1, 0, 0, 0};
-        for (int i = 0; i < 19; ++i) {
-            const ConvSpec& c = n->convs[i];
-            const long long P = (long long)(H >> lv[i]) * (W >> lv[i]);
-            need = std::max(need, P * (long long)std::max(c.Kp, c.Kp2));
-            cl = std::max(cl, P * (long long)std::max(conv_cp(c.ci), conv_cp(c.co)));
+    for (int pass = 0; pass < 2; ++pass) {  // measure, then place
+        size_t off = 0;
+        auto take = [&](long long bytes) {
+            void* p = pass ? (char*)n->arena + off : nullptr;
+            off += ((size_t)bytes + 255) / 256 * 256;
+            return p;
+        };
+        n->act.clear();
+        n->gact.clear();
+        n->act_size.clear();
+        for (auto& ts : g.t) {
+            const long long sz = (long long)ts.c * (H >> ts.level) * (W >> ts.level);
+            n->act.push_back((float*)take(sz * 4));
+            n->gact.push_back((float*)take(sz * 4));
+            n->act_size.push_back(sz);
         }
-    }
-    n->col_elems = need;
-    if (cudaMalloc(&n->col, need * 2) != cudaSuccess || cudaMalloc(&n->cl[0], cl * 2) != cudaSuccess ||
-        cudaMalloc(&n->cl[1], cl * 2) != cudaSuccess ||
-        cudaMalloc(&n->dz, maxt * 4) != cudaSuccess || cudaMalloc(&n->dzq, maxt * 2) != cudaSuccess) {
-        cudaGetLastError();
-        return n->fail(LBM_ENOMEM, "network scratch buffers");
+        n->col = (__nv_bfloat16*)take(col * 2);
+        for (auto& p : n->cl) p = (__nv_bfloat16*)take(cl * 2);
+        n->dz = (float*)take(maxt * 4);
+        n->dzq = (__nv_bfloat16*)take(maxt * 2);
+        if (pass == 0 && off > n->arena_bytes) {
+            cudaStreamSynchronize(n->stream);
+            drop_graphs(n);
+            cudaFree(n->arena);
+            n->arena = nullptr;
+            n->arena_bytes = 0;
+            n->H = n->W = 0;
+            if (cudaMalloc(&n->arena, off) != cudaSuccess) {
+                cudaGetLastError();
+                n->arena = nullptr;
+                return n->fail(LBM_ENOMEM, "network activation buffers");
+            }
+            n->arena_bytes = off;
+        }
     }
     n->H = H;
     n->W = W;
@@ -784,6 +821,58 @@ int forward_cl(lbm_net* n, const Graph& g, int H, int W) {
                                 : conv_im2col(n, ci, A(g.d[0]), n->ch[0], nullptr, 0, H, W, A(g.out));
 }
 
+// Run `body` (the default back end's launches of one sample size: part 0 forward, 1 backward), which
+// uses the net's own buffers only.  The first call of a size launches directly, the second captures a
+// graph, later ones replay it: ~30 and ~95 launches of a few microseconds each are otherwise paced by
+// the host.  A capture the driver refuses falls back to direct launches.
+template <typename Body>
+int run_captured(lbm_net* n, int part, Body body) {
+    auto& gs = n->graphs;
+    size_t k = 0;
+    while (k < gs.size() && (gs[k].H != n->H || gs[k].W != n->W)) ++k;
+    if (k == gs.size()) {
+        if (gs.size() == kMaxNetGraphs) {
+            cudaStreamSynchronize(n->stream);
+            for (auto& e : gs.back().exec)
+                if (e) cudaGraphExecDestroy(e);
+            gs.pop_back();
+        }
+        gs.insert(gs.begin(), NetGraph{n->H, n->W, {false, false}, {nullptr, nullptr}});
+    } else if (k) {
+        std::rotate(gs.begin(), gs.begin() + k, gs.begin() + k + 1);
+    }
+    NetGraph& g = gs.front();
+    if (!g.seen[part]) {
+        g.seen[part] = true;
+        return body();
+    }
+    if (!g.exec[part]) {
+        if (!n->cap_stream && cudaStreamCreateWithFlags(&n->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
+            cudaGetLastError();
+            n->cap_stream = nullptr;
+            return body();
+        }
+        const cudaStream_t st = n->stream;
+        cudaGraph_t graph = nullptr;
+        cudaError_t e = cudaStreamBeginCapture(n->cap_stream, cudaStreamCaptureModeThreadLocal);
+        if (e == cudaSuccess) {
+            n->stream = n->cap_stream;
+            const int rc = body();
+            n->stream = st;
+            e = cudaStreamEndCapture(n->cap_stream, &graph);
+            if (e == cudaSuccess && rc) e = cudaErrorUnknown;
+        }
+        if (e == cudaSuccess) e = cudaGraphInstantiate(&g.exec[part], graph, 0);
+        if (graph) cudaGraphDestroy(graph);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            g.exec[part] = nullptr;
+            return body();
+        }
+    }
+    return n->cuda(cudaGraphLaunch(g.exec[part], n->stream), "network graph launch");
+}
+
 int forward(lbm_net* n, const float* in, int H, int W) {
     int rc = ensure_buffers(n, H, W);
     if (!rc) rc = prep_weights(n);
@@ -792,7 +881,7 @@ int forward(lbm_net* n, const float* in, int H, int W) {
     auto A = [&](int t) { return n->act[t]; };
     if (n->backend == 3) {
         rc = n->cuda(cudaMemcpyAsync(A(g.input), in, n->act_size[g.input] * 4, cudaMemcpyDeviceToDevice, n->stream), "input copy");
-        return rc ? rc : forward_cl(n, g, H, W);
+        return rc ? rc : run_captured(n, 0, [&] { return forward_cl(n, g, H, W); });
     }
     rc = n->cuda(cudaMemcpyAsync(A(g.input), in, n->act_size[g.input] * 4, cudaMemcpyDeviceToDevice, n->stream), "input copy");
     int ci = 0;  // conv index
@@ -854,7 +943,7 @@ int backward(lbm_net* n, int H, int W, const float* gout) {
     auto A = [&](int t) { return n->act[t]; };
     auto G = [&](int t) { return n->gact[t]; };
     int rc = LBM_OK;
-    if (n->backend == 3) return backward_cl(n, g, H, W, gout);
+    if (n->backend == 3) return run_captured(n, 1, [&] { return backward_cl(n, g, H, W, gout); });
     for (size_t t = 0; t < n->gact.size() && !rc; ++t)
         rc = n->cuda(cudaMemsetAsync(n->gact[t], 0, n->act_size[t] * 4, n->stream), "gradient reset");
     if (!rc) rc = n->cuda(cudaMemcpyAsync(G(g.out), gout, n->act_size[g.out] * 4, cudaMemcpyDeviceToDevice, n->stream), "gradient copy");
@@ -943,7 +1032,7 @@ extern "C" int lbm_net_create(int width, unsigned long long seed, lbm_net** out)
         cudaMalloc(&n->wq, q * 2) != cudaSuccess || cudaMalloc(&n->wf, f * 2) != cudaSuccess ||
         cudaMalloc(&n->parts, 1024 * sizeof(double)) != cudaSuccess || cudaMalloc(&n->d_loss, 3 * sizeof(double)) != cudaSuccess ||
         cudaMalloc(&n->d_err, sizeof(int)) != cudaSuccess ||
-        cudaMallocHost(&n->h_loss, sizeof(double)) != cudaSuccess) {
+        cudaMallocHost(&n->h_loss, 2 * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
         return fail("network parameter allocation");
     }
@@ -969,11 +1058,10 @@ extern "C" int lbm_net_create(int width, unsigned long long seed, lbm_net** out)
 extern "C" void lbm_net_destroy(lbm_net* n) {
     if (!n) return;
     cudaStreamSynchronize(n->stream);
-    for (float* p : n->act) cudaFree(p);
-    for (float* p : n->gact) cudaFree(p);
-    for (void* p : {(void*)n->params, (void*)n->grads, (void*)n->adam_m, (void*)n->adam_v, (void*)n->wq, (void*)n->wf,
-                    (void*)n->col, (void*)n->cl[0], (void*)n->cl[1], (void*)n->taps, (void*)n->d_convs, (void*)n->dz, (void*)n->dzq, (void*)n->parts, (void*)n->d_loss,
-                    (void*)n->d_err})
+    drop_graphs(n);
+    if (n->cap_stream) cudaStreamDestroy(n->cap_stream);
+    for (void* p : {(void*)n->params, (void*)n->grads, (void*)n->adam_m, (void*)n->adam_v, (void*)n->wq, (void*)n->wf, (void*)n->taps,
+                    (void*)n->d_convs, n->arena, (void*)n->parts, (void*)n->d_loss, (void*)n->d_err})
         if (p) cudaFree(p);
     if (n->h_loss) cudaFreeHost(n->h_loss);
     delete n;
@@ -1007,11 +1095,12 @@ extern "C" int lbm_net_zero_grads(lbm_net* n) {
     return n->cuda(cudaMemsetAsync(n->grads, 0, n->nparams * 4, n->stream), "gradient reset");
 }
 
-// A tcgen05 GEMM that gave up waiting leaves 1 in d_err (result incomplete).
-static int check_err(lbm_net* n) {
-    int h = 0;
-    int rc = n->cuda(cudaMemcpy(&h, n->d_err, sizeof(int), cudaMemcpyDeviceToHost), "error word copy");
-    if (!rc && h) {
+// Wait for the queued work.  A tcgen05 GEMM that gave up waiting leaves 1 in d_err (result incomplete).
+static int finish(lbm_net* n) {
+    int* h = reinterpret_cast<int*>(n->h_loss + 1);
+    int rc = n->cuda(cudaMemcpyAsync(h, n->d_err, sizeof(int), cudaMemcpyDeviceToHost, n->stream), "error word copy");
+    if (!rc) rc = n->cuda(cudaStreamSynchronize(n->stream), "stream synchronize");
+    if (!rc && *h) {
         cudaMemset(n->d_err, 0, sizeof(int));
         return n->fail(LBM_ETIMEOUT, "a tensor-core GEMM wait ran out");
     }
@@ -1040,10 +1129,7 @@ extern "C" int lbm_net_forward(lbm_net* n, const float* in, int H, int W, float*
         Graph g = make_graph(n->ch);
         rc = n->cuda(cudaMemcpyAsync(out, n->act[g.out], n->act_size[g.out] * 4, cudaMemcpyDeviceToDevice, n->stream), "output copy");
     }
-    if (!rc && n->backend != 0) {
-        rc = n->cuda(cudaStreamSynchronize(n->stream), "stream synchronize");
-        if (!rc) rc = check_err(n);
-    }
+    if (!rc && n->backend != 0) rc = finish(n);
     return rc;
 }
 
@@ -1058,14 +1144,14 @@ extern "C" int lbm_net_backward(lbm_net* n, const float* in, const float* base, 
     const long long P = (long long)H * W;
     const int nb = 512;
     // loss and dL/d(out) (into the dZ scratch, which backward copies before reusing it)
-    k_mask_stats<<<1, 1024, 0, n->stream>>>(mask, n->act[g.out], base, target, P, n->d_loss);
-    k_mse<<<nb, 256, 0, n->stream>>>(n->act[g.out], base, target, mask, P, n->d_loss, n->dz, n->parts);
+    double* stat_part = n->parts + nb;
+    k_mask_stats<<<kStatBlocks, 256, 0, n->stream>>>(mask, n->act[g.out], base, target, P, stat_part);
+    k_mse<<<nb, 256, 0, n->stream>>>(n->act[g.out], base, target, mask, P, stat_part, n->d_loss, n->dz, n->parts);
     k_sum_parts<<<1, 256, 0, n->stream>>>(n->parts, nb, n->d_loss);
     rc = n->cuda(cudaGetLastError(), "loss");
     if (!rc) rc = backward(n, H, W, n->dz);
     if (!rc) rc = n->cuda(cudaMemcpyAsync(n->h_loss, n->d_loss + 1, sizeof(double), cudaMemcpyDeviceToHost, n->stream), "loss copy");
-    if (!rc) rc = n->cuda(cudaStreamSynchronize(n->stream), "stream synchronize");
-    if (!rc) rc = check_err(n);
+    if (!rc) rc = finish(n);
     if (!rc && loss) *loss = *n->h_loss;
     return rc;
 }
