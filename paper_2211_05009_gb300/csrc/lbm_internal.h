@@ -32,15 +32,14 @@ constexpr int kMarchSteps = 4;
 inline bool march_dtype(int dtype) { return dtype == 1 || dtype == 2; }
 // Plain steps per launch of a shape.
 inline int config_steps(int dtype, int cfg) { return cfg < kRowConfigs || !march_dtype(dtype) ? 1 : kMarchSteps; }
-// Fastest row shape per storage type measured on GB300 at 2048 x 2048 (f64, f32, f32s, f16s, bf16s);
-// lbm_autotune re-measures on the caller's size.
+// Row shape behind shape kRowConfigs (f64, f32, f32s, f16s, bf16s, q16s): the fastest at 2048 x 2048.
 inline int default_row_config(int dtype) {
-    constexpr int k[6] = {1, 4, 0, 2, 2, 2};
+    constexpr int k[6] = {3, 0, 0, 2, 2, 2};
     return (dtype >= 0 && dtype < 6) ? k[dtype] : 0;
 }
 // Row shape of the single steps of a shape.
 inline int row_config(int dtype, int cfg) { return cfg < kRowConfigs ? cfg : default_row_config(dtype); }
-// Shape of a new context.
+// Shape of a new context; lbm_autotune measures all of them on the caller's size.
 int default_step_config(int dtype, int nx, int ny);
 
 constexpr int kDtypeQ16S = 5;

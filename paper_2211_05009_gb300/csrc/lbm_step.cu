@@ -16,10 +16,11 @@ cudaError_t launch_step_q16s(int cfg, const StepArgs& a, bool reduce, cudaStream
 
 namespace {
 struct Shape {
-    int R, BY;
+    int V, R, BY;
 };
-// must match launch_step_cfg in lbm_step_kernel.cuh
-constexpr Shape kShapes[kRowConfigs] = {{2, 2}, {1, 4}, {2, 2}, {4, 1}, {2, 4}, {4, 2}};
+// must match launch_step_cfg in lbm_step_kernel.cuh: FP64 and FP32 storage, 16-bit storage
+constexpr Shape kShapes[2][kRowConfigs] = {{{2, 2, 2}, {2, 1, 4}, {1, 1, 4}, {2, 4, 1}, {2, 2, 4}, {1, 1, 1}},
+                                           {{4, 2, 2}, {4, 1, 4}, {4, 2, 2}, {4, 4, 1}, {4, 2, 4}, {4, 4, 2}}};
 }  // namespace
 
 double q16_scale(int j, double U) {
@@ -40,19 +41,29 @@ QCodec q16_codec(double U) {
 }
 
 int default_step_config(int dtype, int nx, int ny) {
+    const long long n = (long long)nx * ny;
+    // Small grids: one node per lane and one row per warp put a step's dependent chain on as many
+    // warps as there are (us a step, shape 0 / the one taken: f64 128^2 11.0 / 4.9, 256^2 12.4 / 11.6;
+    // f32s 128^2 2.7 / 2.1, 500^2 4.1 / 4.0; f16s 128^2 3.6 / 3.0; q16s 256^2 4.3 / 3.3).
+    // Large ones: four rows per warp for FP64 (2048^2 471 / 454).
+    if (dtype == 0) return n < 50000 ? 2 : (n < 100000 ? 5 : (n < 200000 ? 0 : 3));
+    if (dtype >= 3) {
+        if (n < 600000) return 1;
+        return dtype == kDtypeQ16S || n < 8000000 ? 2 : 0;  // f16s 2048^2 25.0 with 2, 26.5 with 0; 4096^2 99.5, 94.9
+    }
+    if (n < (dtype == 2 ? 100000 : 50000)) return 2;
+    if (n < 300000) return 1;
     // Fused steps pay once the two population buffers outgrow the L2 cache; below that the rows that
     // neighbouring segments compute twice cost more than the saved launches.  us a step, row step
     // against fused: f32s 1024^2 8.5 / 8.4, 1500^2 26.1 / 13.8; f32 1024^2 9.1 / 13.1, 1500^2
     // 26.2 / 21.7, 500 x 1000 6.2 / 9.7.
-    const long long from = dtype == 2 ? 1000000 : 1600000;
-    return march_dtype(dtype) && (long long)nx * ny >= from ? kRowConfigs : default_row_config(dtype);
+    return n < (dtype == 2 ? 1000000 : 1600000) ? 0 : kRowConfigs;
 }
 
 StepGeometry step_geometry(int dtype, int cfg, int ny, long long pitch) {
     StepGeometry g{};
-    const int V = storage_bytes(dtype) == 2 ? 4 : 2;  // as launch_step_cfg
-    const Shape s = kShapes[row_config(dtype, cfg)];
-    g.grid_x = (int)(pitch / (32 * V));
+    const Shape s = kShapes[storage_bytes(dtype) == 2][row_config(dtype, cfg)];
+    g.grid_x = (int)(pitch / (32 * s.V));
     g.grid_y = (ny + s.BY * s.R - 1) / (s.BY * s.R);
     g.blocks = g.grid_x * g.grid_y;
     return g;

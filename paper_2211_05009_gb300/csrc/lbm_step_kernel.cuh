@@ -321,7 +321,8 @@ struct Relax {
     C pw9;        // 9 omega w_5
     C khalf;      // FP32: (1 - omega)/2.  FP64: 1 - omega
     C nhalf;      // FP32: -omega/2.       FP64: omega w_0
-    C o12;        // FP32: omega/12 = 3 omega w_5
+    C o12;        // omega/12 = 3 omega w_5
+    C wall;       // FP64: (omega - 1)/omega
 };
 template <typename C>
 __device__ __forceinline__ Relax<C> make_relax(C omega) {
@@ -335,6 +336,7 @@ __device__ __forceinline__ Relax<C> make_relax(C omega) {
     k.khalf = rmul(rsub(C(1.0), omega), C(f64 ? 1.0 : 0.5));
     k.nhalf = rmul(omega, C(f64 ? 4.0 / 9.0 : -0.5));
     k.o12 = rmul(omega, C(1.0 / 12.0));
+    k.wall = f64 ? (omega - C(1.0)) / omega : C(0.0);
     return k;
 }
 
@@ -356,9 +358,13 @@ __device__ __forceinline__ Relax<C> make_relax(C omega) {
 // FP64: 53 FP64 operations (72.7 instructions with the equilibrium formed per direction): the pipe
 // issues 2 lanes per clock and SM, so the operation count is the run time (2048^2: 7.3 GLUPS then).
 // out = keep g + (omega g^eq) with the pair's omega g^eq from two fused multiply-adds.
-template <typename C>
+//
+// FP64 ring nodes: f^eq(rho, u_w) + (1 - omega)(g - f^eq(rho, u)) at a resting wall has the fluid's
+// density terms and its velocity terms times (omega - 1)/omega, so `vel` (1 for a fluid node) turns
+// one into the other for five operations, where wall_shift takes 38 on a pipe that is the bound.
+template <typename C, bool WALLS = false>
 __device__ __forceinline__ void collide(const C (&g)[9], C one_ref, const Relax<C>& k, C (&out)[9], C& drho,
-                                        C& rho, C& ux, C& uy) {
+                                        C& rho, C& ux, C& uy, C vel = C(1.0)) {
     // d1 = g1 - g3, d2 = g2 - g4, and the negated n5 = g7 - g5, n8 = g6 - g8
     const C s1 = radd(g[1], g[3]), d1 = rsub(g[1], g[3]);
     const C s2 = radd(g[2], g[4]), d2 = rsub(g[2], g[4]);
@@ -366,12 +372,16 @@ __device__ __forceinline__ void collide(const C (&g)[9], C one_ref, const Relax<
     const C s8 = radd(g[8], g[6]), n8 = rsub(g[6], g[8]);
     drho = radd(radd(radd(s1, s2), radd(s5, s8)), g[0]);
     // -j and -1/rho, whose signs cancel in u: negations would be instructions of their own
-    const C jx = rsub(radd(n5, n8), d1);
-    const C jy = rsub(rsub(n5, n8), d2);
+    C jx = rsub(radd(n5, n8), d1);
+    C jy = rsub(rsub(n5, n8), d2);
     rho = radd(one_ref, drho);
     const C inv = nrcp<C>(rho);
     ux = rmul(jx, inv);
     uy = rmul(jy, inv);
+    if constexpr (WALLS) {
+        jx = rmul(jx, vel);
+        jy = rmul(jy, vel);
+    }
     // -a, -b, -c and -(a + b).  No sum of two products: the assembler fuses such packed ones.
     const C a = rmul(jx, ux), b = rmul(jy, uy), c = rmul(jx, uy);
     const C ab = rfma(jx, ux, b);
@@ -433,6 +443,23 @@ __device__ __forceinline__ void wall_shift(C rho, C ux, C uy, C W, C (&out)[9]) 
     out[7] = rfma(w5, rsub(q5, mp), out[7]);
     out[8] = rfma(w5, radd(q8, mm), out[8]);
     out[6] = rfma(w5, rsub(q8, mm), out[6]);
+}
+
+// What a wall moving along x with speed W adds to a resting one: f^eq(rho, W) - f^eq(rho, 0).
+template <typename C>
+__device__ __forceinline__ void lid_shift(C rho, C W, C (&out)[9]) {
+    const C j = rmul(rho, W), a = rmul(j, W);
+    const C w1 = C(1.0 / 9.0), w5 = C(1.0 / 36.0);
+    const C a3 = rmul(C(3.0), a), j3 = rmul(C(3.0), j);
+    out[0] = rfma(C(-2.0 / 3.0), a, out[0]);  // -3/2 w_0
+    out[1] = rfma(w1, radd(a3, j3), out[1]);
+    out[3] = rfma(w1, rsub(a3, j3), out[3]);
+    out[2] = rfma(C(-1.5) * w1, a, out[2]);
+    out[4] = rfma(C(-1.5) * w1, a, out[4]);
+    out[5] = rfma(w5, radd(a3, j3), out[5]);
+    out[8] = rfma(w5, radd(a3, j3), out[8]);
+    out[6] = rfma(w5, rsub(a3, j3), out[6]);
+    out[7] = rfma(w5, rsub(a3, j3), out[7]);
 }
 
 // ------------------------------------------------------------------ arithmetic per direction
@@ -569,8 +596,16 @@ __device__ __forceinline__ void pull_segment(const S* __restrict__ src, int lane
     pull_row<S, SHIFTED, V, -1, HINT>(pn + 7 * plane, lane, x0, pitch, C(1.0 / 36.0), q.dec[7], f[7]);
     pull_row<S, SHIFTED, V, 1, HINT>(pn + 8 * plane, lane, x0, pitch, C(1.0 / 36.0), q.dec[8], f[8]);
     if (x0 == 0) {
+        if constexpr (V > 1) {
 #pragma unroll
-        for (int j = 0; j < 9; ++j) f[j][0] = f[j][1];
+            for (int j = 0; j < 9; ++j) f[j][0] = f[j][1];
+        } else {  // x_f = 1 belongs to the next lane: pull it directly
+#pragma unroll
+            for (int j = 0; j < 9; ++j) {
+                const C v = ld1<S, HINT>(src + j * plane + (long long)(yc - cy(j)) * pitch + (1 - cx(j)), q.dec[j]);
+                f[j][0] = SHIFTED ? v : v - C(wd(j));
+            }
+        }
     }
     const int sR = nx - 1 - x0;  // slot of the right wall node in this lane, if any
 #pragma unroll
@@ -671,15 +706,19 @@ __device__ __forceinline__ void step_row(const S* __restrict__ src, S* __restric
         for (int j = 0; j < 9; ++j) g[j] = f[j][i];
         C out[9], drho, rho, ux, uy;
         constexpr bool PAIRS = kOnPairs<S, SHIFTED>;
-        if constexpr (PAIRS) collide<C>(g, one_ref, rx, out, drho, rho, ux, uy);
-        else moments9<C>(g, one_ref, drho, rho, ux, uy);
         const bool wall = EDGE && ((y == 0) | (y == ny - 1) | (x == 0) | (x >= nx - 1));
+        constexpr bool F64 = sizeof(C) == 8;
+        if constexpr (F64 && EDGE) collide<C, true>(g, one_ref, rx, out, drho, rho, ux, uy, wall ? rx.wall : C(1.0));
+        else if constexpr (PAIRS) collide<C>(g, one_ref, rx, out, drho, rho, ux, uy);
+        else moments9<C>(g, one_ref, drho, rho, ux, uy);
         C uox = ux, uoy = uy;
         if (wall) {
             const bool lid = (y == ny - 1) && (cv.corner_moving || (x > 0 && x < nx - 1));
             uox = lid ? cv.Ulid : C(0.0);
             uoy = C(0.0);
-            if constexpr (PAIRS) wall_shift<C>(rho, ux, uy, uox, out);
+            if constexpr (F64) {
+                if (lid) lid_shift<C>(rho, uox, out);
+            } else if constexpr (PAIRS) wall_shift<C>(rho, ux, uy, uox, out);
             else wall9<C>(g, drho, rho, ux, uy, uox, cv.omega, out);
         } else if constexpr (!PAIRS) {
             collide9<kMomentum<S>, C>(g, drho, rho, ux, uy, cv.omega, out);
@@ -831,15 +870,17 @@ static cudaError_t launch_step_shape(const StepArgs& a, bool reduce, cudaStream_
 template <typename S, bool SHIFTED>
 static cudaError_t launch_step_cfg(int cfg, const StepArgs& a, bool reduce, cudaStream_t st) {
     // nodes per lane: 2 for FP64 and FP32 storage (16- and 8-byte vectors; for FP32 the smaller
-    // register footprint buys more resident warps, measured faster than 4), 4 for 16-bit storage
+    // register footprint buys more resident warps, measured faster than 4), 4 for 16-bit storage;
+    // 1 in the shapes for small grids, which spread the nodes over as many warps as there are
     constexpr int V = sizeof(S) == 2 ? 4 : 2;
+    constexpr bool WIDE = sizeof(S) >= 4;
     switch (cfg) {
         case 0: return launch_step_shape<S, SHIFTED, V, 2, 2, 0>(a, reduce, st);
         case 1: return launch_step_shape<S, SHIFTED, V, 1, 4, 0>(a, reduce, st);
-        case 2: return launch_step_shape<S, SHIFTED, V, 2, 2, 1>(a, reduce, st);
+        case 2: return launch_step_shape<S, SHIFTED, WIDE ? 1 : V, WIDE ? 1 : 2, WIDE ? 4 : 2, WIDE ? 0 : 1>(a, reduce, st);
         case 3: return launch_step_shape<S, SHIFTED, V, 4, 1, 0>(a, reduce, st);
         case 4: return launch_step_shape<S, SHIFTED, V, 2, 4, 0>(a, reduce, st);
-        case 5: return launch_step_shape<S, SHIFTED, V, 4, 2, 1>(a, reduce, st);
+        case 5: return launch_step_shape<S, SHIFTED, WIDE ? 1 : V, WIDE ? 1 : 4, WIDE ? 1 : 2, WIDE ? 0 : 1>(a, reduce, st);
         default: return cudaErrorInvalidValue;
     }
 }
