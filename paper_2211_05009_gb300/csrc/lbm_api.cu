@@ -9,6 +9,7 @@
 #include <cstdio>
 #include <cstring>
 #include <string>
+#include <vector>
 
 #include "lbm.h"
 #include "lbm_internal.h"
@@ -33,6 +34,10 @@ std::string fmt(const char* f, ...) {
 }
 
 }  // namespace
+
+// Parts of an interval kept as graphs, and the steps from which one is worth it.
+constexpr size_t kMaxParts = 16;
+constexpr int kPartSteps = 4;
 
 struct lbm_ctx {
     int nx = 0, ny = 0;
@@ -62,7 +67,14 @@ struct lbm_ctx {
 
     cudaStream_t stream = nullptr;
     cudaStream_t cap_stream = nullptr;
-    cudaGraphExec_t chunk[2][2] = {};  // [checkpoint parity][buffer it starts from]
+    cudaGraphExec_t chunk[2][2] = {};  // whole intervals: [checkpoint parity][buffer it starts from]
+    // parts of an interval that callers step again and again (lbm_step(n) from the same place in an
+    // interval), most recently used first; a part is captured the second time it is seen
+    struct Part {
+        int s, n, slot, from;
+        cudaGraphExec_t exec;
+    };
+    std::vector<Part> parts;
     cudaEvent_t ev[2] = {nullptr, nullptr};
 
     ProbeSet probes{};
@@ -144,6 +156,9 @@ struct lbm_ctx {
                     cudaGraphExecDestroy(g);
                     g = nullptr;
                 }
+        for (auto& p : parts)
+            if (p.exec) cudaGraphExecDestroy(p.exec);
+        parts.clear();
     }
 
     // Enqueue one launch from global step gstep and buffer `from` on stream st: a checkpoint step by
@@ -169,25 +184,15 @@ struct lbm_ctx {
         }
         return rc;
     }
-    // Launches of one whole interval (each one changes the buffer).
-    int interval_launches() const {
-        const int f = config_steps(dtype, cfg);
-        return (kInterval - 1 + f - 1) / f + 1;
-    }
-
-    // 100-step graph for chunks that start at an aligned step in buffer `from`; slot = parity of the
-    // checkpoint.
-    int ensure_graph(int slot, int from) {
-        if (chunk[slot][from]) return LBM_OK;
+    // Graph of n steps from global step g0 in buffer `from`.
+    int capture(long long g0, int n, int from, cudaGraphExec_t* exec) {
         cudaGraph_t g = nullptr;
         int rc = cuda(cudaStreamBeginCapture(cap_stream, cudaStreamCaptureModeThreadLocal),
                       "begin graph capture");
         if (rc) return rc;
-        // the chunk ends at a checkpoint of parity `slot`; its first step is a multiple of 100
-        const long long g0 = slot == 1 ? 0 : kInterval;
         int b = from;
-        for (int s = 0, taken = 0; s < kInterval && !rc; s += taken, b ^= 1)
-            rc = enqueue(g0 + s, kInterval - s, b, cap_stream, &taken);
+        for (int s = 0, taken = 0; s < n && !rc; s += taken, b ^= 1)
+            rc = enqueue(g0 + s, n - s, b, cap_stream, &taken);
         cudaError_t e = cudaStreamEndCapture(cap_stream, &g);
         if (rc) {
             if (g) cudaGraphDestroy(g);
@@ -195,33 +200,78 @@ struct lbm_ctx {
         }
         rc = cuda(e, "end graph capture");
         if (rc) return rc;
-        rc = cuda(cudaGraphInstantiate(&chunk[slot][from], g, 0), "graph instantiate");
+        rc = cuda(cudaGraphInstantiate(exec, g, 0), "graph instantiate");
         cudaGraphDestroy(g);
         return rc;
+    }
+    // Launches of n steps from place s of an interval (each one changes the buffer).
+    int launches(int s, int n) const {
+        const int f = config_steps(dtype, cfg), plain = std::min(n, kInterval - 1 - s);
+        return (plain + f - 1) / f + (s + n == kInterval ? 1 : 0);
     }
 
     int advance(long long n) {
         int rc = LBM_OK;
         while (n > 0 && !rc) {
-            if (step % kInterval == 0 && n >= kInterval) {
-                const int slot = (int)(((step + kInterval) / kInterval) & 1);
-                rc = ensure_graph(slot, which);
+            const int s = (int)(step % kInterval), slot = (int)((step / kInterval + 1) & 1);
+            const int m = (int)std::min<long long>(n, kInterval - s);
+            cudaGraphExec_t exec = nullptr;
+            if (m == kInterval) {  // the graph ends at a checkpoint of parity `slot`
+                if (!chunk[slot][which]) rc = capture(slot == 1 ? 0 : kInterval, kInterval, which, &chunk[slot][which]);
                 if (rc) return rc;
-                rc = cuda(cudaGraphLaunch(chunk[slot][which], stream), "graph launch");
+                exec = chunk[slot][which];
+            } else if (m >= kPartSteps) {
+                rc = part(s, m, slot, &exec);
                 if (rc) return rc;
-                which ^= interval_launches() & 1;
-                step += kInterval;
-                n -= kInterval;
+            }
+            if (exec) {
+                rc = cuda(cudaGraphLaunch(exec, stream), "graph launch");
+                if (rc) return rc;
+                which ^= launches(s, m) & 1;
+                step += m;
+                n -= m;
             } else {
-                int taken = 0;
-                rc = enqueue(step, n, which, stream, &taken);
-                if (rc) return rc;
-                which ^= 1;
-                step += taken;
-                n -= taken;
+                for (int t = 0, taken = 0; t < m; t += taken) {
+                    rc = enqueue(step, m - t, which, stream, &taken);
+                    if (rc) return rc;
+                    which ^= 1;
+                    step += taken;
+                    n -= taken;
+                }
             }
         }
         return rc;
+    }
+
+    // The graph of a part, or null at its first sight (then it is launched directly, as it is into a
+    // stream that a caller is capturing).
+    int part(int s, int m, int slot, cudaGraphExec_t* exec) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+            cudaGetLastError();
+            return LBM_OK;
+        }
+        size_t k = 0;
+        while (k < parts.size() && !(parts[k].s == s && parts[k].n == m && parts[k].slot == slot && parts[k].from == which)) ++k;
+        if (k == parts.size()) {
+            if (parts.size() == kMaxParts) {
+                if (parts.back().exec) {
+                    const int rc = sync();  // it may still be running
+                    if (rc) return rc;
+                    cudaGraphExecDestroy(parts.back().exec);
+                }
+                parts.pop_back();
+            }
+            parts.insert(parts.begin(), Part{s, m, slot, which, nullptr});
+            return LBM_OK;
+        }
+        std::rotate(parts.begin(), parts.begin() + k, parts.begin() + k + 1);
+        if (!parts[0].exec) {
+            const int rc = capture((slot == 1 ? 0 : kInterval) + s, m, which, &parts[0].exec);
+            if (rc) return rc;
+        }
+        *exec = parts[0].exec;
+        return LBM_OK;
     }
 
     // Resolve a caller buffer: device pointers are used directly, host pointers go through

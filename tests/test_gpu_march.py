@@ -90,3 +90,22 @@ def test_fused_batch_equals_single_cavities(dtype):
         assert rc == B.LBM_OK and (done == 49).all()
     finally:
         B.lbm_batch_destroy(b)
+
+
+@pytest.mark.parametrize("dtype,cfg", [("f32s", 6), ("f32s", 2), ("f64", 5)])
+def test_repeated_parts_equal_one_call(dtype, cfg):
+    """The same few steps again and again (captured at their second sight, across checkpoints and past
+    the number of parts that are kept) give what one call of all of them gives."""
+    with Cavity(150, 70, Re=300.0, U=0.1, dtype=dtype) as a, Cavity(150, 70, Re=300.0, U=0.1, dtype=dtype) as b:
+        for c in (a, b):
+            B.lbm_set_launch_config(c.ctx, cfg)
+        sa, sb = (c.probe(0.5, 0.3, every=3, cap=700)[1] for c in (a, b))
+        total = 0
+        for k in range(40):
+            for n in (7, 20, 3 + k % 5):
+                a.step(n)
+                total += n
+        b.step(total)
+        assert a.step_count == b.step_count == total
+        assert torch.equal(a.populations(), b.populations()) and torch.equal(sa, sb)
+        assert a.residual() == b.residual()
