@@ -168,9 +168,9 @@ struct lbm_ctx {
         const int s = (int)(gstep % kInterval);
         const bool reduce = s == kInterval - 1;
         const int plain = (int)std::min<long long>(n, kInterval - 1 - s);
-        const int fused = reduce ? 1 : std::min(config_steps(dtype, cfg), plain);
+        const int fused = reduce ? 1 : std::min(config_steps(dtype, cfg, nx, ny), plain);
         *taken = fused;
-        int rc = fused > 1 ? cuda(launch_march(dtype, step_args(from, s), fused, sms, st), "fused step launch")
+        int rc = fused > 1 ? cuda(launch_fused(dtype, cfg, step_args(from, s), fused, sms, st), "fused step launch")
                            : cuda(launch_step(dtype, cfg, step_args(from, s), reduce, st), "step kernel launch");
         if (rc) return rc;
         if (reduce) {
@@ -206,7 +206,7 @@ struct lbm_ctx {
     }
     // Launches of n steps from place s of an interval (each one changes the buffer).
     int launches(int s, int n) const {
-        const int f = config_steps(dtype, cfg), plain = std::min(n, kInterval - 1 - s);
+        const int f = config_steps(dtype, cfg, nx, ny), plain = std::min(n, kInterval - 1 - s);
         return (plain + f - 1) / f + (s + n == kInterval ? 1 : 0);
     }
 
@@ -510,16 +510,16 @@ extern "C" int lbm_autotune(lbm_ctx* c, int steps_per_trial, int* best, double* 
     for (int k = 0; k < kStepConfigs; ++k) plain[k] = red[k] = 1e30f;
     // `n` steps of shape k (steps 0..97 of a checkpoint interval never reduce)
     auto plain_steps = [&](int k, int n) {
-        const int f = config_steps(t->dtype, k);
+        const int f = config_steps(t->dtype, k, t->nx, t->ny);
         for (int s = 0, from = 0; s < n && !rc; s += f, from ^= 1) {
             const int m = std::min(f, n - s);
-            rc = m > 1 ? c->cuda(launch_march(t->dtype, t->step_args(from, s % 94), m, t->sms, t->stream), "autotune launch")
+            rc = m > 1 ? c->cuda(launch_fused(t->dtype, k, t->step_args(from, s % 90), m, t->sms, t->stream), "autotune launch")
                        : c->cuda(launch_step(t->dtype, k, t->step_args(from, s % 98), false, t->stream), "autotune launch");
         }
     };
     for (int round = 0; round < 3 && !rc; ++round) {
         for (int k = 0; k < kStepConfigs && !rc; ++k) {
-            if (k >= kRowConfigs && config_steps(t->dtype, k) == 1) continue;  // the default row shape again
+            if (k >= kRowConfigs && config_steps(t->dtype, k, t->nx, t->ny) == 1) continue;  // the default row shape again
             if (round > 0 && plain[k] > 1.25f * *std::min_element(plain, plain + kStepConfigs)) continue;  // out of the race
             if (round == 0) plain_steps(k, steps_per_trial);  // warm-up
             if (!rc) rc = c->cuda(cudaEventRecord(e0, t->stream), "event record");

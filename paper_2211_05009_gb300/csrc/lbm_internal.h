@@ -26,13 +26,24 @@ struct StepGeometry {
 // storage; steps left over run as one shorter launch, checkpoint steps one by one.  The other types
 // gain nothing from fewer passes over memory and take their default row shape there: FP64 is bound by
 // its pipe, LBM_Q16S by its code conversions, and binary16 / bfloat16 meet the FP32 pipe first
-// (4096^2, fused 178 / 164 GLUPS, row step 177 / 174; 2048^2 145 / 134 against 168 / 162).
-constexpr int kStepConfigs = 7, kRowConfigs = 6;
+// (binary16 4096^2: fused 178 GLUPS, row step 178; 2048^2 150 against 168).
+// 7: several steps per launch in shared-memory tiles (lbm_tile.cuh), for small grids of every type
+// but FP64, whose pipe pays for nodes computed twice.
+constexpr int kStepConfigs = 8, kRowConfigs = 6, kMarchConfig = 6, kTileConfig = 7;
 constexpr int kMarchSteps = 4;
+struct TilePlan {
+    int ow, oh, steps;     // nodes a tile owns, steps per launch
+    int shift_x, shift_y;  // tiles begin at -shift
+};
+TilePlan tile_plan(int nx, int ny);
 inline bool march_dtype(int dtype) { return dtype == 1 || dtype == 2; }
 // Plain steps per launch of a shape.
-inline int config_steps(int dtype, int cfg) { return cfg < kRowConfigs || !march_dtype(dtype) ? 1 : kMarchSteps; }
-// Row shape behind shape kRowConfigs (f64, f32, f32s, f16s, bf16s, q16s): the fastest at 2048 x 2048.
+inline int config_steps(int dtype, int cfg, int nx, int ny) {
+    if (cfg == kMarchConfig && march_dtype(dtype)) return kMarchSteps;
+    if (cfg == kTileConfig && dtype != 0) return tile_plan(nx, ny).steps;
+    return 1;
+}
+// Row shape behind shapes 6 and 7 (f64, f32, f32s, f16s, bf16s, q16s): the fastest at 2048 x 2048.
 inline int default_row_config(int dtype) {
     constexpr int k[6] = {3, 0, 0, 2, 2, 2};
     return (dtype >= 0 && dtype < 6) ? k[dtype] : 0;
@@ -65,6 +76,12 @@ cudaError_t launch_step(int dtype, int cfg, const StepArgs& a, bool reduce, cuda
 // `steps` (1 .. kMarchSteps) plain steps from a.src to a.dst in one launch (march_dtype types only);
 // sms: multiprocessors of the device.
 cudaError_t launch_march(int dtype, const StepArgs& a, int steps, int sms, cudaStream_t st);
+// The same in shared-memory tiles (all types but FP64), steps <= p.steps.
+cudaError_t launch_tile(int dtype, const StepArgs& a, const TilePlan& p, int steps, cudaStream_t st);
+// `steps` plain steps in one launch as shape cfg takes them.
+inline cudaError_t launch_fused(int dtype, int cfg, const StepArgs& a, int steps, int sms, cudaStream_t st) {
+    return cfg == kTileConfig ? launch_tile(dtype, a, tile_plan(a.nx, a.ny), steps, st) : launch_march(dtype, a, steps, sms, st);
+}
 cudaError_t launch_finalize_checkpoint(const double* partials, int nblocks, double nodes,
                                        DevState* st, cudaStream_t s);
 

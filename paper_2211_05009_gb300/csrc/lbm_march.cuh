@@ -92,13 +92,14 @@ struct RowCodec {
     }
     // what put and get make of values that stay in registers
     __device__ static __forceinline__ void round(int j, f32x2 (&p)[HV]) {
-        if constexpr (sizeof(S) == 4 && SHIFTED) return;
+        if constexpr (sizeof(S) != 4 || !SHIFTED) {
 #pragma unroll
-        for (int k = 0; k < HV; ++k) {
-            const f32x2 v = SHIFTED ? p[k] : radd(p[k], f32x2(wd(j)));
-            p[k] = f32x2(to(from(v.lo())), to(from(v.hi())));
+            for (int k = 0; k < HV; ++k) {
+                const f32x2 v = SHIFTED ? p[k] : radd(p[k], f32x2(wd(j)));
+                p[k] = f32x2(to(from(v.lo())), to(from(v.hi())));
+            }
+            unshift(j, p);
         }
-        unshift(j, p);
     }
 };
 
@@ -139,7 +140,8 @@ __device__ __forceinline__ void march(const S* __restrict__ src, S* __restrict__
     const long long pitch = cv.pitch, plane = cv.plane;
     const Relax<float> rs = make_relax<float>(cv.omega);
     const Relax<f32x2> rx{f32x2(rs.ow1), f32x2(rs.ow5), f32x2(rs.w4), f32x2(rs.w9),
-                          f32x2(rs.pw9), f32x2(rs.khalf), f32x2(rs.nhalf), f32x2(rs.o12)};
+                          f32x2(rs.pw9), f32x2(rs.khalf), f32x2(rs.nhalf), f32x2(rs.o12), f32x2(0.0f)};
+    const Omega<f32x2> om = make_omega<f32x2>(cv.omega);
     const f32x2 one_ref(1.0f);
     const int x0 = xs + lane * V;
     const bool own = lane >= G::kHalo && lane < 32 - G::kHalo && x0 >= 0 && x0 < nx;
@@ -297,45 +299,73 @@ __device__ __forceinline__ void march(const S* __restrict__ src, S* __restrict__
                 }
             }
         } else {
-            auto node = [&](int k, float (&g)[9], float& drho, float& rho) {
+            f32x2 rho[HV], drho[HV], ux[HV], uy[HV];
 #pragma unroll
-                for (int j = 0; j < 9; ++j) g[j] = pair_get(f[j][k % HV], k / HV);
-                moments9<float>(g, 1.0f, drho, rho, vx[k], vy[k]);
-            };
-            auto put = [&](f32x2 (&w)[9][HV], int k, const float (&out)[9]) {
+            for (int k = 0; k < HV; ++k) {
+                f32x2 g[9];
+#pragma unroll
+                for (int j = 0; j < 9; ++j) g[j] = f[j][k];
+                moments9<f32x2>(g, one_ref, drho[k], rho[k], ux[k], uy[k]);
+            }
+            const bool special = edge | top | sampled | (y == 1);
+            if (special) {
+#pragma unroll
+                for (int k = 0; k < V; ++k) {
+                    vx[k] = pair_get(ux[k % HV], k / HV);
+                    vy[k] = pair_get(uy[k % HV], k / HV);
+                }
+            }
+            // the wall node that takes the values slot k pulled
+            auto wall = [&](int k, float W, float (&out)[9]) {
                 const int h = k / HV, m = k % HV;
+                float g[9];
 #pragma unroll
-                for (int j = 0; j < 9; ++j) w[j][m] = h ? f32x2(w[j][m].lo(), out[j]) : f32x2(out[j], w[j][m].hi());
+                for (int j = 0; j < 9; ++j) g[j] = pair_get(f[j][m], h);
+                wall9(g, pair_get(drho[m], h), pair_get(rho[m], h), vx[k], vy[k], W, cv.omega, out);
             };
             if (y == 1) {
                 f32x2 w[9][HV];
 #pragma unroll
-                for (int k = 0; k < V; ++k) {
-                    float g[9], out[9], drho, rho;
-                    node(k, g, drho, rho);
-                    wall9<float>(g, drho, rho, vx[k], vy[k], 0.0f, cv.omega, out);
-                    if (k < HV) {
+                for (int m = 0; m < HV; ++m) {
+                    float lo[9], hi[9];
+                    wall(m, 0.0f, lo);
+                    wall(m + HV, 0.0f, hi);
 #pragma unroll
-                        for (int j = 0; j < 9; ++j) w[j][k] = f32x2(out[j]);
-                    } else {
-                        put(w, k, out);
-                    }
+                    for (int j = 0; j < 9; ++j) w[j][m] = f32x2(lo[j], hi[j]);
                 }
                 emit_bottom(w);
             }
+            if (edge | top) {  // wall nodes from the pulled values, the others as below
 #pragma unroll
-            for (int k = 0; k < V; ++k) {
-                const int x = x0 + k;
-                float g[9], out[9], drho, rho;
-                node(k, g, drho, rho);
-                if ((edge | top) && (top | (x == 0) | (x == nx - 1))) {
-                    wall9<float>(g, drho, rho, vx[k], vy[k], wall_speed(x), cv.omega, out);
-                    vx[k] = wall_speed(x);
-                    vy[k] = 0.0f;
-                } else {
-                    collide9<kMomentum<S>, float>(g, drho, rho, vx[k], vy[k], cv.omega, out);
+                for (int k = 0; k < HV; ++k) {
+                    f32x2 g[9], out[9];
+#pragma unroll
+                    for (int j = 0; j < 9; ++j) g[j] = f[j][k];
+                    collide9<kMomentum<S>, f32x2>(g, drho[k], rho[k], ux[k], uy[k], om, out);
+                    float wo[2][9];
+                    bool is[2];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int x = x0 + k + h * HV;
+                        is[h] = top | (x == 0) | (x == nx - 1);
+                        if (!is[h]) continue;
+                        wall(k + h * HV, wall_speed(x), wo[h]);
+                        vx[k + h * HV] = wall_speed(x);
+                        vy[k + h * HV] = 0.0f;
+                    }
+#pragma unroll
+                    for (int j = 0; j < 9; ++j) f[j][k] = f32x2(is[0] ? wo[0][j] : out[j].lo(), is[1] ? wo[1][j] : out[j].hi());
                 }
-                put(f, k, out);
+            } else {
+#pragma unroll
+                for (int k = 0; k < HV; ++k) {
+                    f32x2 g[9], out[9];
+#pragma unroll
+                    for (int j = 0; j < 9; ++j) g[j] = f[j][k];
+                    collide9<kMomentum<S>, f32x2>(g, drho[k], rho[k], ux[k], uy[k], om, out);
+#pragma unroll
+                    for (int j = 0; j < 9; ++j) f[j][k] = out[j];
+                }
             }
         }
         if (sampled) {

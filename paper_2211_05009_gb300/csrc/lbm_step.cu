@@ -42,22 +42,22 @@ QCodec q16_codec(double U) {
 
 int default_step_config(int dtype, int nx, int ny) {
     const long long n = (long long)nx * ny;
-    // Small grids: one node per lane and one row per warp put a step's dependent chain on as many
-    // warps as there are (us a step, shape 0 / the one taken: f64 128^2 11.0 / 4.9, 256^2 12.4 / 11.6;
-    // f32s 128^2 2.7 / 2.1, 500^2 4.1 / 4.0; f16s 128^2 3.6 / 3.0; q16s 256^2 4.3 / 3.3).
-    // Large ones: four rows per warp for FP64 (2048^2 471 / 454).
+    // FP64 (us a step, shape 0 / the one taken: 128^2 11.0 / 4.9, 256^2 12.4 / 11.6, 2048^2 471 / 454):
+    // one node per lane on small grids spreads a step's dependent chain over as many warps as there
+    // are, four rows per warp on large ones.
     if (dtype == 0) return n < 50000 ? 2 : (n < 100000 ? 5 : (n < 200000 ? 0 : 3));
-    if (dtype >= 3) {
-        if (n < 600000) return 1;
-        return dtype == kDtypeQ16S || n < 8000000 ? 2 : 0;  // f16s 2048^2 25.0 with 2, 26.5 with 0; 4096^2 99.5, 94.9
-    }
-    if (n < (dtype == 2 ? 100000 : 50000)) return 2;
-    if (n < 300000) return 1;
-    // Fused steps pay once the two population buffers outgrow the L2 cache; below that the rows that
-    // neighbouring segments compute twice cost more than the saved launches.  us a step, row step
-    // against fused: f32s 1024^2 8.5 / 8.4, 1500^2 26.1 / 13.8; f32 1024^2 9.1 / 13.1, 1500^2
-    // 26.2 / 21.7, 500 x 1000 6.2 / 9.7.
-    return n < (dtype == 2 ? 1000000 : 1600000) ? 0 : kRowConfigs;
+    // Other types: tiles in shared memory while the grid is L2 resident and a step is mostly launch and
+    // latency (us a step, best row shape / tiles: f32s 128^2 2.1 / 1.0, 500^2 4.0 / 2.8, 500x1000 5.3 /
+    // 4.7; f32 128^2 2.2 / 1.3, 500x1000 6.2 / 6.1; f16s 128^2 3.0 / 1.3, 500x1000 6.7 / 5.7; q16s
+    // 128^2 3.3 / 1.6, 500x1000 9.6 / 8.9).
+    if (n < (dtype == 1 || dtype == kDtypeQ16S ? 600000 : 800000)) return kTileConfig;
+    // f16s 2048^2 25.0 with shape 2, 26.5 with 0; 4096^2 99.5, 94.9
+    if (dtype >= 3) return dtype == kDtypeQ16S || n < 8000000 ? 2 : 0;
+    // Steps fused in the march once the two population buffers outgrow the L2 cache; below that the
+    // rows that neighbouring segments compute twice cost more than the saved launches.  us a step, row
+    // step against fused: f32s 1024^2 8.5 / 8.4, 1500^2 26.1 / 13.8; f32 1024^2 9.1 / 11.9, 1500^2
+    // 26.2 / 19.3.
+    return n < (dtype == 2 ? 1000000 : 1600000) ? 0 : kMarchConfig;
 }
 
 StepGeometry step_geometry(int dtype, int cfg, int ny, long long pitch) {

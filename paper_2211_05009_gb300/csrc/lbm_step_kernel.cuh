@@ -466,80 +466,53 @@ __device__ __forceinline__ void lid_shift(C rho, C W, C (&out)[9]) {
 // LBM_F32 and 16-bit storage: what these store is rounded far above FP32 arithmetic on deviations
 // (4e-6 of the velocity after 250 steps of a 500 x 1000 cavity in LBM_F32, 5e-4 in binary16), so
 // their results are that rounding's noise.  They keep the arithmetic that forms every direction by
-// itself, and with it their results bit for bit.
-
-// Deviation equilibrium g^eq_j = w_j (drho + rho A_j), A_j = 3 c.u + 9/2 (c.u)^2 - 3/2 u.u (Eq. 2).
+// itself, and with it their results bit for bit; the rounding of each operation is spelled out here
+// too, scalar and packed.  Signs are placed so that nothing is negated by itself (rounding to
+// nearest is symmetric).
 template <typename C>
-__device__ __forceinline__ void geq9(C drho, C rho, C ux, C uy, C (&e)[9]) {
-    const C usq = C(1.5) * (ux * ux + uy * uy);
-    const C w0 = C(4.0 / 9.0), w1 = C(1.0 / 9.0), w5 = C(1.0 / 36.0);
-    auto A = [&](C cu) { return cu * (C(3.0) + C(4.5) * cu) - usq; };
-    const C up = ux + uy, um = ux - uy;
-    e[0] = w0 * (drho - rho * usq);
-    e[1] = w1 * (drho + rho * A(ux));
-    e[2] = w1 * (drho + rho * A(uy));
-    e[3] = w1 * (drho + rho * A(-ux));
-    e[4] = w1 * (drho + rho * A(-uy));
-    e[5] = w5 * (drho + rho * A(up));
-    e[6] = w5 * (drho + rho * A(-um));
-    e[7] = w5 * (drho + rho * A(-up));
-    e[8] = w5 * (drho + rho * A(um));
-}
-
-// BGK collision of a fluid node, f*_j = g_j + omega (g^eq_j - g_j) with g^eq_j = w_j (drho + rho A_j)
-// (Eq. 1, Eq. 2), written per opposite pair (j, jbar): A = c2 +- 3 c.u with c2 = 9/2 (c.u)^2 - usq,
-// so a pair shares c2, drho + rho c2 and 3 rho c.u.  About 50 operations per node instead of the
-// 65 of forming all nine g^eq and then relaxing towards them.  ow = omega w for the three weights.
+struct Omega {
+    C om, nom;        // omega, -omega
+    C ow0, ow1, ow5;  // omega w_j
+};
 template <typename C>
-__device__ __forceinline__ void collide_pairs(C drho, C rho, C ux, C uy, C omega, C ow0, C ow1, C ow5,
-                                              const C (&g)[9], C (&out)[9]) {
-    const C usq = C(1.5) * (ux * ux + uy * uy);
-    const C r3 = C(3.0) * rho;
-    out[0] = fma(ow0, fma(-rho, usq, drho), fma(-omega, g[0], g[0]));
-    auto pair = [&](int a, int b, C cu, C ow) {
-        const C c2 = fma(C(4.5) * cu, cu, -usq);
-        const C base = fma(rho, c2, drho);
-        const C sft = r3 * cu;
-        out[a] = fma(ow, base + sft, fma(-omega, g[a], g[a]));
-        out[b] = fma(ow, base - sft, fma(-omega, g[b], g[b]));
-    };
-    pair(1, 3, ux, ow1);
-    pair(2, 4, uy, ow1);
-    pair(5, 7, ux + uy, ow5);
-    pair(8, 6, ux - uy, ow5);
-}
-
-// FP32: hardware reciprocal estimate refined by one Newton-Raphson step r + r(1 - v r) (error
-// below one ulp for the densities rho ~ 1 met here; no subnormals).  The IEEE-rounded reciprocal
-// costs several times the instructions in a kernel that is partly issue-bound.
-__device__ __forceinline__ float rcp(float v) {
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
-    const float e = fmaf(-v, r, 1.0f);
-    return fmaf(r, e, r);
+__device__ __forceinline__ Omega<C> make_omega(float w) {
+    return Omega<C>{C(w), C(-w), C(rmul(w, float(4.0 / 9.0))), C(rmul(w, float(1.0 / 9.0))), C(rmul(w, float(1.0 / 36.0)))};
 }
 
 // Moments of a node (Eq. 3).
 template <typename C>
 __device__ __forceinline__ void moments9(const C (&g)[9], C one_ref, C& drho, C& rho, C& ux, C& uy) {
-    drho = ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7])) + g[8];
-    rho = one_ref + drho;
-    const C jx = (g[1] - g[3]) + (g[5] - g[6]) + (g[8] - g[7]);
-    const C jy = (g[2] - g[4]) + (g[5] + g[6]) - (g[7] + g[8]);
-    const C inv = rcp(rho);
-    ux = jx * inv;
-    uy = jy * inv;
+    drho = radd(radd(radd(radd(g[0], g[1]), radd(g[2], g[3])), radd(radd(g[4], g[5]), radd(g[6], g[7]))), g[8]);
+    rho = radd(one_ref, drho);
+    const C inv = nrcp<C>(rho);  // -1/rho, against -j
+    ux = rmul(radd(radd(rsub(g[3], g[1]), rsub(g[6], g[5])), rsub(g[7], g[8])), inv);
+    uy = rmul(radd(rsub(rsub(g[4], g[2]), radd(g[5], g[6])), radd(g[7], g[8])), inv);
+}
+
+// t_j with g^eq_j = w_j t_j, t_j = drho + rho A_j, A_j = 3 c.u + 9/2 (c.u)^2 - 3/2 u.u (Eq. 2).
+template <typename C>
+__device__ __forceinline__ void eq_terms(C drho, C rho, C ux, C uy, C (&t)[9]) {
+    const C nusq = rmul(C(-1.5), rfma(ux, ux, rmul(uy, uy)));
+    t[0] = rfma(rho, nusq, drho);
+    auto pair = [&](int a, int b, C cu) {
+        t[a] = rfma(rho, rfma(cu, rfma(C(4.5), cu, C(3.0)), nusq), drho);
+        t[b] = rfma(rho, rfma(cu, rfma(C(4.5), cu, C(-3.0)), nusq), drho);
+    };
+    pair(1, 3, ux);
+    pair(2, 4, uy);
+    pair(5, 7, radd(ux, uy));
+    pair(8, 6, rsub(ux, uy));
 }
 
 // Wall closure of a ring node from the values g pulled by its inner neighbour.
-template <typename C>
-__device__ __forceinline__ void wall9(const C (&g)[9], C drho, C rho, C ux, C uy, C W, C omega, C (&out)[9]) {
-    const C keep = C(1.0) - omega;  // 1 - 1/tau
-    C e[9], ew[9];
-    geq9<C>(drho, rho, ux, uy, e);
-    geq9<C>(drho, rho, W, C(0.0), ew);
+__device__ __forceinline__ void wall9(const float (&g)[9], float drho, float rho, float ux, float uy, float W, float omega,
+                                      float (&out)[9]) {
+    const float keep = rsub(1.0f, omega);  // 1 - 1/tau
+    float t[9], tw[9];
+    eq_terms<float>(drho, rho, ux, uy, t);
+    eq_terms<float>(drho, rho, W, 0.0f, tw);
 #pragma unroll
-    for (int j = 0; j < 9; ++j) out[j] = ew[j] + keep * (g[j] - e[j]);
+    for (int j = 0; j < 9; ++j) out[j] = rfma(float(wd(j)), tw[j], rmul(keep, rfma(-float(wd(j)), t[j], g[j])));
 }
 
 // Collision of a fluid node.  MOMENTUM: BGK as an increment d_j = (f^eq_j - f_j)/tau added to the
@@ -547,26 +520,40 @@ __device__ __forceinline__ void wall9(const C (&g)[9], C drho, C rho, C ux, C uy
 // rounding of f^eq otherwise shifts the momentum by a few ulps in the same direction every step.
 // LBM_Q16S rounds its stores to nearest, which passes such a bias on unchanged on average, so it
 // needs the correction as much as LBM_F32 does.  binary16 / bfloat16 swamp the bias and take the
-// pairwise form with fewer operations.
+// form per opposite pair, f*_j = g_j + omega (g^eq_j - g_j) with A = c2 +- 3 c.u.
 template <bool MOMENTUM, typename C>
-__device__ __forceinline__ void collide9(const C (&g)[9], C drho, C rho, C ux, C uy, C omega, C (&out)[9]) {
+__device__ __forceinline__ void collide9(const C (&g)[9], C drho, C rho, C ux, C uy, const Omega<C>& k, C (&out)[9]) {
     if constexpr (MOMENTUM) {
-        C e[9];
-        geq9<C>(drho, rho, ux, uy, e);
-        C d[9];
+        C t[9], n[9];
+        eq_terms<C>(drho, rho, ux, uy, t);
 #pragma unroll
-        for (int j = 0; j < 9; ++j) d[j] = omega * (e[j] - g[j]);
-        const C mx = (d[1] - d[3]) + (d[5] - d[6]) + (d[8] - d[7]);
-        const C my = (d[2] - d[4]) + (d[5] + d[6]) - (d[7] + d[8]);
-        d[1] -= C(0.5) * mx;
-        d[3] += C(0.5) * mx;
-        d[2] -= C(0.5) * my;
-        d[4] += C(0.5) * my;
-#pragma unroll
-        for (int j = 0; j < 9; ++j) out[j] = g[j] + d[j];
+        for (int j = 0; j < 9; ++j) n[j] = rfma(C(-wd(j)), t[j], g[j]);  // -d_j / omega
+        const C d3 = rmul(k.nom, n[3]), d4 = rmul(k.nom, n[4]), d6 = rmul(k.nom, n[6]), d7 = rmul(k.nom, n[7]);
+        // minus the x momentum, and the y momentum, of the increments
+        const C nmx = radd(radd(rfma(k.om, n[1], d3), rfma(k.om, n[5], d6)), rfma(k.om, n[8], d7));
+        const C my = rsub(rsub(rfma(k.nom, n[5], d6), rfma(k.om, n[2], d4)), rfma(k.nom, n[8], d7));
+        out[0] = rfma(k.nom, n[0], g[0]);
+        out[1] = radd(g[1], rfma(k.nom, n[1], rmul(C(0.5), nmx)));
+        out[3] = radd(g[3], rfma(C(-0.5), nmx, d3));
+        out[2] = radd(g[2], rfma(k.nom, n[2], rmul(C(-0.5), my)));
+        out[4] = radd(g[4], rfma(C(0.5), my, d4));
+        out[5] = rfma(k.nom, n[5], g[5]);
+        out[8] = rfma(k.nom, n[8], g[8]);
+        out[6] = radd(g[6], d6);
+        out[7] = radd(g[7], d7);
     } else {
-        const C ow0 = omega * C(4.0 / 9.0), ow1 = omega * C(1.0 / 9.0), ow5 = omega * C(1.0 / 36.0);
-        collide_pairs<C>(drho, rho, ux, uy, omega, ow0, ow1, ow5, g, out);
+        const C nusq = rmul(C(-1.5), rfma(ux, ux, rmul(uy, uy)));
+        const C r3 = rmul(C(3.0), rho), n3 = rmul(C(-3.0), rho);
+        out[0] = rfma(k.ow0, rfma(rho, nusq, drho), rfma(k.nom, g[0], g[0]));
+        auto pair = [&](int a, int b, C cu, C ow) {
+            const C base = rfma(rho, rfma(rmul(C(4.5), cu), cu, nusq), drho);
+            out[a] = rfma(ow, rfma(r3, cu, base), rfma(k.nom, g[a], g[a]));
+            out[b] = rfma(ow, rfma(n3, cu, base), rfma(k.nom, g[b], g[b]));
+        };
+        pair(1, 3, ux, k.ow1);
+        pair(2, 4, uy, k.ow1);
+        pair(5, 7, radd(ux, uy), k.ow5);
+        pair(8, 6, rsub(ux, uy), k.ow5);
     }
 }
 
@@ -677,6 +664,7 @@ __device__ __forceinline__ void step_row(const S* __restrict__ src, S* __restric
     const int nx = cv.nx, ny = cv.ny;
     const long long pitch = cv.pitch, plane = cv.plane;
     const Relax<C> rx = make_relax<C>(cv.omega);
+    const Omega<float> om = make_omega<float>(float(cv.omega));
     C f[9][V];
     pull_segment<S, SHIFTED, V, HINT>(src, lane, x0, y, nx, ny, pitch, plane, cv.q, f);
     // LBM_Q16S works on h = g - w rho_ref: BGK and the wall closure keep their form in h with
@@ -719,9 +707,9 @@ __device__ __forceinline__ void step_row(const S* __restrict__ src, S* __restric
             if constexpr (F64) {
                 if (lid) lid_shift<C>(rho, uox, out);
             } else if constexpr (PAIRS) wall_shift<C>(rho, ux, uy, uox, out);
-            else wall9<C>(g, drho, rho, ux, uy, uox, cv.omega, out);
+            else wall9(g, drho, rho, ux, uy, uox, cv.omega, out);
         } else if constexpr (!PAIRS) {
-            collide9<kMomentum<S>, C>(g, drho, rho, ux, uy, cv.omega, out);
+            collide9<kMomentum<S>, C>(g, drho, rho, ux, uy, om, out);
         }
 #pragma unroll
         for (int j = 0; j < 9; ++j) f[j][i] = out[j];
