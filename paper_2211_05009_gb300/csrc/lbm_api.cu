@@ -146,6 +146,7 @@ struct lbm_ctx {
         a.snap = snap;
         a.partials = partials;
         a.q = q;
+        a.rx = relax_f64(a.omega);
         return a;
     }
 
@@ -382,10 +383,10 @@ extern "C" int lbm_create_ex(int nx, int ny, double tau, double U, lbm_dtype dty
     c->q = q16_codec(U);
     c->plane = c->pitch * (long long)ny;
     c->cfg = default_step_config(c->dtype, nx, ny);
-    c->geo = step_geometry(c->dtype, c->cfg, ny, c->pitch);
+    c->geo = step_geometry(c->dtype, c->cfg, nx, ny);
     int max_blocks = 0;
     for (int k = 0; k < kStepConfigs; ++k) {
-        const int b = step_geometry(c->dtype, k, ny, c->pitch).blocks;
+        const int b = step_geometry(c->dtype, k, nx, ny).blocks;
         max_blocks = b > max_blocks ? b : max_blocks;
     }
 
@@ -476,7 +477,7 @@ extern "C" int lbm_set_launch_config(lbm_ctx* c, int cfg) {
     int rc = c->sync();
     if (rc) return rc;
     c->cfg = cfg;
-    c->geo = step_geometry(c->dtype, cfg, c->ny, c->pitch);
+    c->geo = step_geometry(c->dtype, cfg, c->nx, c->ny);
     c->invalidate_graphs();
     return LBM_OK;
 }

@@ -52,11 +52,15 @@ struct BatchShape {
 constexpr BatchShape kBatchShapes[LBM_BATCH_SHAPES] = {{2, 2, 5}, {1, 2, 5}, {4, 2, 5}, {2, 3, 5}, {1, 3, 5},
                                                        {4, 3, 5}, {2, 3, 4}, {4, 3, 4}, {2, 2, 8}, {4, 3, 8}};
 
+// Nodes per lane.
+template <int BYTES> constexpr int kBatchV = BYTES == 8 ? 1 : 4;
+
 struct BatchCav {
     long long off;       // population offset (storage elements) in each pool
     long long snap_off;  // snapshot offset (arithmetic-type elements)
     long long pitch, plane;
     int nx, ny;
+    Relax<double> rx;    // LBM_F64 only
     double omega, U;
     float omega_f, U_f;
     int corner_moving;
@@ -192,6 +196,7 @@ __global__ void __launch_bounds__(kBatchThreads, MINB) k_batch(const BatchArgs a
             cv.omega = sizeof(C) == 4 ? C(cd.omega_f) : C(cd.omega);
             cv.Ulid = sizeof(C) == 4 ? C(cd.U_f) : C(cd.U);
             cv.corner_moving = cd.corner_moving;
+            if constexpr (sizeof(C) == 8) cv.rx = cd.rx;
             cv.sref = cv.sref_w = C(0);  // reference density: LBM_Q16S only, which batches do not take
             ProbeOne pr;
             pr.n_ = (cd.series && !a.no_probe) ? 1 : 0;
@@ -446,7 +451,7 @@ static int batch_march_blocks(int dtype) {
 
 template <typename S, bool SHIFTED, int HINT, int MINB>
 static cudaError_t launch_batch_h(const BatchArgs& a, bool reduce, int blocks, cudaStream_t st) {
-    constexpr int V = sizeof(S) == 8 ? 2 : 4;
+    constexpr int V = kBatchV<sizeof(S)>;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(blocks);
     cfg.blockDim = dim3(kBatchThreads);
@@ -472,7 +477,7 @@ static cudaError_t launch_batch_t(const BatchShape& sh, const BatchArgs& a, bool
 
 template <typename S, bool SHIFTED, int HINT, int MINB>
 static int batch_blocks_h() {
-    constexpr int V = sizeof(S) == 8 ? 2 : 4;
+    constexpr int V = kBatchV<sizeof(S)>;
     int dev = 0, sms = 0, p0 = 0, p1 = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
@@ -909,7 +914,7 @@ extern "C" int lbm_batch_create(int n, const int* nx, const int* ny, const doubl
     lbm_batch* b = new lbm_batch();
     b->n = n;
     b->dtype = (int)dtype;
-    const int V = storage_bytes(b->dtype) == 8 ? 2 : 4;
+    const int V = storage_bytes(b->dtype) == 8 ? kBatchV<8> : kBatchV<4>;
     long long off = 0, soff = 0;
     int item0 = 0;
     size_t max_psi = 0;
@@ -922,12 +927,13 @@ extern "C" int lbm_batch_create(int n, const int* nx, const int* ny, const doubl
         const double tau = 3.0 * U[i] * nx[i] / Re[i] + 0.5;  // Re = U nx / nu, Eq. 5
         b->tau.push_back(tau);
         c.omega = 1.0 / tau;
+        c.rx = relax_f64(c.omega);
         c.U = U[i];
         c.omega_f = (float)c.omega;
         c.U_f = (float)U[i];
         c.off = off;
         c.snap_off = soff;
-        c.strips = (int)(c.pitch / (32 * V));
+        c.strips = (c.nx + 32 * V - 1) / (32 * V);
         c.items = c.strips * ny[i];  // one row per item: the largest item count of any shape
         c.item0 = item0;
         c.series = nullptr;

@@ -133,6 +133,45 @@ struct DevState {
     int pad2;
 };
 
+// Constants of the collision for one cavity (the FP32 and the FP64 form use different ones).
+template <typename C>
+struct Relax {
+    C ow1, ow5;   // omega w_1, omega w_5
+    C w4, w9;     // -9/2 omega w_1, -9 omega w_5
+    C pw9;        // 9 omega w_5
+    C khalf;      // FP32: (1 - omega)/2.  FP64: 1 - omega
+    C nhalf;      // FP32: -omega/2.       FP64: omega w_0
+    C o12;        // omega/12 = 3 omega w_5
+};
+// FP64: formed on the host (a division and nine products per thread were 9.6 of the 60.7 FP64
+// instructions a node and warp of a 500 x 1000 step), with the plain numbers of the collision beside
+// them: they are wanted in registers (collide).
+template <>
+struct Relax<double> {
+    double ow1, ow5, w4, w9, khalf, nhalf, o12;
+    double m1;           // 3 omega w_1
+    double one, nzero;   // 1, -0
+    double c15, cm3;     // 1.5, -3
+    double wall;         // (omega - 1)/omega
+};
+inline Relax<double> relax_f64(double omega) {
+    Relax<double> k;
+    k.ow1 = omega * (1.0 / 9.0);
+    k.ow5 = omega * (1.0 / 36.0);
+    k.w4 = k.ow1 * -4.5;
+    k.w9 = k.ow5 * -9.0;
+    k.khalf = 1.0 - omega;
+    k.nhalf = omega * (4.0 / 9.0);
+    k.o12 = omega * (1.0 / 12.0);
+    k.m1 = k.ow1 * 3.0;
+    k.one = 1.0;
+    k.nzero = -0.0;
+    k.c15 = 1.5;
+    k.cm3 = -3.0;
+    k.wall = (omega - 1.0) / omega;
+    return k;
+}
+
 struct StepArgs {
     const void* src;
     void* dst;
@@ -149,6 +188,7 @@ struct StepArgs {
     void* snap;        // [2][ny][pitch] Eq. 6 velocity snapshot, arithmetic type (REDUCE only)
     double* partials;  // [blocks][3]               (REDUCE only)
     QCodec q;          // LBM_Q16S scales (unused by the other storage types)
+    Relax<double> rx;  // LBM_F64 only
 };
 
 __device__ __forceinline__ double warp_sum(double v) {

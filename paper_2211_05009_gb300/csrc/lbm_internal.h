@@ -63,7 +63,7 @@ double q16_scale(int j, double U);
 QCodec q16_codec(double U);
 
 // Geometry of the step launch for a shape (also the number of reduction partials).
-StepGeometry step_geometry(int dtype, int cfg, int ny, long long pitch);
+StepGeometry step_geometry(int dtype, int cfg, int nx, int ny);
 
 // Bytes of the arithmetic type (FP64 for FP64 storage, FP32 otherwise): the Eq. 6 snapshot type.
 inline int arith_bytes(int dtype) { return dtype == 0 ? 8 : 4; }

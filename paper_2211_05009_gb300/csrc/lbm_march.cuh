@@ -140,7 +140,7 @@ __device__ __forceinline__ void march(const S* __restrict__ src, S* __restrict__
     const long long pitch = cv.pitch, plane = cv.plane;
     const Relax<float> rs = make_relax<float>(cv.omega);
     const Relax<f32x2> rx{f32x2(rs.ow1), f32x2(rs.ow5), f32x2(rs.w4), f32x2(rs.w9),
-                          f32x2(rs.pw9), f32x2(rs.khalf), f32x2(rs.nhalf), f32x2(rs.o12), f32x2(0.0f)};
+                          f32x2(rs.pw9), f32x2(rs.khalf), f32x2(rs.nhalf), f32x2(rs.o12)};
     const Omega<f32x2> om = make_omega<f32x2>(cv.omega);
     const f32x2 one_ref(1.0f);
     const int x0 = xs + lane * V;

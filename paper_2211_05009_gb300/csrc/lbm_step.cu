@@ -18,8 +18,9 @@ namespace {
 struct Shape {
     int V, R, BY;
 };
-// must match launch_step_cfg in lbm_step_kernel.cuh: FP64 and FP32 storage, 16-bit storage
-constexpr Shape kShapes[2][kRowConfigs] = {{{2, 2, 2}, {2, 1, 4}, {1, 1, 4}, {2, 4, 1}, {2, 2, 4}, {1, 1, 1}},
+// must match launch_step_cfg in lbm_step_kernel.cuh: FP64, FP32 storage, 16-bit storage
+constexpr Shape kShapes[3][kRowConfigs] = {{{1, 2, 2}, {1, 2, 4}, {1, 1, 4}, {1, 4, 1}, {1, 2, 1}, {1, 1, 1}},
+                                           {{2, 2, 2}, {2, 1, 4}, {1, 1, 4}, {2, 4, 1}, {2, 2, 4}, {1, 1, 1}},
                                            {{4, 2, 2}, {4, 1, 4}, {4, 2, 2}, {4, 4, 1}, {4, 2, 4}, {4, 4, 2}}};
 }  // namespace
 
@@ -42,10 +43,11 @@ QCodec q16_codec(double U) {
 
 int default_step_config(int dtype, int nx, int ny) {
     const long long n = (long long)nx * ny;
-    // FP64 (us a step, shape 0 / the one taken: 128^2 11.0 / 4.9, 256^2 12.4 / 11.6, 2048^2 471 / 454):
-    // one node per lane on small grids spreads a step's dependent chain over as many warps as there
-    // are, four rows per warp on large ones.
-    if (dtype == 0) return n < 50000 ? 2 : (n < 100000 ? 5 : (n < 200000 ? 0 : 3));
+    // FP64: one node per lane and one row per one-warp block at every size.  The FP64 pipe is the bound,
+    // a warp's node takes 1.7 us of it by itself, and the smaller the piece the more evenly the pieces
+    // fill the 608 pipes (us a step, best shape of two nodes per lane / this one: 128^2 7.2 / 4.5, 256^2
+    // 11.2 / 10.0, 500x1000 59.5 / 56.6, 700^2 55.8 / 54.6, 2048^2 435.5 / 435.3).
+    if (dtype == 0) return 5;
     // Other types: tiles in shared memory while the grid is L2 resident and a step is mostly launch and
     // latency (us a step, best row shape / tiles: f32s 128^2 2.1 / 1.0, 500^2 4.0 / 2.8, 500x1000 5.3 /
     // 4.7; f32 128^2 2.2 / 1.3, 500x1000 6.2 / 6.1; f16s 128^2 3.0 / 1.3, 500x1000 6.7 / 5.7; q16s
@@ -60,10 +62,10 @@ int default_step_config(int dtype, int nx, int ny) {
     return n < (dtype == 2 ? 1000000 : 1600000) ? 0 : kMarchConfig;
 }
 
-StepGeometry step_geometry(int dtype, int cfg, int ny, long long pitch) {
+StepGeometry step_geometry(int dtype, int cfg, int nx, int ny) {
     StepGeometry g{};
-    const Shape s = kShapes[storage_bytes(dtype) == 2][row_config(dtype, cfg)];
-    g.grid_x = (int)(pitch / (32 * s.V));
+    const Shape s = kShapes[dtype == 0 ? 0 : (storage_bytes(dtype) == 2 ? 2 : 1)][row_config(dtype, cfg)];
+    g.grid_x = (nx + 32 * s.V - 1) / (32 * s.V);
     g.grid_y = (ny + s.BY * s.R - 1) / (s.BY * s.R);
     g.blocks = g.grid_x * g.grid_y;
     return g;

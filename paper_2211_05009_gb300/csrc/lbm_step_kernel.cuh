@@ -305,38 +305,68 @@ template <> __device__ __forceinline__ f32x2 nrcp<f32x2>(f32x2 v) {
 // FP64: hardware estimate of 1/v (relative error below 2^-20) refined by one third-order step of
 // Householder's family, r (1 + e + e^2) with e = 1 - v r: the error e^3 is below 2^-60, so three
 // FP64 operations give 1/v to the last bit or the one beside it.  Densities are near 1 here; an
-// infinity or NaN comes out as NaN, which the checkpoint reports.
-template <> __device__ __forceinline__ double nrcp<double>(double v) {
+// infinity or NaN comes out as NaN, which the checkpoint reports.  `one` is 1 in a register.
+__device__ __forceinline__ double nrcp(double v, double one) {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(v));
-    const double e = __fma_rn(-v, r, 1.0);
+    const double e = __fma_rn(-v, r, one);
     return __fma_rn(-r, __fma_rn(e, e, e), -r);
 }
 
-// Constants of the collision for one cavity (the FP32 and the FP64 form use different ones).
+// The FP64 pipe takes 16.8 cycles for a warp's fused multiply-add of three registers and 19.9 for an
+// addition, a product, or a multiply-add with a literal or kernel-parameter operand (measured, 4 to 28
+// warps per SM).  So sums and products of the FP64 collision are multiply-adds by 1 and of -0, which
+// round to the same values, and every constant sits in a register.
 template <typename C>
-struct Relax {
-    C ow1, ow5;   // omega w_1, omega w_5
-    C w4, w9;     // -9/2 omega w_1, -9 omega w_5
-    C pw9;        // 9 omega w_5
-    C khalf;      // FP32: (1 - omega)/2.  FP64: 1 - omega
-    C nhalf;      // FP32: -omega/2.       FP64: omega w_0
-    C o12;        // omega/12 = 3 omega w_5
-    C wall;       // FP64: (omega - 1)/omega
+struct Ops {
+    const Relax<C>& k;
+    __device__ __forceinline__ C add(C a, C b) const {
+        if constexpr (std::is_same<C, double>::value) return rfma(a, k.one, b);
+        else return radd(a, b);
+    }
+    __device__ __forceinline__ C sub(C a, C b) const {
+        if constexpr (std::is_same<C, double>::value) return rfma(-b, k.one, a);
+        else return rsub(a, b);
+    }
+    __device__ __forceinline__ C mul(C a, C b) const {
+        if constexpr (std::is_same<C, double>::value) return rfma(a, b, k.nzero);
+        else return rmul(a, b);
+    }
 };
+
+// A parameter in a register: a value that went through a shuffle is no longer known to be uniform, so
+// the compiler keeps it where a lane's own values are.
+__device__ __forceinline__ Relax<double> in_registers(const Relax<double>& p) {
+    Relax<double> k;
+    auto own = [](double v) { return __shfl_sync(kFull, v, 0); };
+    k.ow1 = own(p.ow1);
+    k.ow5 = own(p.ow5);
+    k.w4 = own(p.w4);
+    k.w9 = own(p.w9);
+    k.khalf = own(p.khalf);
+    k.nhalf = own(p.nhalf);
+    k.o12 = own(p.o12);
+    k.m1 = own(p.m1);
+    k.one = own(p.one);
+    k.nzero = own(p.nzero);
+    k.c15 = own(p.c15);
+    k.cm3 = own(p.cm3);
+    k.wall = p.wall;
+    return k;
+}
+
+// Collision constants in FP32 (the FP64 ones come from the host, relax_f64).
 template <typename C>
 __device__ __forceinline__ Relax<C> make_relax(C omega) {
-    constexpr bool f64 = sizeof(C) == 8;
     Relax<C> k;
     k.ow1 = rmul(omega, C(1.0 / 9.0));
     k.ow5 = rmul(omega, C(1.0 / 36.0));
     k.w4 = rmul(k.ow1, C(-4.5));
     k.w9 = rmul(k.ow5, C(-9.0));
     k.pw9 = -k.w9;
-    k.khalf = rmul(rsub(C(1.0), omega), C(f64 ? 1.0 : 0.5));
-    k.nhalf = rmul(omega, C(f64 ? 4.0 / 9.0 : -0.5));
+    k.khalf = rmul(rsub(C(1.0), omega), C(0.5));
+    k.nhalf = rmul(omega, C(-0.5));
     k.o12 = rmul(omega, C(1.0 / 12.0));
-    k.wall = f64 ? (omega - C(1.0)) / omega : C(0.0);
     return k;
 }
 
@@ -365,32 +395,46 @@ __device__ __forceinline__ Relax<C> make_relax(C omega) {
 template <typename C, bool WALLS = false>
 __device__ __forceinline__ void collide(const C (&g)[9], C one_ref, const Relax<C>& k, C (&out)[9], C& drho,
                                         C& rho, C& ux, C& uy, C vel = C(1.0)) {
+    constexpr bool F64 = std::is_same<C, double>::value;
+    const Ops<C> o{k};
     // d1 = g1 - g3, d2 = g2 - g4, and the negated n5 = g7 - g5, n8 = g6 - g8
-    const C s1 = radd(g[1], g[3]), d1 = rsub(g[1], g[3]);
-    const C s2 = radd(g[2], g[4]), d2 = rsub(g[2], g[4]);
-    const C s5 = radd(g[5], g[7]), n5 = rsub(g[7], g[5]);
-    const C s8 = radd(g[8], g[6]), n8 = rsub(g[6], g[8]);
-    drho = radd(radd(radd(s1, s2), radd(s5, s8)), g[0]);
+    const C s1 = o.add(g[1], g[3]), d1 = o.sub(g[1], g[3]);
+    const C s2 = o.add(g[2], g[4]), d2 = o.sub(g[2], g[4]);
+    const C s5 = o.add(g[5], g[7]), n5 = o.sub(g[7], g[5]);
+    const C s8 = o.add(g[8], g[6]), n8 = o.sub(g[6], g[8]);
+    drho = o.add(o.add(o.add(s1, s2), o.add(s5, s8)), g[0]);
     // -j and -1/rho, whose signs cancel in u: negations would be instructions of their own
-    C jx = rsub(radd(n5, n8), d1);
-    C jy = rsub(rsub(n5, n8), d2);
-    rho = radd(one_ref, drho);
-    const C inv = nrcp<C>(rho);
-    ux = rmul(jx, inv);
-    uy = rmul(jy, inv);
+    C jx = o.sub(o.add(n5, n8), d1);
+    C jy = o.sub(o.sub(n5, n8), d2);
+    C inv;
+    if constexpr (F64) {
+        rho = o.add(drho, k.one);
+        inv = nrcp(rho, k.one);
+    } else {
+        rho = radd(one_ref, drho);
+        inv = nrcp<C>(rho);
+    }
+    ux = o.mul(jx, inv);
+    uy = o.mul(jy, inv);
     if constexpr (WALLS) {
-        jx = rmul(jx, vel);
-        jy = rmul(jy, vel);
+        jx = o.mul(jx, vel);
+        jy = o.mul(jy, vel);
     }
     // -a, -b, -c and -(a + b).  No sum of two products: the assembler fuses such packed ones.
-    const C a = rmul(jx, ux), b = rmul(jy, uy), c = rmul(jx, uy);
+    const C a = o.mul(jx, ux), b = o.mul(jy, uy), c = o.mul(jx, uy);
     const C ab = rfma(jx, ux, b);
-    const C jp = radd(jx, jy), jm = rsub(jx, jy);
-    const C base = rfma(C(1.5), ab, drho);
-    const C p1 = rmul(k.ow1, base), p5 = rmul(k.ow5, rfma(C(-3.0), ab, drho));
+    const C jp = o.add(jx, jy), jm = o.sub(jx, jy);
+    C c15, cm3;
+    if constexpr (F64) c15 = k.c15, cm3 = k.cm3;
+    else c15 = C(1.5), cm3 = C(-3.0);
+    const C base = rfma(c15, ab, drho);
+    const C p1 = o.mul(k.ow1, base), p5 = o.mul(k.ow5, rfma(cm3, ab, drho));
     const C q1 = rfma(k.w4, a, p1), q2 = rfma(k.w4, b, p1);
-    const C q5 = rfma(k.w9, c, p5), q8 = rfma(k.pw9, c, p5);
-    if constexpr (!std::is_same<C, double>::value) {
+    const C q5 = rfma(k.w9, c, p5);
+    C q8;
+    if constexpr (F64) q8 = rfma(-k.w9, c, p5);
+    else q8 = rfma(k.pw9, c, p5);
+    if constexpr (!F64) {
         const C u1 = rfma(k.khalf, s1, q1), u2 = rfma(k.khalf, s2, q2);
         const C u5 = rfma(k.khalf, s5, q5), u8 = rfma(k.khalf, s8, q8);
         const C e5 = rfma(k.nhalf, n5, rmul(k.o12, jp));  // -delta_5
@@ -407,8 +451,8 @@ __device__ __forceinline__ void collide(const C (&g)[9], C one_ref, const Relax<
         out[8] = rsub(u8, v8);
         out[6] = radd(u8, v8);
     } else {
-        const C m1 = rmul(k.ow1, C(3.0)), m5 = k.o12;
-        out[0] = rfma(k.khalf, g[0], rmul(k.nhalf, base));
+        const C m1 = k.m1, m5 = k.o12;
+        out[0] = rfma(k.khalf, g[0], o.mul(k.nhalf, base));
         out[1] = rfma(k.khalf, g[1], rfma(-m1, jx, q1));
         out[3] = rfma(k.khalf, g[3], rfma(m1, jx, q1));
         out[2] = rfma(k.khalf, g[2], rfma(-m1, jy, q2));
@@ -570,6 +614,17 @@ __device__ __forceinline__ void pull_segment(const S* __restrict__ src, int lane
                                              typename St<S>::C (&f)[9][V]) {
     using C = typename St<S>::C;
     const int yc = min(max(y, 1), ny - 2);  // gather centre row
+    if constexpr (V == 1) {
+        // one node per lane: every lane gathers at its own x_f.  The three columns of a row share their
+        // cache lines, and no load waits for a shuffle or sits in a branch.
+        const S* pf = src + (long long)yc * pitch + min(max(x0, 1), nx - 2);
+#pragma unroll
+        for (int j = 0; j < 9; ++j) {
+            vload_g<S, 1, HINT>(pf + j * plane - cy(j) * pitch - cx(j), q.dec[j], f[j]);
+            if constexpr (!SHIFTED) f[j][0] -= C(wd(j));
+        }
+        return;
+    }
     const S* pc = src + (long long)yc * pitch + x0;
     const S* ps = pc - pitch;  // row yc - 1: source of c_y = +1
     const S* pn = pc + pitch;  // row yc + 1: source of c_y = -1
@@ -582,18 +637,9 @@ __device__ __forceinline__ void pull_segment(const S* __restrict__ src, int lane
     pull_row<S, SHIFTED, V, -1, HINT>(ps + 6 * plane, lane, x0, pitch, C(1.0 / 36.0), q.dec[6], f[6]);
     pull_row<S, SHIFTED, V, -1, HINT>(pn + 7 * plane, lane, x0, pitch, C(1.0 / 36.0), q.dec[7], f[7]);
     pull_row<S, SHIFTED, V, 1, HINT>(pn + 8 * plane, lane, x0, pitch, C(1.0 / 36.0), q.dec[8], f[8]);
-    if (x0 == 0) {
-        if constexpr (V > 1) {
+    if (x0 == 0)
 #pragma unroll
-            for (int j = 0; j < 9; ++j) f[j][0] = f[j][1];
-        } else {  // x_f = 1 belongs to the next lane: pull it directly
-#pragma unroll
-            for (int j = 0; j < 9; ++j) {
-                const C v = ld1<S, HINT>(src + j * plane + (long long)(yc - cy(j)) * pitch + (1 - cx(j)), q.dec[j]);
-                f[j][0] = SHIFTED ? v : v - C(wd(j));
-            }
-        }
-    }
+        for (int j = 0; j < 9; ++j) f[j][0] = f[j][V > 1 ? 1 : 0];
     const int sR = nx - 1 - x0;  // slot of the right wall node in this lane, if any
 #pragma unroll
     for (int i = 1; i < V; ++i)
@@ -643,6 +689,7 @@ struct CavityView {
     long long pitch, plane;
     C omega, Ulid;
     int corner_moving;
+    Relax<C> rx;     // FP64 only
     QCodec q;        // LBM_Q16S only
     C sref, sref_w;  // LBM_Q16S only: rho_ref the populations are read against / stored against
 };
@@ -663,7 +710,9 @@ __device__ __forceinline__ void step_row(const S* __restrict__ src, S* __restric
     using C = typename St<S>::C;
     const int nx = cv.nx, ny = cv.ny;
     const long long pitch = cv.pitch, plane = cv.plane;
-    const Relax<C> rx = make_relax<C>(cv.omega);
+    Relax<C> rx;
+    if constexpr (sizeof(C) == 8) rx = cv.rx;
+    else rx = make_relax<C>(cv.omega);
     const Omega<float> om = make_omega<float>(float(cv.omega));
     C f[9][V];
     pull_segment<S, SHIFTED, V, HINT>(src, lane, x0, y, nx, ny, pitch, plane, cv.q, f);
@@ -696,7 +745,9 @@ __device__ __forceinline__ void step_row(const S* __restrict__ src, S* __restric
         constexpr bool PAIRS = kOnPairs<S, SHIFTED>;
         const bool wall = EDGE && ((y == 0) | (y == ny - 1) | (x == 0) | (x >= nx - 1));
         constexpr bool F64 = sizeof(C) == 8;
-        if constexpr (F64 && EDGE) collide<C, true>(g, one_ref, rx, out, drho, rho, ux, uy, wall ? rx.wall : C(1.0));
+        C vel = C(1.0);
+        if constexpr (F64) vel = wall ? rx.wall : rx.one;
+        if constexpr (F64 && EDGE) collide<C, true>(g, one_ref, rx, out, drho, rho, ux, uy, vel);
         else if constexpr (PAIRS) collide<C>(g, one_ref, rx, out, drho, rho, ux, uy);
         else moments9<C>(g, one_ref, drho, rho, ux, uy);
         C uox = ux, uoy = uy;
@@ -821,6 +872,7 @@ __global__ void __launch_bounds__(32 * BY, (kStepMinBlocks<S, BY>)) k_step(const
     cv.omega = sizeof(C) == 4 ? C(a.omega_f) : C(a.omega);
     cv.Ulid = sizeof(C) == 4 ? C(a.U_f) : C(a.U);
     cv.corner_moving = a.corner_moving;
+    if constexpr (sizeof(C) == 8) cv.rx = in_registers(a.rx);
     cv.sref = cv.sref_w = C(0);
     if constexpr (kIsQ16<S>) {
         cv.q = a.q;
@@ -846,7 +898,7 @@ __global__ void __launch_bounds__(32 * BY, (kStepMinBlocks<S, BY>)) k_step(const
 template <typename S, bool SHIFTED, int V, int R, int BY, int HINT>
 static cudaError_t launch_step_shape(const StepArgs& a, bool reduce, cudaStream_t st) {
     dim3 block(32, BY);
-    dim3 grid((unsigned)(a.pitch / (32 * V)), (unsigned)((a.ny + BY * R - 1) / (BY * R)));
+    dim3 grid((unsigned)((a.nx + 32 * V - 1) / (32 * V)), (unsigned)((a.ny + BY * R - 1) / (BY * R)));
     if (reduce)
         k_step<S, SHIFTED, true, V, R, BY, HINT><<<grid, block, 0, st>>>(a);
     else
@@ -862,6 +914,17 @@ static cudaError_t launch_step_cfg(int cfg, const StepArgs& a, bool reduce, cuda
     // 1 in the shapes for small grids, which spread the nodes over as many warps as there are
     constexpr int V = sizeof(S) == 2 ? 4 : 2;
     constexpr bool WIDE = sizeof(S) >= 4;
+    if constexpr (sizeof(S) == 8) {
+        switch (cfg) {
+            case 0: return launch_step_shape<S, SHIFTED, 1, 2, 2, 0>(a, reduce, st);
+            case 1: return launch_step_shape<S, SHIFTED, 1, 2, 4, 0>(a, reduce, st);
+            case 2: return launch_step_shape<S, SHIFTED, 1, 1, 4, 0>(a, reduce, st);
+            case 3: return launch_step_shape<S, SHIFTED, 1, 4, 1, 0>(a, reduce, st);
+            case 4: return launch_step_shape<S, SHIFTED, 1, 2, 1, 0>(a, reduce, st);
+            case 5: return launch_step_shape<S, SHIFTED, 1, 1, 1, 0>(a, reduce, st);
+            default: return cudaErrorInvalidValue;
+        }
+    } else {
     switch (cfg) {
         case 0: return launch_step_shape<S, SHIFTED, V, 2, 2, 0>(a, reduce, st);
         case 1: return launch_step_shape<S, SHIFTED, V, 1, 4, 0>(a, reduce, st);
@@ -870,6 +933,7 @@ static cudaError_t launch_step_cfg(int cfg, const StepArgs& a, bool reduce, cuda
         case 4: return launch_step_shape<S, SHIFTED, V, 2, 4, 0>(a, reduce, st);
         case 5: return launch_step_shape<S, SHIFTED, WIDE ? 1 : V, WIDE ? 1 : 4, WIDE ? 1 : 2, WIDE ? 0 : 1>(a, reduce, st);
         default: return cudaErrorInvalidValue;
+    }
     }
 }
 

@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(32 * kTileWarps, 2) k_tile(const TileArgs m) {
     const C omega = a.omega_f;
     const Relax<C> rs = make_relax<C>(omega);
     const Relax<f32x2> rx{f32x2(rs.ow1), f32x2(rs.ow5), f32x2(rs.w4), f32x2(rs.w9),
-                          f32x2(rs.pw9), f32x2(rs.khalf), f32x2(rs.nhalf), f32x2(rs.o12), f32x2(0.0f)};
+                          f32x2(rs.pw9), f32x2(rs.khalf), f32x2(rs.nhalf), f32x2(rs.o12)};
     const Omega<f32x2> om = make_omega<f32x2>(omega);
     C sref = C(0);
     if constexpr (kIsQ16<S>) sref = C(__ldcg(&a.state->rho_ref[0]));
