@@ -137,8 +137,8 @@ int lbm_get_info(const lbm_ctx *ctx, lbm_info *info);
 /* Advance n >= 0 time steps of Eq. 1 with the Sec. 2.2 (ii) walls: for every node pull
  * f_j(x - c_j) (streaming), form rho and u (Eq. 3) and collide towards f^eq (Eq. 2); wall nodes
  * take f^eq(rho_f, u_w) + (1 - 1/tau)[f(x_f) - f^eq(rho_f, u_f)] from their inner neighbour
- * x_f.  One fused kernel per step, or per few steps (launch shapes below).  After every step whose global index is a multiple of 100
- * the library also forms, in FP64, the mass sum rho and the Eq. 6 residual against the velocity
+ * x_f.  One fused kernel per step, or per few steps (launch shapes below).  After every step whose
+ * global index is a multiple of 100 the library also forms, in FP64, the mass sum rho and the Eq. 6 residual against the velocity
  * field of 100 steps earlier, and samples the probes (lbm_probe).  Asynchronous.
  * Errors: LBM_EINVAL (n < 0), LBM_ECUDA. */
 int lbm_step(lbm_ctx *ctx, long n);
@@ -153,9 +153,10 @@ int lbm_run_to_residual(lbm_ctx *ctx, double tol, long max_steps, long *steps_do
 
 /* ------------------------------------------------------------------ launch shapes */
 
-/* The time step has several launch shapes (rows per thread, warps per block, register budget; the
- * last one advances four steps per launch in FP32 storage).  They compute bitwise-identical populations; only
- * speed differs (the FP64 checkpoint sums may differ in the last bits, since the partial sums are
+/* The time step has several launch shapes: 0..5 take one step per launch (nodes per lane, rows per
+ * thread, warps per block), 6 takes four per launch in FP32 storage (grids beyond the L2 cache), 7 four
+ * in shared-memory tiles in every type but FP64 (small grids).  They compute bitwise-identical
+ * populations; only speed differs (the FP64 checkpoint sums may differ in the last bits, since the partial sums are
  * grouped by block). */
 int lbm_launch_config_count(void);
 
@@ -163,7 +164,8 @@ int lbm_launch_config_count(void);
 int lbm_set_launch_config(lbm_ctx *ctx, int cfg);
 
 /* Time every shape on a scratch context of the same size (the caller's state is not touched; the
- * scratch needs as much device memory as ctx): three rounds over all shapes of steps_per_trial
+ * scratch needs as much device memory as ctx): three rounds over all shapes (those more than a
+ * quarter behind after the first drop out) of steps_per_trial
  * (>= 2) plain steps and two checkpoint steps each, best time per shape, and select the shape
  * with the lowest cost of a 100-step interval (99 plain + 1 checkpoint).  *best / *best_glups
  * (either may be NULL) receive the choice and its step rate in 1e9 lattice updates per second.
@@ -283,7 +285,8 @@ int lbm_fma_peak(int fp64, int trips, double *flops_per_s, double *ms);
  * is bounded (default 2 s) and a wait that runs out makes the call return LBM_ETIMEOUT.  A whole
  * 100-step interval (both launches) is captured once in a CUDA graph and replayed.  Work items
  * are (cavity, 32-lane column strip, rows per item) with a tile shape from LBM_BATCH_SHAPES
- * (lbm_batch_autotune picks one).  Device memory comes from cudaMalloc (the allocator hook
+ * (lbm_batch_autotune picks one); plain steps of FP32 batches large enough run three per pass
+ * instead, unless lbm_batch_autotune measured that slower.  Device memory comes from cudaMalloc (the allocator hook
  * applies to single cavities only). */
 #define LBM_BATCH_MAX 512
 typedef struct lbm_batch lbm_batch;
@@ -409,9 +412,9 @@ int lbm_net_backward(lbm_net *n, const float *in, const float *base, const float
  * slower: its gather is bound by instruction issue); 3 = tcgen05 with those products as implicit
  * GEMMs over a channels-last BF16 copy of the input whose A tiles arrive as TMA boxes
  * (lbm_nn_conv3x3_bf16_tma; the default: the same sums as 1 in another order, equal to FP32
- * rounding, and a forward + backward pass 14-22 % faster); the weight gradient always runs on the
- * explicit im2col; 0 =
- * mma.sync.  Shapes a back end does not take run on 1.  With tcgen05, lbm_net_forward
+ * rounding; activations stay channels-last between convolutions, and the passes of an image size
+ * are captured in CUDA graphs at their second sight, at most 16 sizes); the weight gradient always
+ * runs on the explicit im2col; 0 = mma.sync.  Shapes a back end does not take run on 1.  With tcgen05, lbm_net_forward
  * synchronises, and a bounded tensor-core wait that runs out makes forward/backward return
  * LBM_ETIMEOUT. */
 int lbm_net_set_backend(lbm_net *n, int backend);

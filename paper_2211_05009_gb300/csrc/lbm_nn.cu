@@ -3,8 +3,10 @@
 // training (forward, backward, Adam) written as CUDA kernels.  Not part of the paper; it serves
 // the time-to-steady-state of the method's runs (Eq. 6 criterion) and is measured by it.
 //
-// Tensors are FP32 [C][H][W] (one sample).  Every 3x3 convolution (zero padding, stride 1) runs as
-// im2col + the BF16 tensor-core GEMM of lbm_nn_gemm.cu with FP32 accumulation:
+// Tensors are FP32 [C][H][W] (one sample).  Every 3x3 convolution (zero padding, stride 1) runs on a
+// BF16 tensor-core GEMM with FP32 accumulation, by default without a stored im2col: activations go
+// channels-last in BF16 from one GEMM's epilogue (bias, activation, skip split) to the next one's TMA
+// boxes.  Levels whose shape the boxes do not take, and the other back ends, use im2col:
 //   forward        Y[co][p]  = sum_k Wq[co][k] Xc[p][k]           (Xc: im2col of X, pixel-major)
 //   data grad      dX[ci][p] = sum_k Wf[ci][k] dZc[p][k]          (Wf: flipped, transposed W;
 //                                                                   dZc: im2col of dZ)

@@ -48,18 +48,21 @@ int default_step_config(int dtype, int nx, int ny) {
     // fill the 608 pipes (us a step, best shape of two nodes per lane / this one: 128^2 7.2 / 4.5, 256^2
     // 11.2 / 10.0, 500x1000 59.5 / 56.6, 700^2 55.8 / 54.6, 2048^2 435.5 / 435.3).
     if (dtype == 0) return 5;
-    // Other types: tiles in shared memory while the grid is L2 resident and a step is mostly launch and
-    // latency (us a step, best row shape / tiles: f32s 128^2 2.1 / 1.0, 500^2 4.0 / 2.8, 500x1000 5.3 /
-    // 4.7; f32 128^2 2.2 / 1.3, 500x1000 6.2 / 6.1; f16s 128^2 3.0 / 1.3, 500x1000 6.7 / 5.7; q16s
-    // 128^2 3.3 / 1.6, 500x1000 9.6 / 8.9).
-    if (n < (dtype == 1 || dtype == kDtypeQ16S ? 600000 : 800000)) return kTileConfig;
+    // Other types: tiles in shared memory while the grid is small enough that a step is mostly launch and
+    // latency (us a step, best other shape / tiles: f32s 250^2 1.9 / 1.4, 500^2 3.3 / 2.8, 900x1000 7.8 /
+    // 7.6, 950x1000 7.8 / 7.9; f32 128^2 1.7 / 1.3, 250^2 2.0 / 1.8, 350^2 2.5 / 3.1; q16s 500^2 5.9 / 5.0,
+    // 1050x1000 16.7 / 16.0, 1200x1000 17.8 / 17.7; f16s 500x1000 7.1 / 5.3, 1200x1000 10.3 / 10.2, 1200^2
+    // 11.7 / 12.2).
+    if (n < (dtype == 1 ? 90000 : (dtype == 2 ? 950000 : 1200000))) return kTileConfig;
     // f16s 2048^2 25.0 with shape 2, 26.5 with 0; 4096^2 99.5, 94.9
     if (dtype >= 3) return dtype == kDtypeQ16S || n < 8000000 ? 2 : 0;
     // Steps fused in the march once the two population buffers outgrow the L2 cache; below that the
-    // rows that neighbouring segments compute twice cost more than the saved launches.  us a step, row
-    // step against fused: f32s 1024^2 8.5 / 8.4, 1500^2 26.1 / 13.8; f32 1024^2 9.1 / 11.9, 1500^2
-    // 26.2 / 19.3.
-    return n < (dtype == 2 ? 1000000 : 1600000) ? 0 : kMarchConfig;
+    // rows that neighbouring segments compute twice cost more than the saved launches.  us a step,
+    // others against fused: f32s 950x1000 7.9 / 7.8, 1000x1050 8.9 / 8.6, 1500^2 26.1 / 13.8; f32 1100^2
+    // 11.8 / 12.9, 1500^2 26.2 / 19.3.
+    if (dtype == 2 || n >= 1600000) return kMarchConfig;
+    // f32, shape 0 / 2: 500x1000 6.4 / 5.7, 900x1000 9.3 / 8.8, 1000x1100 10.6 / 10.5, 1100^2 11.8 / 12.0
+    return n < 1150000 ? 2 : 0;
 }
 
 StepGeometry step_geometry(int dtype, int cfg, int nx, int ny) {

@@ -14,10 +14,11 @@
 // the new snapshot: per node in the arithmetic type, per thread over its few nodes, and in FP64
 // from the warp level up (FP64 throughput on this part is a small fraction of FP32's).
 //
-// Thread mapping: blockDim = (32, BY); each lane owns V consecutive nodes (V = 2: a 16-byte vector
-// for FP64, 8 bytes for FP32; V = 4: 8 bytes for 16-bit storage) of R consecutive rows, a warp
-// 32*V nodes per row.  The row pitch is a multiple of 32*V for every launch shape, so all vector
-// accesses are in bounds; padding nodes (x >= nx) store the rest state.
+// Thread mapping: blockDim = (32, BY); each lane owns V consecutive nodes (FP64: 1; FP32: 2, an 8-byte
+// vector, or 1 on small grids; 16-bit storage: 4, 8 bytes) of R consecutive rows, a warp 32*V nodes per
+// row.  The row pitch is a multiple of 32*V for every launch shape, so all vector accesses are in
+// bounds; the padding nodes (x >= nx) of the last strip that holds a node store the rest state, those
+// beyond keep what they had, and no node reads either.
 #pragma once
 
 #include <type_traits>
@@ -316,7 +317,8 @@ __device__ __forceinline__ double nrcp(double v, double one) {
 // The FP64 pipe takes 16.8 cycles for a warp's fused multiply-add of three registers and 19.9 for an
 // addition, a product, or a multiply-add with a literal or kernel-parameter operand (measured, 4 to 28
 // warps per SM).  So sums and products of the FP64 collision are multiply-adds by 1 and of -0, which
-// round to the same values, and every constant sits in a register.
+// round to the same values, and every constant sits in a register: 500 x 1000 56.2 -> 52.2 us a step,
+// 2048^2 434 -> 402.
 template <typename C>
 struct Ops {
     const Relax<C>& k;
@@ -386,7 +388,8 @@ __device__ __forceinline__ Relax<C> make_relax(C omega) {
 // direction with their momentum taken out 3.6e-7 U.)
 //
 // FP64: 53 FP64 operations (72.7 instructions with the equilibrium formed per direction): the pipe
-// issues 2 lanes per clock and SM, so the operation count is the run time (2048^2: 7.3 GLUPS then).
+// issues 2 lanes per clock and SM, so the operation count is the run time (2048^2: 7.3 GLUPS then, 10.4
+// now, 0.94 of what the pipe takes for 54.1 instructions a node at 16.8 cycles).
 // out = keep g + (omega g^eq) with the pair's omega g^eq from two fused multiply-adds.
 //
 // FP64 ring nodes: f^eq(rho, u_w) + (1 - omega)(g - f^eq(rho, u)) at a resting wall has the fluid's
@@ -909,11 +912,9 @@ static cudaError_t launch_step_shape(const StepArgs& a, bool reduce, cudaStream_
 // The shape tables; kShapes* in lbm_step.cu mirror them.
 template <typename S, bool SHIFTED>
 static cudaError_t launch_step_cfg(int cfg, const StepArgs& a, bool reduce, cudaStream_t st) {
-    // nodes per lane: 2 for FP64 and FP32 storage (16- and 8-byte vectors; for FP32 the smaller
-    // register footprint buys more resident warps, measured faster than 4), 4 for 16-bit storage;
-    // 1 in the shapes for small grids, which spread the nodes over as many warps as there are
-    constexpr int V = sizeof(S) == 2 ? 4 : 2;
-    constexpr bool WIDE = sizeof(S) >= 4;
+    // nodes per lane: 1 for FP64 (default_step_config), 2 for FP32 storage (8-byte vectors; the smaller
+    // register footprint buys more resident warps, measured faster than 4), 4 for 16-bit storage; 1 in
+    // the FP32 shapes for small grids, which spread the nodes over as many warps as there are
     if constexpr (sizeof(S) == 8) {
         switch (cfg) {
             case 0: return launch_step_shape<S, SHIFTED, 1, 2, 2, 0>(a, reduce, st);
@@ -925,15 +926,17 @@ static cudaError_t launch_step_cfg(int cfg, const StepArgs& a, bool reduce, cuda
             default: return cudaErrorInvalidValue;
         }
     } else {
-    switch (cfg) {
-        case 0: return launch_step_shape<S, SHIFTED, V, 2, 2, 0>(a, reduce, st);
-        case 1: return launch_step_shape<S, SHIFTED, V, 1, 4, 0>(a, reduce, st);
-        case 2: return launch_step_shape<S, SHIFTED, WIDE ? 1 : V, WIDE ? 1 : 2, WIDE ? 4 : 2, WIDE ? 0 : 1>(a, reduce, st);
-        case 3: return launch_step_shape<S, SHIFTED, V, 4, 1, 0>(a, reduce, st);
-        case 4: return launch_step_shape<S, SHIFTED, V, 2, 4, 0>(a, reduce, st);
-        case 5: return launch_step_shape<S, SHIFTED, WIDE ? 1 : V, WIDE ? 1 : 4, WIDE ? 1 : 2, WIDE ? 0 : 1>(a, reduce, st);
-        default: return cudaErrorInvalidValue;
-    }
+        constexpr int V = sizeof(S) == 2 ? 4 : 2;
+        constexpr bool WIDE = sizeof(S) == 4;
+        switch (cfg) {
+            case 0: return launch_step_shape<S, SHIFTED, V, 2, 2, 0>(a, reduce, st);
+            case 1: return launch_step_shape<S, SHIFTED, V, 1, 4, 0>(a, reduce, st);
+            case 2: return launch_step_shape<S, SHIFTED, WIDE ? 1 : V, WIDE ? 1 : 2, WIDE ? 4 : 2, WIDE ? 0 : 1>(a, reduce, st);
+            case 3: return launch_step_shape<S, SHIFTED, V, 4, 1, 0>(a, reduce, st);
+            case 4: return launch_step_shape<S, SHIFTED, V, 2, 4, 0>(a, reduce, st);
+            case 5: return launch_step_shape<S, SHIFTED, WIDE ? 1 : V, WIDE ? 1 : 4, WIDE ? 1 : 2, WIDE ? 0 : 1>(a, reduce, st);
+            default: return cudaErrorInvalidValue;
+        }
     }
 }
 
