@@ -14,7 +14,8 @@ The metric is lattice updates per second (GLUPS = nx*ny*100 per step / time).
   e2e       the same metric through the C ABI with HOST buffers: every step uploads the initial
             macroscopic field (rho, u_x, u_y; FP64, pinned) with lbm_set_moments, advances 100
             steps, reads the residual and downloads rho, u_x, u_y with lbm_moments
-  roofline  the step kernel: 18 populations x 4 bytes per node and launch / its average duration
+  roofline  the step kernel: 18 populations x 4 bytes per node and launch / the average duration of a
+            launch (launch shape 6 advances four steps per launch, and its bound is the FP32 pipe)
   cpu_baseline  the FP64 CPU oracle on a bounded sample of the same workload (first steps of
             the same 2048^2 cavity): its OpenMP build on every host core, and the plain build
             on one thread
@@ -44,7 +45,9 @@ CHUNK = 100
 BYTES_PER_LU = 18 * 4  # 9 populations read + 9 written, 4 bytes each
 METRIC = "D2Q9 GLUPS (fused step, lattice updates per second)"
 WORKLOAD = "square lid-driven cavity 2048x2048, Re=8000, U=0.05, FP32 arithmetic, FP32 shifted-deviation storage"
-PROFILE = os.path.join(ROOT, "profiles", "k_step_f32s_2048x2048.txt")
+FUSED_SHAPE, FUSED_STEPS = 6, 4  # the march: steps per launch
+PROFILES = {False: ("k_step_f32s_2048x2048.txt", ["lbm_step_kernel.cuh"]),
+            True: ("k_march_f32s_2048x2048.txt", ["lbm_march.cuh", "lbm_step_kernel.cuh"])}
 
 
 def parse_args():
@@ -159,7 +162,8 @@ def read_profile_traffic(shape: int):
     """Per-launch DRAM bytes of the step kernel's launch shape `shape` from the committed ncu
     summary, if it was taken on the current kernel source."""
     try:
-        text = open(PROFILE).read()
+        name, sources = PROFILES[shape == FUSED_SHAPE]
+        text = open(os.path.join(ROOT, "profiles", name)).read()
     except OSError:
         return None
     vals = {}
@@ -167,8 +171,8 @@ def read_profile_traffic(shape: int):
         if ":" in ln:
             k, v = ln.split(":", 1)
             vals[k.strip()] = v.strip()
-    src = os.path.join(ROOT, "paper_2211_05009_gb300", "csrc", "lbm_step_kernel.cuh")
-    digest = hashlib.sha256(open(src, "rb").read()).hexdigest()[:16]
+    digest = hashlib.sha256(b"".join(open(os.path.join(ROOT, "paper_2211_05009_gb300", "csrc", f), "rb").read()
+                                     for f in sources)).hexdigest()[:16]
     if vals.get("kernel_source_sha256_16") != digest:
         return None
     try:
@@ -251,7 +255,10 @@ def our_arm(args, rank, world, local_rank):
         torch.distributed.barrier()
     clk = clocks.stop()
     elapsed = start.elapsed_time(end) / 1e3
-    step_kernel_s = sum(a.elapsed_time(b) for a, b in ev_chunk) / 1e3 / (CHUNK * args.steps)
+    fused = cfg == FUSED_SHAPE
+    # launches of a chunk: its plain steps, fused or not, and the checkpoint step
+    launches = -(-(CHUNK - 1) // FUSED_STEPS) + 1 if fused else CHUNK
+    step_kernel_s = sum(a.elapsed_time(b) for a, b in ev_chunk) / 1e3 / (launches * args.steps)
     residual = B.lbm_residual(ctx)
     mass = B.lbm_mass(ctx)
     elapsed = max_over_ranks(elapsed, world)
@@ -320,14 +327,15 @@ def our_arm(args, rank, world, local_rank):
         "config": {"workload": WORKLOAD, "nx": NX, "ny": NY, "Re": RE, "U": U, "storage": STORAGE,
                    "lbm_steps_per_step": CHUNK, "parallelism": f"replicas{world}",
                    "l2": "population working set 302 MB > 129 MB L2; no flush"},
-        "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
+        "roofline": {"bound": "fp32 pipe" if fused else "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic,
-                     "peak_kind": peak_kind, "kernel": f"k_step<float, shifted> launch shape {cfg}",
+                     "peak_kind": peak_kind, "kernel": f"{'k_march' if fused else 'k_step'}<float, shifted> launch shape {cfg}",
+                     "steps_per_launch": FUSED_STEPS if fused else 1,
                      "algorithmic_bytes_per_launch": algo_bytes,
                      "avg_launch_us": step_kernel_s * 1e6},
         "cpu_baseline": cpu,
         "e2e": e2e,
-        "gpu_launches": args.steps * (CHUNK + 1 + 2),
+        "gpu_launches": args.steps * (launches + 1 + 2),
         "clocks": clk,
         "result": {"residual_eq6": residual, "mass": mass, "psi_min": psi_min, "xc": xc, "yc": yc,
                    "lbm_steps": (args.warmup + args.steps) * CHUNK},

@@ -1,7 +1,7 @@
 // lbm_march.cuh -- T time steps of the D2Q9 cavity in one pass over memory (FP32 arithmetic).
 //
-// 2048^2 LBM_F32S, T = 4: 20.5 us a step (205 GLUPS) against 46.6 (90) of the row step, which HBM
-// bounds at 94; 4096^2 76 against 175 us.  What bounds it now is the FP32 pipe: 61 packed operations
+// 2048^2 LBM_F32S, T = 4: 21.8 us a step (192 GLUPS) against 46.6 (90) of the row step, which HBM
+// bounds at 94; 4096^2 76 against 175 us; LBM_F32 2048^2 31.3 against 46.6.  What bounds it now is the FP32 pipe: 61 packed operations
 // a node, 15 % more of them for rows and 7 % for columns computed twice, take two thirds of the time,
 // register moves that pairs need most of the rest (336 instructions per 128 nodes and step).
 //
@@ -147,11 +147,17 @@ __device__ __forceinline__ void march(const S* __restrict__ src, S* __restrict__
     const bool own = lane >= G::kHalo && lane < 32 - G::kHalo && x0 >= 0 && x0 < nx;
     const bool edge = xs <= 0 || xs + 32 * V >= nx;  // the warp holds a wall column or padding
     const long long xl = min((long long)max(x0, 0), pitch - V);  // column loads stay in the row
-    // observing points in this strip's own columns and in rows [y0, y1)
+    // observing points in this strip's own columns and in rows [y0, y1), of this lane and of any lane
     unsigned pmask = 0;
     for (int p = 0; p < probes.n(); ++p)
         if (own && probes.px(p) >= x0 && probes.px(p) < x0 + V && probes.py(p) >= y0 && probes.py(p) < y1) pmask |= 1u << p;
-    const bool sampled = __any_sync(kFull, pmask != 0);
+    const unsigned watch = __reduce_or_sync(kFull, pmask);
+    // Only the rows around a point leave the plain path, decided once per row of step 1: the warp with the
+    // most to do ends last, and the rest wait for it (2048^2, two points in one strip: 30.7 us a step with
+    // every row of their segments on the other path, 22.6 so; 21.9 without points).  The batch decides
+    // once per segment: its kernel has no register left for the rows (20.5 -> 20.8 ms for 45 cavities).
+    constexpr bool kByRow = !std::is_same<Probes, ProbeOne>::value;
+    bool sampled = !kByRow && watch;
     Ring* const ring = static_cast<Ring*>(ring_v) + lane;
 
     const int i0 = max(1, y0 - (n - 1)), i1 = y1 + n - 2;
@@ -394,6 +400,13 @@ __device__ __forceinline__ void march(const S* __restrict__ src, S* __restrict__
     f32x2 row[9][HV];  // the row that the previous step has just produced
 #pragma unroll 1
     for (int i = i0; i <= i1; ++i) {
+        if constexpr (kByRow) {
+            if (watch) {
+                sampled = false;
+                for (int p = 0; p < probes.n(); ++p)  // step l is at row i - l + 1; row 0 goes with row 1
+                    if ((watch >> p) & 1u) sampled |= abs(2 * (i - max(probes.py(p), 1)) - n + 1) <= n + 1;
+            }
+        }
         bool on = i <= ny - 1;  // step 1 covers every row from i0 on
         if (on) {
             load_rows(i, row);
