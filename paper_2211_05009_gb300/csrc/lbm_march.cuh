@@ -154,9 +154,10 @@ __device__ __forceinline__ void march(const S* __restrict__ src, S* __restrict__
     const unsigned watch = __reduce_or_sync(kFull, pmask);
     // Only the rows around a point leave the plain path, decided once per row of step 1: the warp with the
     // most to do ends last, and the rest wait for it (2048^2, two points in one strip: 30.7 us a step with
-    // every row of their segments on the other path, 22.6 so; 21.9 without points).  The batch decides
-    // once per segment: its kernel has no register left for the rows (20.5 -> 20.8 ms for 45 cavities).
-    constexpr bool kByRow = !std::is_same<Probes, ProbeOne>::value;
+    // every row of their segments on the other path, 22.6 so; 21.9 without points).  The batch and
+    // LBM_F32 decide once per segment: their kernels have no register left for the rows (45 cavities 20.5
+    // -> 20.8 ms; LBM_F32 2048^2 without points 31.3 -> 34.1 us a step).
+    constexpr bool kByRow = SHIFTED && !std::is_same<Probes, ProbeOne>::value;
     bool sampled = !kByRow && watch;
     Ring* const ring = static_cast<Ring*>(ring_v) + lane;
 
