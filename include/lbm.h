@@ -402,7 +402,9 @@ int lbm_net_forward(lbm_net *n, const float *in, int H, int W, float *out);
 /* Forward, loss = mean over masked pixels and 3 channels of e^2, e = base + out - target with the
  * masked mean of e removed in channel 0 (the density channel counts up to a constant), backward:
  * gradients are ADDED to the accumulated gradient (lbm_net_zero_grads clears it).  mask [H][W]
- * is 0/1; base, target [3][H][W].  *loss (host, may be NULL).  Synchronising. */
+ * is 0/1; base, target [3][H][W].  *loss (host, may be NULL).  Gradients have the same bits on every
+ * run, but for the weights of convolutions over 16,384 pixels or more: those are summed in slices that
+ * arrive in any order.  Synchronising. */
 int lbm_net_backward(lbm_net *n, const float *in, const float *base, const float *target,
                      const float *mask, int H, int W, double *loss);
 /* GEMM back end of the convolutions: 1 = tcgen05 (5th-generation tensor cores, TMEM

@@ -153,19 +153,48 @@ __global__ void __launch_bounds__(256) k_to_channels_last(const float* __restric
 }
 
 // dz = dy act'(y) in BF16, channel-major [co][P] (the weight gradient's operand) and channels-last
-// [P][Cp] (the data gradient's input), and db[c] += sum_p dz in FP32: one pixel and 8 channels per
-// thread.
+// [P][Cp] (the data gradient's input): one pixel and 8 channels per thread.  The blocks from row Cp / 8
+// of the grid on add db[c] += sum_p dz in FP32, a channel each, in the order of k_act_back, so that a
+// bias gradient has the same bits on every run; they run beside the other blocks.
 __global__ void __launch_bounds__(256) k_act_back_cl(const float* __restrict__ y, const float* __restrict__ dy, int C, int P,
                                                      int Cp, int act, float* __restrict__ db, __nv_bfloat16* __restrict__ dzq,
                                                      __nv_bfloat16* __restrict__ X) {
-    __shared__ float sh[8][8];
+    if (blockIdx.y >= Cp / 8) {
+        const int c = (blockIdx.y - Cp / 8) * gridDim.x + blockIdx.x;
+        if (c >= C) return;
+        __shared__ float sh[256];
+        const float* __restrict__ gp = dy + (long long)c * P;
+        const float* __restrict__ yp = y + (long long)c * P;
+        float s = 0.f;
+        constexpr int kBatch = 16;  // loads in flight: the sum is a chain, its operands are not
+        int p = threadIdx.x;
+        for (; p + (kBatch - 1) * 256 < P; p += kBatch * 256) {
+            float g[kBatch], v[kBatch];
+#pragma unroll
+            for (int j = 0; j < kBatch; ++j) {
+                g[j] = gp[p + j * 256];
+                v[j] = act ? yp[p + j * 256] : 1.f;
+            }
+#pragma unroll
+            for (int j = 0; j < kBatch; ++j) s = __fadd_rn(s, v[j] <= 0.f ? __fmul_rn(g[j], kLeak) : g[j]);
+        }
+        for (; p < P; p += 256) s = __fadd_rn(s, act && yp[p] <= 0.f ? __fmul_rn(gp[p], kLeak) : gp[p]);
+        sh[threadIdx.x] = s;
+        __syncthreads();
+        for (int o = 128; o > 0; o >>= 1) {
+            if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) db[c] += sh[0];
+        return;
+    }
     const int p = blockIdx.x * blockDim.x + threadIdx.x, cg = blockIdx.y * 8;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (p >= P) return;
     __nv_bfloat16 b[8];
     float gv[8], yv[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {  // all loads in flight before the first use
-        const bool in = cg + j < C && p < P;
+        const bool in = cg + j < C;
         const long long i = in ? (long long)(cg + j) * P + p : 0;
         gv[j] = in ? dy[i] : 0.f;
         yv[j] = in && act ? y[i] : 1.f;
@@ -175,19 +204,9 @@ __global__ void __launch_bounds__(256) k_act_back_cl(const float* __restrict__ y
         float g = gv[j];
         if (yv[j] <= 0.f) g *= kLeak;
         b[j] = __float2bfloat16_rn(g);
-        if (cg + j < C && p < P) dzq[(long long)(cg + j) * P + p] = b[j];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
-        if (lane == 0) sh[warp][j] = g;
+        if (cg + j < C) dzq[(long long)(cg + j) * P + p] = b[j];
     }
-    if (p < P) *reinterpret_cast<uint4*>(X + (long long)p * Cp + cg) = *reinterpret_cast<const uint4*>(b);
-    __syncthreads();
-    if (threadIdx.x < 8 && cg + threadIdx.x < C) {
-        float s = 0.f;
-#pragma unroll
-        for (int w = 0; w < 8; ++w) s += sh[w][threadIdx.x];
-        atomicAdd(db + cg + threadIdx.x, s);
-    }
+    *reinterpret_cast<uint4*>(X + (long long)p * Cp + cg) = *reinterpret_cast<const uint4*>(b);
 }
 
 // Weights of every convolution as BF16 from the FP32 parameters, one launch per change of them.
@@ -698,22 +717,25 @@ int im2col_kp(lbm_net* n, const ConvSpec& c, const float* x1, int c1, const floa
     return n->cuda(cudaGetLastError(), "im2col (k-major)");
 }
 
+// Slices of the weight gradient's sum over P pixels: one below 16,384, so that its order is fixed, and
+// one per 4096 pixels (at most 32) from there on, added in the order of their arrival.  Slices until the
+// tiles fill the GPU take 6.3 instead of 8.5 ms for eight 128-wide samples (width 20, P = 8,192 ..
+// 22,528), but then every gradient has other bits on every run, 5e-4 of the BF16-rounded ones apart.
+inline int pixel_slices(long long P) { return P >= 16384 ? (int)std::min<long long>(32, P / 4096) : 1; }
+
 // Backend 3: given dL/dy (gy) and y, accumulate dW and db and store dL/dx (gx1: c1 channels, gx2: c2).
-// The weight gradient is split over the pixels until its tiles fill the GPU, down to four K steps each:
-// with one slice per 4096 pixels a 128-wide level-0 layer ran on 8 CTAs.
 int conv_bwd_cl(lbm_net* n, int ci, const float* x1, int c1, const float* x2, int c2, int H, int W, const float* y,
                 const float* gy, float* gx1, float* gx2) {
     const ConvSpec& c = n->convs[ci];
     const int P = H * W, cp = conv_cp(c.co);
-    k_act_back_cl<<<dim3(nblk(P), (unsigned)(cp / 8)), 256, 0, n->stream>>>(y, gy, c.co, P, cp, c.act, n->grads + c.boff, n->dzq,
-                                                                         n->cl[0]);
+    const unsigned blocks = nblk(P), sums = (c.co + blocks - 1) / blocks;
+    k_act_back_cl<<<dim3(blocks, (unsigned)(cp / 8) + sums), 256, 0, n->stream>>>(y, gy, c.co, P, cp, c.act, n->grads + c.boff,
+                                                                               n->dzq, n->cl[0]);
     int rc = n->cuda(cudaGetLastError(), "activation backward");
     if (!rc) rc = im2col_kp(n, c, x1, c1, x2, c2, H, W);
-    if (!rc) {
-        const int tiles = (c.ci * 9 + 127) / 128, split = std::max(1, std::min(152 / tiles, P / 256));
-        rc = n->cuda(gemm_bf16_nt_umma(c.ci * 9, c.co, P, n->col, P, n->dzq, P, n->grads + c.woff, c.ci * 9, kAtomicAdd, true, split,
-                                       n->d_err, n->stream), "weight-gradient gemm (tcgen05)");
-    }
+    if (!rc)
+        rc = n->cuda(gemm_bf16_nt_umma(c.ci * 9, c.co, P, n->col, P, n->dzq, P, n->grads + c.woff, c.ci * 9, kAtomicAdd, true,
+                                       pixel_slices(P), n->d_err, n->stream), "weight-gradient gemm (tcgen05)");
     if (rc || !gx1) return rc;
     const int rows = c1 + (gx2 ? c2 : 0);
     if (conv_tma_takes(H, W))
@@ -739,7 +761,7 @@ int conv_bwd(lbm_net* n, const ConvSpec& c, const float* x1, int c1, const float
         rc = im2col_kp(n, c, x1, c1, x2, c2, H, W);
     }
     if (!rc) {
-        const int split = P >= 16384 ? (int)std::min<long long>(32, P / 4096) : 1;
+        const int split = pixel_slices(P);
         if (n->backend != 0)  // rows k of the k-major im2col on the 128-row side, co on N
             rc = n->cuda(gemm_bf16_nt_umma(c.ci * 9, c.co, (int)P, n->col, (int)P, n->dzq, (int)P, n->grads + c.woff, c.ci * 9,
                                            kAtomicAdd, true, split, n->d_err, n->stream), "weight-gradient gemm (tcgen05)");
