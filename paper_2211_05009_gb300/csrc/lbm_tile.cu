@@ -1,15 +1,37 @@
 // lbm_tile.cu -- launches of the shared-memory tile kernel (lbm_tile.cuh): several plain time steps of
 // a small cavity per launch.
+#include <atomic>
+
 #include "lbm_internal.h"
 #include "lbm_tile.cuh"
 
 namespace lbm {
 
 namespace {
+constexpr int kTileSteps = 4, kTileLow = 10, kTileHigh = 24;  // steps of a launch, rows a tile owns
+constexpr int tile_bytes(int oh, int n, int elem) { return 2 * 9 * kTileCols * (oh + 2 * n) * elem; }
+
+// Opt in to the largest tile's shared memory, once per device.  The attribute belongs to the kernel on the
+// device: a launch that set it to its own size would lower it between another context's set and launch
+// (contexts are independent, each with a thread of its own), and that launch would be refused.
+template <typename S, bool SHIFTED>
+cudaError_t opt_in() {
+    static std::atomic<unsigned long long> done{0};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
+    if (done.load(std::memory_order_relaxed) & bit) return cudaSuccess;
+    e = cudaFuncSetAttribute(k_tile<S, SHIFTED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             tile_bytes(kTileHigh, kTileSteps, (int)sizeof(S)));
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_relaxed);
+    return e;
+}
+
 template <typename S, bool SHIFTED>
 cudaError_t launch_tile_t(const StepArgs& a, const TilePlan& p, int n, cudaStream_t st) {
-    const int smem = 2 * 9 * kTileCols * (p.oh + 2 * n) * (int)sizeof(S);
-    const cudaError_t e = cudaFuncSetAttribute(k_tile<S, SHIFTED>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const int smem = tile_bytes(p.oh, n, (int)sizeof(S));
+    const cudaError_t e = opt_in<S, SHIFTED>();
     if (e != cudaSuccess) return e;
     TileArgs m;
     m.a = a;
@@ -23,12 +45,12 @@ cudaError_t launch_tile_t(const StepArgs& a, const TilePlan& p, int n, cudaStrea
 
 TilePlan tile_plan(int nx, int ny) {
     TilePlan p{};
-    p.steps = 4;
+    p.steps = kTileSteps;
     p.ow = kTileCols - 2 * p.steps;
     // Rows so that the row pairs of a step fill the warps once (10 + 2 x 3 rows, 8 pairs) or twice
     // (24): the taller tile computes fewer nodes twice, the lower one makes more blocks.
     const int cols = (nx + p.ow - 1) / p.ow;
-    p.oh = (long long)cols * ((ny + 9) / 10) <= 2 * 148 ? 10 : 24;
+    p.oh = (long long)cols * ((ny + 9) / 10) <= 2 * 148 ? kTileLow : kTileHigh;
     // a wall is never the only column or row of a tile; columns move by a copy's alignment
     p.shift_x = nx % p.ow == 1 ? 4 : 0;
     p.shift_y = ny % p.oh == 1 ? 1 : 0;

@@ -1,0 +1,36 @@
+"""Contexts beside one another and beside a caller's own CUDA work: threads, captured streams, work that
+is still queued, device memory from a caller's allocator."""
+import threading
+
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_2211_05009_gb300.cavity import Cavity  # noqa: E402
+
+
+def test_contexts_step_in_two_threads():
+    """Tiles of two heights at once, in launches of 2, 3 and 4 steps: what each alone gives."""
+    sizes, calls, got, errors = ((500, 500), (128, 128)), 3000, {}, []
+
+    def work(size):
+        try:
+            stream = torch.cuda.Stream()
+            with Cavity(*size, Re=300.0, U=0.1, dtype="f32s", stream=stream) as cav:
+                for k in range(calls):
+                    cav.step(2 + k % 3)
+                got[size] = cav.populations(host=True)
+        except Exception as e:
+            errors.append(f"{size}: {e}")
+
+    threads = [threading.Thread(target=work, args=(s,)) for s in sizes]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors
+    for size in sizes:
+        with Cavity(*size, Re=300.0, U=0.1, dtype="f32s") as cav:
+            cav.step(3 * calls)
+            assert (cav.populations(host=True) == got[size]).all(), size
