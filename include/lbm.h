@@ -139,7 +139,8 @@ int lbm_get_info(const lbm_ctx *ctx, lbm_info *info);
  * take f^eq(rho_f, u_w) + (1 - 1/tau)[f(x_f) - f^eq(rho_f, u_f)] from their inner neighbour
  * x_f.  One fused kernel per step, or per few steps (launch shapes below).  After every step whose
  * global index is a multiple of 100 the library also forms, in FP64, the mass sum rho and the Eq. 6 residual against the velocity
- * field of 100 steps earlier, and samples the probes (lbm_probe).  Asynchronous.
+ * field of 100 steps earlier, and samples the probes (lbm_probe).  Asynchronous.  Plain steps may be
+ * captured into a caller's graph: the replays of an even number of them advance the state.
  * Errors: LBM_EINVAL (n < 0), LBM_ECUDA. */
 int lbm_step(lbm_ctx *ctx, long n);
 

@@ -213,6 +213,7 @@ struct lbm_ctx {
 
     int advance(long long n) {
         int rc = LBM_OK;
+        const bool recording = n > 0 && caller_captures();
         while (n > 0 && !rc) {
             const int s = (int)(step % kInterval), slot = (int)((step / kInterval + 1) & 1);
             const int m = (int)std::min<long long>(n, kInterval - s);
@@ -221,7 +222,7 @@ struct lbm_ctx {
                 if (!chunk[slot][which]) rc = capture(slot == 1 ? 0 : kInterval, kInterval, which, &chunk[slot][which]);
                 if (rc) return rc;
                 exec = chunk[slot][which];
-            } else if (m >= kPartSteps) {
+            } else if (m >= kPartSteps && !recording) {
                 rc = part(s, m, slot, &exec);
                 if (rc) return rc;
             }
@@ -232,8 +233,14 @@ struct lbm_ctx {
                 step += m;
                 n -= m;
             } else {
-                for (int t = 0, taken = 0; t < m; t += taken) {
-                    rc = enqueue(step, m - t, which, stream, &taken);
+                // What a caller captures it replays, so an even number of steps has to end in the buffer it
+                // began in, fused or not: one launch more where the launches do not have the steps' parity.
+                const int plain = std::min(m, kInterval - 1 - s);
+                int left = launches(s, plain);
+                if (recording && ((left ^ plain) & 1)) ++left;
+                for (int t = 0, taken = 0; t < m; t += taken, --left) {
+                    const int most = t < plain && left > 1 ? plain - t - (left - 1) : m - t;
+                    rc = enqueue(step, most, which, stream, &taken);
                     if (rc) return rc;
                     which ^= 1;
                     step += taken;
@@ -244,14 +251,17 @@ struct lbm_ctx {
         return rc;
     }
 
+    // Whether the caller is capturing the context's stream into a graph of its own.
+    bool caller_captures() const {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(stream, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
+        cudaGetLastError();  // the legacy stream while another stream is captured
+        return true;
+    }
+
     // The graph of a part, or null at its first sight (then it is launched directly, as it is into a
     // stream that a caller is capturing).
     int part(int s, int m, int slot, cudaGraphExec_t* exec) {
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-            cudaGetLastError();
-            return LBM_OK;
-        }
         size_t k = 0;
         while (k < parts.size() && !(parts[k].s == s && parts[k].n == m && parts[k].slot == slot && parts[k].from == which)) ++k;
         if (k == parts.size()) {

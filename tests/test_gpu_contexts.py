@@ -7,6 +7,7 @@ import pytest
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
+from paper_2211_05009_gb300 import binding as B  # noqa: E402
 from paper_2211_05009_gb300.cavity import Cavity  # noqa: E402
 
 
@@ -34,3 +35,25 @@ def test_contexts_step_in_two_threads():
         with Cavity(*size, Re=300.0, U=0.1, dtype="f32s") as cav:
             cav.step(3 * calls)
             assert (cav.populations(host=True) == got[size]).all(), size
+
+
+@pytest.mark.parametrize("calls", [(2,), (4,), (12,), (3, 5), (20, 40), (1, 7, 6)])
+@pytest.mark.parametrize("dtype,cfg", [("f32s", 7), ("f32s", 6), ("f16s", 7), ("f64", 5)])
+def test_replays_of_captured_steps_advance(dtype, cfg, calls):
+    """Calls of an even number of steps together, captured once by the caller and replayed."""
+    stream, replays = torch.cuda.Stream(), 5
+    with Cavity(150, 70, Re=300.0, U=0.1, dtype=dtype, stream=stream) as cav, \
+            Cavity(150, 70, Re=300.0, U=0.1, dtype=dtype) as ref:
+        B.lbm_set_launch_config(cav.ctx, cfg)
+        cav.step(7)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            for n in calls:
+                cav.step(n)
+        torch.cuda.synchronize()
+        for _ in range(replays):
+            graph.replay()
+        torch.cuda.synchronize()
+        for _ in range(7 + sum(calls) * replays):
+            ref.step(1)
+        assert torch.equal(cav.populations(), ref.populations())
