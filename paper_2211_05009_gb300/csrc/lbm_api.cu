@@ -187,8 +187,9 @@ struct lbm_ctx {
     }
     // Graph of n steps from global step g0 in buffer `from`.
     int capture(long long g0, int n, int from, cudaGraphExec_t* exec) {
+        const CaptureApart apart;
         cudaGraph_t g = nullptr;
-        int rc = cuda(cudaStreamBeginCapture(cap_stream, cudaStreamCaptureModeThreadLocal),
+        int rc = cuda(cudaStreamBeginCapture(cap_stream, cudaStreamCaptureModeRelaxed),
                       "begin graph capture");
         if (rc) return rc;
         int b = from;

@@ -17,6 +17,17 @@ struct NvtxRange {
     NvtxRange& operator=(const NvtxRange&) = delete;
 };
 
+// For as long as it lives, this thread's captures do not forbid it calls that allocate or wait: a graph
+// captured and instantiated inside a library call would otherwise invalidate a capture that the caller
+// has under way on another stream.
+struct CaptureApart {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    CaptureApart() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~CaptureApart() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    CaptureApart(const CaptureApart&) = delete;
+    CaptureApart& operator=(const CaptureApart&) = delete;
+};
+
 struct StepGeometry {
     int grid_x, grid_y, blocks;
 };

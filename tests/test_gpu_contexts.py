@@ -57,3 +57,30 @@ def test_replays_of_captured_steps_advance(dtype, cfg, calls):
         for _ in range(7 + sum(calls) * replays):
             ref.step(1)
         assert torch.equal(cav.populations(), ref.populations())
+
+
+@pytest.mark.parametrize("cfg", [5, 6, 7])
+def test_steps_beside_a_capture_of_another_stream(cfg):
+    """Calls that capture a part or an interval of their own, launched directly and replayed, while the
+    caller captures something else: both go on."""
+    x = torch.zeros(1000, device="cuda")
+    with Cavity(150, 70, Re=300.0, U=0.1, dtype="f32s", stream=torch.cuda.Stream()) as cav, \
+            Cavity(150, 70, Re=300.0, U=0.1, dtype="f32s") as ref:
+        start = ref.moments()
+        B.lbm_set_launch_config(cav.ctx, cfg)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=torch.cuda.Stream()):
+            x += 1
+            for _ in range(3):
+                cav.set_moments(*start)
+                cav.step(7)
+            cav.step(93)
+            cav.step(100)
+            x += 1
+        graph.replay()
+        ref.set_moments(*start)
+        ref.step(200)
+        torch.cuda.synchronize()
+        assert float(x.sum()) == 2000.0
+        assert torch.equal(cav.populations(), ref.populations())
