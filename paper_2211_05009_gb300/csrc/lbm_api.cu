@@ -75,6 +75,7 @@ struct lbm_ctx {
         cudaGraphExec_t exec;
     };
     std::vector<Part> parts;
+    std::vector<cudaGraphExec_t> retired;  // of parts no longer kept, perhaps still running: until the next wait
     cudaEvent_t ev[2] = {nullptr, nullptr};
 
     ProbeSet probes{};
@@ -160,6 +161,10 @@ struct lbm_ctx {
         for (auto& p : parts)
             if (p.exec) cudaGraphExecDestroy(p.exec);
         parts.clear();
+    }
+    void drop_retired() {
+        for (auto& g : retired) cudaGraphExecDestroy(g);
+        retired.clear();
     }
 
     // Enqueue one launch from global step gstep and buffer `from` on stream st: a checkpoint step by
@@ -268,9 +273,8 @@ struct lbm_ctx {
         if (k == parts.size()) {
             if (parts.size() == kMaxParts) {
                 if (parts.back().exec) {
-                    const int rc = sync();  // it may still be running
-                    if (rc) return rc;
-                    cudaGraphExecDestroy(parts.back().exec);
+                    if (retired.size() == kMaxParts) return LBM_OK;  // none is captured before the caller waits
+                    retired.push_back(parts.back().exec);
                 }
                 parts.pop_back();
             }
@@ -279,8 +283,11 @@ struct lbm_ctx {
         }
         std::rotate(parts.begin(), parts.begin() + k, parts.begin() + k + 1);
         if (!parts[0].exec) {
-            const int rc = capture((slot == 1 ? 0 : kInterval) + s, m, which, &parts[0].exec);
-            if (rc) return rc;
+            if (capture((slot == 1 ? 0 : kInterval) + s, m, which, &parts[0].exec)) {  // no memory for it: directly
+                cudaGetLastError();
+                parts.erase(parts.begin());
+                return LBM_OK;
+            }
         }
         *exec = parts[0].exec;
         return LBM_OK;
@@ -323,7 +330,11 @@ struct lbm_ctx {
         return stage ? LBM_OK : fail(LBM_ENOMEM, fmt("staging buffer of %zu bytes", bytes));
     }
 
-    int sync() { return cuda(cudaStreamSynchronize(stream), "stream synchronize"); }
+    int sync() {
+        const int rc = cuda(cudaStreamSynchronize(stream), "stream synchronize");
+        if (!rc) drop_retired();
+        return rc;
+    }
 };
 
 // ------------------------------------------------------------------ lifetime
@@ -339,6 +350,7 @@ extern "C" void lbm_destroy(lbm_ctx* c) {
     if (!c) return;
     if (c->stream || c->cap_stream) cudaStreamSynchronize(c->stream);
     c->invalidate_graphs();
+    c->drop_retired();
     for (auto& e : c->ev)
         if (e) cudaEventDestroy(e);
     c->dfree(c->buf[0]);
