@@ -56,6 +56,7 @@ struct lbm_ctx {
     void* buf[2] = {nullptr, nullptr};  // populations, ping-pong; current = buf[which]
     int which = 0;
     int sms = 0;  // multiprocessors of the device
+    bool wide = true;  // population buffers take the 16-byte accesses of fused FP32 steps
     void* snap = nullptr;               // [2][ny][pitch] Eq. 6 snapshot (arithmetic type)
     double* partials = nullptr;         // reduction partials
     int npartials = 0;
@@ -128,6 +129,9 @@ struct lbm_ctx {
     }
     FieldArgs cur() const { return field(which); }
 
+    // Plain steps per launch of a shape.
+    int steps_of(int k) const { return wide ? config_steps(dtype, k, nx, ny) : 1; }
+
     StepArgs step_args(int from, int s) const {
         StepArgs a{};
         a.src = buf[from];
@@ -174,7 +178,7 @@ struct lbm_ctx {
         const int s = (int)(gstep % kInterval);
         const bool reduce = s == kInterval - 1;
         const int plain = (int)std::min<long long>(n, kInterval - 1 - s);
-        const int fused = reduce ? 1 : std::min(config_steps(dtype, cfg, nx, ny), plain);
+        const int fused = reduce ? 1 : std::min(steps_of(cfg), plain);
         *taken = fused;
         int rc = fused > 1 ? cuda(launch_fused(dtype, cfg, step_args(from, s), fused, sms, st), "fused step launch")
                            : cuda(launch_step(dtype, cfg, step_args(from, s), reduce, st), "step kernel launch");
@@ -213,7 +217,7 @@ struct lbm_ctx {
     }
     // Launches of n steps from place s of an interval (each one changes the buffer).
     int launches(int s, int n) const {
-        const int f = config_steps(dtype, cfg, nx, ny), plain = std::min(n, kInterval - 1 - s);
+        const int f = steps_of(cfg), plain = std::min(n, kInterval - 1 - s);
         return (plain + f - 1) / f + (s + n == kInterval ? 1 : 0);
     }
 
@@ -418,6 +422,9 @@ extern "C" int lbm_create_ex(int nx, int ny, double tau, double U, lbm_dtype dty
     for (int b = 0; b < 2; ++b) {
         c->buf[b] = c->dalloc(pop_bytes);
         if (!c->buf[b]) return create_fail(c, LBM_ENOMEM, fmt("population buffer of %zu bytes", pop_bytes));
+        // an FP32 lane loads 2 nodes in the row step, 4 in the march and in a tile's copy: memory that a
+        // caller's allocator aligns to 8 bytes is taken, by the row step
+        if (storage_bytes(c->dtype) == 4 && ((uintptr_t)c->buf[b] & 15)) c->wide = false;
     }
     c->snap = c->dalloc(2ull * (size_t)c->plane * arith_bytes(c->dtype));
     c->npartials = 3 * max_blocks > 4096 ? 3 * max_blocks : 4096;
@@ -533,8 +540,9 @@ extern "C" int lbm_autotune(lbm_ctx* c, int steps_per_trial, int* best, double* 
     float plain[kStepConfigs], red[kStepConfigs];
     for (int k = 0; k < kStepConfigs; ++k) plain[k] = red[k] = 1e30f;
     // `n` steps of shape k (steps 0..97 of a checkpoint interval never reduce)
+    auto steps_of = [&](int k) { return std::min(c->steps_of(k), t->steps_of(k)); };
     auto plain_steps = [&](int k, int n) {
-        const int f = config_steps(t->dtype, k, t->nx, t->ny);
+        const int f = steps_of(k);
         for (int s = 0, from = 0; s < n && !rc; s += f, from ^= 1) {
             const int m = std::min(f, n - s);
             rc = m > 1 ? c->cuda(launch_fused(t->dtype, k, t->step_args(from, s % 90), m, t->sms, t->stream), "autotune launch")
@@ -543,7 +551,7 @@ extern "C" int lbm_autotune(lbm_ctx* c, int steps_per_trial, int* best, double* 
     };
     for (int round = 0; round < 3 && !rc; ++round) {
         for (int k = 0; k < kStepConfigs && !rc; ++k) {
-            if (k >= kRowConfigs && config_steps(t->dtype, k, t->nx, t->ny) == 1) continue;  // the default row shape again
+            if (k >= kRowConfigs && steps_of(k) == 1) continue;  // the default row shape again
             if (round > 0 && plain[k] > 1.25f * *std::min_element(plain, plain + kStepConfigs)) continue;  // out of the race
             if (round == 0) plain_steps(k, steps_per_trial);  // warm-up
             if (!rc) rc = c->cuda(cudaEventRecord(e0, t->stream), "event record");
