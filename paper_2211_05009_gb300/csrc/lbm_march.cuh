@@ -312,7 +312,7 @@ __device__ __forceinline__ void march(const S* __restrict__ src, S* __restrict__
                 f32x2 g[9];
 #pragma unroll
                 for (int j = 0; j < 9; ++j) g[j] = f[j][k];
-                moments9<f32x2>(g, one_ref, drho[k], rho[k], ux[k], uy[k]);
+                moments9(g, one_ref, drho[k], rho[k], ux[k], uy[k]);
             }
             const bool special = edge | top | sampled | (y == 1);
             if (special) {
@@ -348,7 +348,7 @@ __device__ __forceinline__ void march(const S* __restrict__ src, S* __restrict__
                     f32x2 g[9], out[9];
 #pragma unroll
                     for (int j = 0; j < 9; ++j) g[j] = f[j][k];
-                    collide9<kMomentum<S>, f32x2>(g, drho[k], rho[k], ux[k], uy[k], om, out);
+                    collide9<kMomentum<S>>(g, drho[k], rho[k], ux[k], uy[k], om, out);
                     float wo[2][9];
                     bool is[2];
 #pragma unroll
@@ -369,7 +369,7 @@ __device__ __forceinline__ void march(const S* __restrict__ src, S* __restrict__
                     f32x2 g[9], out[9];
 #pragma unroll
                     for (int j = 0; j < 9; ++j) g[j] = f[j][k];
-                    collide9<kMomentum<S>, f32x2>(g, drho[k], rho[k], ux[k], uy[k], om, out);
+                    collide9<kMomentum<S>>(g, drho[k], rho[k], ux[k], uy[k], om, out);
 #pragma unroll
                     for (int j = 0; j < 9; ++j) f[j][k] = out[j];
                 }

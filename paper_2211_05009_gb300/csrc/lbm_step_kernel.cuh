@@ -514,8 +514,11 @@ __device__ __forceinline__ void lid_shift(C rho, C W, C (&out)[9]) {
 // (4e-6 of the velocity after 250 steps of a 500 x 1000 cavity in LBM_F32, 5e-4 in binary16), so
 // their results are that rounding's noise.  They keep the arithmetic that forms every direction by
 // itself, and with it their results bit for bit; the rounding of each operation is spelled out here
-// too, scalar and packed.  Signs are placed so that nothing is negated by itself (rounding to
-// nearest is symmetric).
+// too, in two spellings that round alike (rounding to nearest is symmetric).  Packed nodes (march,
+// tiles): a negation is an instruction, so signs are placed where nothing is negated by itself.
+// Single nodes (row step): operands take a sign for nothing, and the plain signs cost one product less
+// and let the compiler order the chain better (us a step, packed spelling / this one: LBM_F32 300^2 4.3 /
+// 3.8, 1000^2 9.9 / 9.4, binary16 1200^2 11.9 / 11.6, 1500^2 15.9 / 15.4).
 template <typename C>
 struct Omega {
     C om, nom;        // omega, -omega
@@ -527,23 +530,42 @@ __device__ __forceinline__ Omega<C> make_omega(float w) {
 }
 
 // Moments of a node (Eq. 3).
-template <typename C>
-__device__ __forceinline__ void moments9(const C (&g)[9], C one_ref, C& drho, C& rho, C& ux, C& uy) {
+__device__ __forceinline__ void moments9(const f32x2 (&g)[9], f32x2 one_ref, f32x2& drho, f32x2& rho, f32x2& ux, f32x2& uy) {
     drho = radd(radd(radd(radd(g[0], g[1]), radd(g[2], g[3])), radd(radd(g[4], g[5]), radd(g[6], g[7]))), g[8]);
     rho = radd(one_ref, drho);
-    const C inv = nrcp<C>(rho);  // -1/rho, against -j
+    const f32x2 inv = nrcp<f32x2>(rho);  // -1/rho, against -j
     ux = rmul(radd(radd(rsub(g[3], g[1]), rsub(g[6], g[5])), rsub(g[7], g[8])), inv);
     uy = rmul(radd(rsub(rsub(g[4], g[2]), radd(g[5], g[6])), radd(g[7], g[8])), inv);
 }
+__device__ __forceinline__ void moments9(const float (&g)[9], float one_ref, float& drho, float& rho, float& ux, float& uy) {
+    drho = radd(radd(radd(radd(g[0], g[1]), radd(g[2], g[3])), radd(radd(g[4], g[5]), radd(g[6], g[7]))), g[8]);
+    rho = radd(one_ref, drho);
+    const float jx = radd(radd(rsub(g[1], g[3]), rsub(g[5], g[6])), rsub(g[8], g[7]));
+    const float jy = rsub(radd(rsub(g[2], g[4]), radd(g[5], g[6])), radd(g[7], g[8]));
+    const float inv = -nrcp<float>(rho);
+    ux = rmul(jx, inv);
+    uy = rmul(jy, inv);
+}
 
 // t_j with g^eq_j = w_j t_j, t_j = drho + rho A_j, A_j = 3 c.u + 9/2 (c.u)^2 - 3/2 u.u (Eq. 2).
-template <typename C>
-__device__ __forceinline__ void eq_terms(C drho, C rho, C ux, C uy, C (&t)[9]) {
-    const C nusq = rmul(C(-1.5), rfma(ux, ux, rmul(uy, uy)));
+__device__ __forceinline__ void eq_terms(f32x2 drho, f32x2 rho, f32x2 ux, f32x2 uy, f32x2 (&t)[9]) {
+    const f32x2 nusq = rmul(f32x2(-1.5), rfma(ux, ux, rmul(uy, uy)));
     t[0] = rfma(rho, nusq, drho);
-    auto pair = [&](int a, int b, C cu) {
-        t[a] = rfma(rho, rfma(cu, rfma(C(4.5), cu, C(3.0)), nusq), drho);
-        t[b] = rfma(rho, rfma(cu, rfma(C(4.5), cu, C(-3.0)), nusq), drho);
+    auto pair = [&](int a, int b, f32x2 cu) {
+        t[a] = rfma(rho, rfma(cu, rfma(f32x2(4.5), cu, f32x2(3.0)), nusq), drho);
+        t[b] = rfma(rho, rfma(cu, rfma(f32x2(4.5), cu, f32x2(-3.0)), nusq), drho);
+    };
+    pair(1, 3, ux);
+    pair(2, 4, uy);
+    pair(5, 7, radd(ux, uy));
+    pair(8, 6, rsub(ux, uy));
+}
+__device__ __forceinline__ void eq_terms(float drho, float rho, float ux, float uy, float (&t)[9]) {
+    const float usq = rmul(1.5f, rfma(ux, ux, rmul(uy, uy)));
+    t[0] = rfma(-rho, usq, drho);
+    auto pair = [&](int a, int b, float cu) {
+        t[a] = rfma(rho, rfma(cu, rfma(4.5f, cu, 3.0f), -usq), drho);
+        t[b] = rfma(rho, rfma(-cu, rfma(4.5f, -cu, 3.0f), -usq), drho);
     };
     pair(1, 3, ux);
     pair(2, 4, uy);
@@ -555,11 +577,44 @@ __device__ __forceinline__ void eq_terms(C drho, C rho, C ux, C uy, C (&t)[9]) {
 __device__ __forceinline__ void wall9(const float (&g)[9], float drho, float rho, float ux, float uy, float W, float omega,
                                       float (&out)[9]) {
     const float keep = rsub(1.0f, omega);  // 1 - 1/tau
-    float t[9], tw[9];
-    eq_terms<float>(drho, rho, ux, uy, t);
-    eq_terms<float>(drho, rho, W, 0.0f, tw);
+    float t[9];
+    eq_terms(drho, rho, ux, uy, t);
+    // the wall's own terms, u = (W, 0): one each for c_x = 0, 1, -1
+    const float usq = rmul(1.5f, rmul(W, W));
+    const float w0 = rfma(-rho, usq, drho);
+    const float wp = rfma(rho, rfma(W, rfma(4.5f, W, 3.0f), -usq), drho), wm = rfma(rho, rfma(-W, rfma(4.5f, -W, 3.0f), -usq), drho);
 #pragma unroll
-    for (int j = 0; j < 9; ++j) out[j] = rfma(float(wd(j)), tw[j], rmul(keep, rfma(-float(wd(j)), t[j], g[j])));
+    for (int j = 0; j < 9; ++j)
+        out[j] = rfma(float(wd(j)), cx(j) == 0 ? w0 : (cx(j) > 0 ? wp : wm), rmul(keep, rfma(-float(wd(j)), t[j], g[j])));
+}
+
+// The same closure with its contractions left to the compiler, which makes the ones spelled out above (the
+// launch shapes' bitwise tests hold the tiles' walls against these).  For the row step in binary16 and
+// bfloat16 alone: at its 64 registers the wall path decides which values spill, and of five spellings of it
+// only this one leaves the interior path alone (binary16, us a step, this / the others: 1200^2 11.6 / 11.85
+// .. 12.1, 2048^2 26.4 / 26.5 .. 28.1).
+__device__ __forceinline__ void wall9_contracted(const float (&g)[9], float drho, float rho, float ux, float uy, float W,
+                                                 float omega, float (&out)[9]) {
+    auto equilibrium = [&](float vx, float vy, float (&e)[9]) {
+        const float usq = 1.5f * (vx * vx + vy * vy);
+        const float up = vx + vy, um = vx - vy;
+        auto term = [&](float cu) { return drho + rho * (cu * (3.0f + 4.5f * cu) - usq); };
+        e[0] = float(wd(0)) * (drho - rho * usq);
+        e[1] = float(wd(1)) * term(vx);
+        e[2] = float(wd(2)) * term(vy);
+        e[3] = float(wd(3)) * term(-vx);
+        e[4] = float(wd(4)) * term(-vy);
+        e[5] = float(wd(5)) * term(up);
+        e[6] = float(wd(6)) * term(-um);
+        e[7] = float(wd(7)) * term(-up);
+        e[8] = float(wd(8)) * term(um);
+    };
+    const float keep = 1.0f - omega;
+    float e[9], ew[9];
+    equilibrium(ux, uy, e);
+    equilibrium(W, 0.0f, ew);
+#pragma unroll
+    for (int j = 0; j < 9; ++j) out[j] = ew[j] + keep * (g[j] - e[j]);
 }
 
 // Collision of a fluid node.  MOMENTUM: BGK as an increment d_j = (f^eq_j - f_j)/tau added to the
@@ -568,11 +623,13 @@ __device__ __forceinline__ void wall9(const float (&g)[9], float drho, float rho
 // LBM_Q16S rounds its stores to nearest, which passes such a bias on unchanged on average, so it
 // needs the correction as much as LBM_F32 does.  binary16 / bfloat16 swamp the bias and take the
 // form per opposite pair, f*_j = g_j + omega (g^eq_j - g_j) with A = c2 +- 3 c.u.
-template <bool MOMENTUM, typename C>
-__device__ __forceinline__ void collide9(const C (&g)[9], C drho, C rho, C ux, C uy, const Omega<C>& k, C (&out)[9]) {
+template <bool MOMENTUM>
+__device__ __forceinline__ void collide9(const f32x2 (&g)[9], f32x2 drho, f32x2 rho, f32x2 ux, f32x2 uy, const Omega<f32x2>& k,
+                                         f32x2 (&out)[9]) {
+    using C = f32x2;
     if constexpr (MOMENTUM) {
         C t[9], n[9];
-        eq_terms<C>(drho, rho, ux, uy, t);
+        eq_terms(drho, rho, ux, uy, t);
 #pragma unroll
         for (int j = 0; j < 9; ++j) n[j] = rfma(C(-wd(j)), t[j], g[j]);  // -d_j / omega
         const C d3 = rmul(k.nom, n[3]), d4 = rmul(k.nom, n[4]), d6 = rmul(k.nom, n[6]), d7 = rmul(k.nom, n[7]);
@@ -596,6 +653,41 @@ __device__ __forceinline__ void collide9(const C (&g)[9], C drho, C rho, C ux, C
             const C base = rfma(rho, rfma(rmul(C(4.5), cu), cu, nusq), drho);
             out[a] = rfma(ow, rfma(r3, cu, base), rfma(k.nom, g[a], g[a]));
             out[b] = rfma(ow, rfma(n3, cu, base), rfma(k.nom, g[b], g[b]));
+        };
+        pair(1, 3, ux, k.ow1);
+        pair(2, 4, uy, k.ow1);
+        pair(5, 7, radd(ux, uy), k.ow5);
+        pair(8, 6, rsub(ux, uy), k.ow5);
+    }
+}
+template <bool MOMENTUM>
+__device__ __forceinline__ void collide9(const float (&g)[9], float drho, float rho, float ux, float uy, const Omega<float>& k,
+                                         float (&out)[9]) {
+    if constexpr (MOMENTUM) {
+        float t[9], n[9];
+        eq_terms(drho, rho, ux, uy, t);
+#pragma unroll
+        for (int j = 0; j < 9; ++j) n[j] = rfma(float(wd(j)), t[j], -g[j]);  // d_j / omega
+        const float d3 = rmul(k.om, n[3]), d4 = rmul(k.om, n[4]), d6 = rmul(k.om, n[6]), d7 = rmul(k.om, n[7]);
+        const float mx = radd(radd(rfma(k.om, n[1], -d3), rfma(k.om, n[5], -d6)), rfma(k.om, n[8], -d7));
+        const float my = rsub(radd(rfma(k.om, n[2], -d4), rfma(k.om, n[5], d6)), rfma(k.om, n[8], d7));
+        out[0] = rfma(k.om, n[0], g[0]);
+        out[1] = radd(g[1], rfma(k.om, n[1], rmul(-0.5f, mx)));
+        out[3] = radd(g[3], rfma(0.5f, mx, d3));
+        out[2] = radd(g[2], rfma(k.om, n[2], rmul(-0.5f, my)));
+        out[4] = radd(g[4], rfma(0.5f, my, d4));
+        out[5] = rfma(k.om, n[5], g[5]);
+        out[8] = rfma(k.om, n[8], g[8]);
+        out[6] = radd(g[6], d6);
+        out[7] = radd(g[7], d7);
+    } else {
+        const float usq = rmul(1.5f, rfma(ux, ux, rmul(uy, uy)));
+        const float r3 = rmul(3.0f, rho);
+        out[0] = rfma(k.ow0, rfma(-rho, usq, drho), rfma(-k.om, g[0], g[0]));
+        auto pair = [&](int a, int b, float cu, float ow) {
+            const float base = rfma(rho, rfma(rmul(4.5f, cu), cu, -usq), drho);
+            out[a] = rfma(ow, rfma(r3, cu, base), rfma(-k.om, g[a], g[a]));
+            out[b] = rfma(ow, rfma(-r3, cu, base), rfma(-k.om, g[b], g[b]));
         };
         pair(1, 3, ux, k.ow1);
         pair(2, 4, uy, k.ow1);
@@ -752,7 +844,7 @@ __device__ __forceinline__ void step_row(const S* __restrict__ src, S* __restric
         if constexpr (F64) vel = wall ? rx.wall : rx.one;
         if constexpr (F64 && EDGE) collide<C, true>(g, one_ref, rx, out, drho, rho, ux, uy, vel);
         else if constexpr (PAIRS) collide<C>(g, one_ref, rx, out, drho, rho, ux, uy);
-        else moments9<C>(g, one_ref, drho, rho, ux, uy);
+        else moments9(g, one_ref, drho, rho, ux, uy);
         C uox = ux, uoy = uy;
         if (wall) {
             const bool lid = (y == ny - 1) && (cv.corner_moving || (x > 0 && x < nx - 1));
@@ -761,9 +853,10 @@ __device__ __forceinline__ void step_row(const S* __restrict__ src, S* __restric
             if constexpr (F64) {
                 if (lid) lid_shift<C>(rho, uox, out);
             } else if constexpr (PAIRS) wall_shift<C>(rho, ux, uy, uox, out);
-            else wall9(g, drho, rho, ux, uy, uox, cv.omega, out);
+            else if constexpr (kMomentum<S>) wall9(g, drho, rho, ux, uy, uox, cv.omega, out);
+            else wall9_contracted(g, drho, rho, ux, uy, uox, cv.omega, out);
         } else if constexpr (!PAIRS) {
-            collide9<kMomentum<S>, C>(g, drho, rho, ux, uy, om, out);
+            collide9<kMomentum<S>>(g, drho, rho, ux, uy, om, out);
         }
 #pragma unroll
         for (int j = 0; j < 9; ++j) f[j][i] = out[j];

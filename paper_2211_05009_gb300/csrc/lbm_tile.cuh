@@ -128,8 +128,8 @@ __global__ void __launch_bounds__(32 * kTileWarps, 2) k_tile(const TileArgs m) {
             if constexpr (PAIRS) {
                 collide<f32x2>(gp, f32x2(1.0f), rx, op, d, r, u, v);
             } else {
-                moments9<f32x2>(gp, f32x2(one_ref), d, r, u, v);
-                collide9<kMomentum<S>, f32x2>(gp, d, r, u, v, om, op);
+                moments9(gp, f32x2(one_ref), d, r, u, v);
+                collide9<kMomentum<S>>(gp, d, r, u, v, om, op);
             }
 #pragma unroll
             for (int j = 0; j < 9; ++j) {
