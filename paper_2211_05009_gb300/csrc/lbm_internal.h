@@ -62,6 +62,8 @@ inline int default_row_config(int dtype) {
 }
 // Row shape of the single steps of a shape.
 inline int row_config(int dtype, int cfg) { return cfg < kRowConfigs ? cfg : default_row_config(dtype); }
+// Columns that the march's strips of an nx-wide grid own together (lbm_march.cu).
+int march_columns(int nx);
 // Shape of a new context; lbm_autotune measures all of them on the caller's size.
 int default_step_config(int dtype, int nx, int ny);
 

@@ -39,6 +39,11 @@ cudaError_t launch_march_s(const StepArgs& a, int steps, int sms, cudaStream_t s
 }
 }  // namespace
 
+int march_columns(int nx) {
+    using G = StripGeometry<kV, kMarchSteps>;
+    return G::strips(nx) * G::kWidth;
+}
+
 cudaError_t launch_march(int dtype, const StepArgs& a, int steps, int sms, cudaStream_t st) {
     if (steps < 1 || steps > kMarchSteps) return cudaErrorInvalidValue;
     switch (dtype) {

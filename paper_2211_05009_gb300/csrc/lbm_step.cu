@@ -20,7 +20,7 @@ struct Shape {
 };
 // must match launch_step_cfg in lbm_step_kernel.cuh: FP64, FP32 storage, 16-bit storage
 constexpr Shape kShapes[3][kRowConfigs] = {{{1, 2, 2}, {1, 2, 4}, {1, 1, 4}, {1, 4, 1}, {1, 2, 1}, {1, 1, 1}},
-                                           {{2, 2, 2}, {2, 1, 4}, {1, 1, 4}, {2, 4, 1}, {2, 2, 4}, {1, 1, 1}},
+                                           {{2, 2, 2}, {2, 1, 4}, {1, 1, 4}, {2, 4, 1}, {2, 2, 4}, {2, 2, 2}},
                                            {{4, 2, 2}, {4, 1, 4}, {4, 2, 2}, {4, 4, 1}, {4, 2, 4}, {4, 4, 2}}};
 }  // namespace
 
@@ -49,20 +49,25 @@ int default_step_config(int dtype, int nx, int ny) {
     // 11.2 / 10.0, 500x1000 59.5 / 56.6, 700^2 55.8 / 54.6, 2048^2 435.5 / 435.3).
     if (dtype == 0) return 5;
     // Other types: tiles in shared memory while the grid is small enough that a step is mostly launch and
-    // latency (us a step, best other shape / tiles: f32s 250^2 1.9 / 1.4, 500^2 3.3 / 2.8, 900x1000 7.8 /
-    // 7.6, 950x1000 7.8 / 7.9; f32 128^2 1.7 / 1.3, 250^2 2.0 / 1.8, 350^2 2.5 / 3.1; q16s 500^2 5.9 / 5.0,
-    // 1050x1000 16.7 / 16.0, 1200x1000 17.8 / 17.7; f16s 500x1000 7.1 / 5.3, 1200x1000 10.3 / 10.2, 1200^2
-    // 11.7 / 12.2).
+    // latency (us a step, best other shape / tiles: f32s 250^2 1.9 / 1.4, 500^2 3.4 / 2.9, 900^2 7.4 / 7.0,
+    // 1000^2 8.0 / 8.4; f32 128^2 1.8 / 1.3, 250^2 2.1 / 1.7, 300^2 2.2 / 2.6; q16s 500^2 5.9 / 5.0, 1050x1000
+    // 16.7 / 16.0, 1200x1000 17.8 / 17.7; f16s 500x1000 7.1 / 5.3, 1200x1000 10.3 / 10.2, 1200^2 11.6 / 12.0).
     if (n < (dtype == 1 ? 90000 : (dtype == 2 ? 950000 : 1200000))) return kTileConfig;
-    // f16s 2048^2 25.0 with shape 2, 26.5 with 0; 4096^2 99.5, 94.9
+    // f16s 2048^2 26.5 with shape 2, 27.5 with 0; 4096^2 100.3, 95.6
     if (dtype >= 3) return dtype == kDtypeQ16S || n < 8000000 ? 2 : 0;
-    // Steps fused in the march once the two population buffers outgrow the L2 cache; below that the
-    // rows that neighbouring segments compute twice cost more than the saved launches.  us a step,
-    // others against fused: f32s 950x1000 7.9 / 7.8, 1000x1050 8.9 / 8.6, 1500^2 26.1 / 13.8; f32 1100^2
-    // 11.8 / 12.9, 1500^2 26.2 / 19.3.
-    if (dtype == 2 || n >= 1600000) return kMarchConfig;
-    // f32, shape 0 / 2: 500x1000 6.4 / 5.7, 900x1000 9.3 / 8.8, 1000x1100 10.6 / 10.5, 1100^2 11.8 / 12.0
-    return n < 1150000 ? 2 : 0;
+    // f32, shapes 0 / 2: 500x1000 6.2 / 5.8, 900^2 8.3 / 8.1, 1000^2 9.4 / 9.6
+    if (dtype == 1 && n < 950000) return 2;
+    // Steps fused in the march: f32s from there on, f32 once the two population buffers outgrow the L2 cache
+    // (below that the rows that neighbouring segments compute twice cost more than the saved launches).  Where a
+    // strip's 120 columns are filled to less than 1 / 1.4 the tiles' 24 are the better cut.  us a step, march /
+    // tiles / best row shape, columns filled: f32s 1200^2 (1.0) 10.3 / 13.5 / 12.9, 361x5000 (1 / 1.33) 14.6 / 17.8
+    // / 21.6, 361x3000 10.5 / 9.9 / 10.0, 160x8000 (1 / 1.5) 14.8 / 12.7 / 13.1, 121x20000 (1 / 1.98) 27.2 / 24.9 /
+    // 30.9; f32 1500x1200 16.4 / 20.1 / 18.4, 361x5000 21.2 / 21.4 / 21.5, 121x20000 41.6 / 31.0 / 31.5.
+    const int filled = march_columns(nx);
+    if (dtype == 2 || n >= 1600000) return 7ll * nx >= 5ll * filled ? kMarchConfig : kTileConfig;
+    // f32 between: loads that leave L1 alone, shapes 0 / 5: 1000^2 9.4 / 9.4, 1150x1100 11.5 / 11.1, 1200^2 15.2 / 13.4,
+    // 1300x1200 17.6 / 15.5 (march 14.9); a row that fills little of a warp's 64 nodes takes tiles (20x60000 55.6, 19.6)
+    return nx < 40 ? kTileConfig : 5;
 }
 
 StepGeometry step_geometry(int dtype, int cfg, int nx, int ny) {

@@ -1007,7 +1007,7 @@ template <typename S, bool SHIFTED>
 static cudaError_t launch_step_cfg(int cfg, const StepArgs& a, bool reduce, cudaStream_t st) {
     // nodes per lane: 1 for FP64 (default_step_config), 2 for FP32 storage (8-byte vectors; the smaller
     // register footprint buys more resident warps, measured faster than 4), 4 for 16-bit storage; 1 in
-    // the FP32 shapes for small grids, which spread the nodes over as many warps as there are
+    // the FP32 shape for small grids, which spreads the nodes over as many warps as there are
     if constexpr (sizeof(S) == 8) {
         switch (cfg) {
             case 0: return launch_step_shape<S, SHIFTED, 1, 2, 2, 0>(a, reduce, st);
@@ -1027,7 +1027,7 @@ static cudaError_t launch_step_cfg(int cfg, const StepArgs& a, bool reduce, cuda
             case 2: return launch_step_shape<S, SHIFTED, WIDE ? 1 : V, WIDE ? 1 : 2, WIDE ? 4 : 2, WIDE ? 0 : 1>(a, reduce, st);
             case 3: return launch_step_shape<S, SHIFTED, V, 4, 1, 0>(a, reduce, st);
             case 4: return launch_step_shape<S, SHIFTED, V, 2, 4, 0>(a, reduce, st);
-            case 5: return launch_step_shape<S, SHIFTED, WIDE ? 1 : V, WIDE ? 1 : 4, WIDE ? 1 : 2, WIDE ? 0 : 1>(a, reduce, st);
+            case 5: return launch_step_shape<S, SHIFTED, V, WIDE ? 2 : 4, 2, 1>(a, reduce, st);
             default: return cudaErrorInvalidValue;
         }
     }
