@@ -367,6 +367,10 @@ int lbm_batch_autotune(lbm_batch *b, int steps, int *chosen, float *ms);
 int lbm_batch_launch_info(lbm_batch *b, int *shape, int *rows_per_item, int *blocks,
                           long *graph_launches);
 
+/* Plain steps that the batch takes per pass over memory with the cavities active now: 3 where an FP32 batch
+ * fuses them, else 1 (also for NULL). */
+int lbm_batch_steps_per_pass(lbm_batch *b);
+
 /* Limit of each grid-barrier wait in seconds (default 2).  absent_block >= 0 makes that block of
  * the next launch leave before its first barrier -- a fault-injection hook for testing the
  * timeout path (the other blocks' waits run out and the call returns LBM_ETIMEOUT). */

@@ -96,6 +96,7 @@ _SIGS = [
     ("lbm_batch_set_shape", _I, [_P, _I]),
     ("lbm_batch_autotune", _I, [_P, _I, _P, _P]),
     ("lbm_batch_launch_info", _I, [_P, _P, _P, _P, _P]),
+    ("lbm_batch_steps_per_pass", _I, [_P]),
     ("lbm_net_create", _I, [_I, ctypes.c_ulonglong, ctypes.POINTER(_P)]),
     ("lbm_net_destroy", None, [_P]),
     ("lbm_net_last_error", ctypes.c_char_p, [_P]),
@@ -424,6 +425,10 @@ def lbm_batch_launch_info(b):
     _bcheck(b, library().lbm_batch_launch_info(b, ctypes.byref(sh), ctypes.byref(rows), ctypes.byref(blocks),
                                                ctypes.byref(gl)))
     return sh.value, rows.value, blocks.value, gl.value
+
+
+def lbm_batch_steps_per_pass(b) -> int:
+    return library().lbm_batch_steps_per_pass(b)
 
 
 # ------------------------------------------------------------------ learned warm start

@@ -630,14 +630,19 @@ struct lbm_batch {
     }
 
     // Whether plain steps run fused: FP32 storage while every warp has enough rows that the few a
-    // segment computes twice stay cheap.  Follows the active list as of the last pull_state.
+    // segment computes twice stay cheap.  LBM_F32, whose fused step takes 0.76 of a row step's time a strip,
+    // not where the strips of 120 columns are more than 4/3 of the row step's of 128 (100 cavities 121 wide: 58.6
+    // us a step fused, 45.9 by rows; 45 of 500: 153, 160); LBM_F32S takes 0.44 of it and fuses at twice the strips
+    // (35.2, 47.1).  Follows the active list as of the last pull_state.
     bool fuses() const {
         if (march_blocks <= 0 || fuse_slower) return false;
-        long long rows = 0;
+        long long rows = 0, single = 0;
         for (int k = 0; k < h_state->n_active; ++k) {
             const BatchCav& c = cavs[h_state->active[k]];
             rows += (long long)BatchStrips::strips(c.nx) * c.ny;
+            single += (long long)c.strips * c.ny;
         }
+        if (dtype == 1 && 3 * rows > 4 * single) return false;
         return rows >= (long long)kBatchFuseRows * march_blocks * (kBatchThreads / 32);
     }
     // Enqueue a.nsteps plain steps.
@@ -1200,6 +1205,8 @@ extern "C" int lbm_batch_launch_info(lbm_batch* b, int* shape, int* rows_per_ite
     if (graph_launches) *graph_launches = (long)b->graph_launches;
     return b->graph_broken ? b->fail(LBM_ECUDA, b->err) : LBM_OK;
 }
+
+extern "C" int lbm_batch_steps_per_pass(lbm_batch* b) { return b && b->fuses() ? kBatchFuse : 1; }
 
 extern "C" int lbm_batch_set_barrier_limit(lbm_batch* b, double seconds, int absent_block) {
     if (!b || !(seconds > 0)) return LBM_EINVAL;
