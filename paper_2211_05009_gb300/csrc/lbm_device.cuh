@@ -11,6 +11,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cmath>
+
 namespace lbm {
 
 // D2Q9 velocity set and weights, Sec. 2.1 (after Eq. 2), c = 1 (Sec. 3).
@@ -154,16 +156,27 @@ struct Relax<double> {
     double c15, cm3;     // 1.5, -3
     double wall;         // (omega - 1)/omega
 };
+// The parts of omega add up to it without rounding: 2 m1 + 4 o12 = omega, so that a collision keeps the
+// momentum, and nhalf + 4 ow1 + 4 ow5 = omega, so that it keeps the mass.  Each rounded to its own nearest,
+// they miss omega by up to a unit in its last place, the same way every step: of the FP64 velocity error over
+// 50 .. 200 steps of 41 cavities up to 200 wide, 1.7e-15 with them and 2.0e-16 so (geometric means against
+// extended precision; 1.9e-15 with the equilibrium formed per direction).  For that they lie on a grid of
+// a quarter unit in omega's last place, of which four make a whole.
 inline Relax<double> relax_f64(double omega) {
+    int e;
+    const double m = std::frexp(omega, &e), grid = 0x1p-55;  // omega = m 2^e, 1/2 <= m < 1
+    auto on_grid = [&](double v) { return std::nearbyint(v / grid) * grid; };
+    auto scaled = [&](double v) { return std::ldexp(v, e); };
+    const double ow1 = on_grid(m / 9.0), ow5 = on_grid(m / 36.0), o12 = on_grid(m / 12.0);
     Relax<double> k;
-    k.ow1 = omega * (1.0 / 9.0);
-    k.ow5 = omega * (1.0 / 36.0);
-    k.w4 = k.ow1 * -4.5;
-    k.w9 = k.ow5 * -9.0;
+    k.ow1 = scaled(ow1);
+    k.ow5 = scaled(ow5);
+    k.w4 = -0.5 * omega;
+    k.w9 = -0.25 * omega;
     k.khalf = 1.0 - omega;
-    k.nhalf = omega * (4.0 / 9.0);
-    k.o12 = omega * (1.0 / 12.0);
-    k.m1 = k.ow1 * 3.0;
+    k.nhalf = scaled(m - 4.0 * (ow1 + ow5));
+    k.o12 = scaled(o12);
+    k.m1 = scaled(0.5 * (m - 4.0 * o12));
     k.one = 1.0;
     k.nzero = -0.0;
     k.c15 = 1.5;
