@@ -303,10 +303,10 @@ template <> __device__ __forceinline__ f32x2 nrcp<f32x2>(f32x2 v) {
     const f32x2 r(r0, r1);
     return rfma(r, rfma(v, r, f32x2(1.0f)), r);
 }
-// FP64: hardware estimate of 1/v (relative error below 2^-20) refined by one third-order step of
-// Householder's family, r (1 + e + e^2) with e = 1 - v r: the error e^3 is below 2^-60, so three
-// FP64 operations give 1/v to the last bit or the one beside it.  Densities are near 1 here; an
-// infinity or NaN comes out as NaN, which the checkpoint reports.  `one` is 1 in a register.
+// FP64: hardware estimate of 1/v (20 leading bits in, 20 out: relative error within 2^-19) refined by one
+// third-order step of Householder's family, r (1 + e + e^2) with e = 1 - v r: the error e^3 is within
+// 2^-57, so three FP64 operations give 1/v to the nearest value or the one beside it.  Densities are near 1
+// here; an infinity or NaN comes out as NaN, which the checkpoint reports.  `one` is 1 in a register.
 __device__ __forceinline__ double nrcp(double v, double one) {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(v));
