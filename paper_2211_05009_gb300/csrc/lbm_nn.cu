@@ -590,9 +590,9 @@ void drop_graphs(lbm_net* n) {
     n->graphs.clear();
 }
 
-// Lays the tensors of an H x W sample out in the arena, which is one allocation that only grows: a
-// mini-batch of uneven heights otherwise freed and allocated some 80 buffers per sample (half of the
-// time of a training step).
+// Lays the tensors of an H x W sample out in the arena, one allocation that is kept while a sample needs
+// between an eighth of it and all of it: a mini-batch of uneven heights otherwise freed and allocated some
+// 80 buffers per sample (half of the time of a training step).
 int ensure_buffers(lbm_net* n, int H, int W) {
     if (n->H == H && n->W == W) return LBM_OK;
     Graph g = make_graph(n->ch);
@@ -626,7 +626,7 @@ int ensure_buffers(lbm_net* n, int H, int W) {
         for (auto& p : n->cl) p = (__nv_bfloat16*)take(cl * 2);
         n->dz = (float*)take(maxt * 4);
         n->dzq = (__nv_bfloat16*)take(maxt * 2);
-        if (pass == 0 && off > n->arena_bytes) {
+        if (pass == 0 && (off > n->arena_bytes || off < n->arena_bytes / 8)) {
             cudaStreamSynchronize(n->stream);
             drop_graphs(n);
             cudaFree(n->arena);
