@@ -1,8 +1,8 @@
 // lbm_march.cuh -- T time steps of the D2Q9 cavity in one pass over memory (FP32 arithmetic).
 //
 // 2048^2 LBM_F32S, T = 4: 21.8 us a step (192 GLUPS) against 46.6 (90) of the row step, which HBM
-// bounds at 94; 4096^2 76 against 175 us; LBM_F32 2048^2 31.3 against 46.6.  What bounds it now is the FP32 pipe: 61 packed operations
-// a node, 15 % more of them for rows and 7 % for columns computed twice, take two thirds of the time,
+// bounds at 94; 4096^2 76 against 175 us; LBM_F32 2048^2 30.9 against 46.6.  What bounds it now is the FP32
+// pipe: 61 packed operations a node, 15 % more of them for rows and 7 % for columns computed twice, take two thirds of the time,
 // register moves that pairs need most of the rest (336 instructions per 128 nodes and step).
 //
 // A step of its own reads and writes every population once (18 values a node), which is what bounds
@@ -33,40 +33,29 @@
 
 namespace lbm {
 
-// V populations of one direction as V/2 pairs (nodes k, k + V/2): `Mem` is their layout in memory,
-// `Ring` the layout between two fused steps (FP32: the register pairs as they are; 16-bit storage:
-// the codes of one pair in a word).
-template <typename S, bool SHIFTED, int V>
+// V populations of one direction as V/2 pairs (nodes k, k + V/2): `Mem` is their layout in memory, `Ring`
+// that between two fused steps, a pair as it lies in registers.  LBM_F32 is rounded to f = g + w wherever a
+// step of its own would store it.
+template <bool SHIFTED, int V>
 struct RowCodec {
     static constexpr int HV = V / 2;
-    using Mem = typename Raw<V * (int)sizeof(S)>::T;
-    using Ring = typename Raw<2 * (int)sizeof(S)>::T;
-    __device__ static __forceinline__ void unshift(int j, f32x2 (&p)[HV]) {
-        if constexpr (!SHIFTED) {
-#pragma unroll
-            for (int k = 0; k < HV; ++k) p[k] = rsub(p[k], f32x2(wd(j)));
-        }
-    }
-    __device__ static __forceinline__ float to(S s) {
-        return St<S>::to(s);
-    }
-    __device__ static __forceinline__ S from(float v) {
-        return St<S>::from(v);
-    }
+    using Mem = typename Raw<V * 4>::T;
+    using Ring = typename Raw<8>::T;
+    __device__ static __forceinline__ f32x2 in(f32x2 p, int j) { return SHIFTED ? p : rsub(p, f32x2(wd(j))); }
+    __device__ static __forceinline__ f32x2 out(f32x2 p, int j) { return SHIFTED ? p : radd(p, f32x2(wd(j))); }
     __device__ static __forceinline__ void load(Mem r, int j, f32x2 (&p)[HV]) {
-        union { Mem u; S s[V]; } b;
+        union { Mem u; float s[V]; } b;
         b.u = r;
 #pragma unroll
-        for (int k = 0; k < HV; ++k) p[k] = f32x2(to(b.s[k]), to(b.s[k + HV]));
-        unshift(j, p);
+        for (int k = 0; k < HV; ++k) p[k] = in(f32x2(b.s[k], b.s[k + HV]), j);
     }
     __device__ static __forceinline__ Mem store(const f32x2 (&p)[HV], int j) {
-        union { Mem u; S s[V]; } b;
+        union { Mem u; float s[V]; } b;
 #pragma unroll
         for (int k = 0; k < HV; ++k) {
-            const f32x2 v = SHIFTED ? p[k] : radd(p[k], f32x2(wd(j)));
-            b.s[k] = from(v.lo());
-            b.s[k + HV] = from(v.hi());
+            const f32x2 v = out(p[k], j);
+            b.s[k] = v.lo();
+            b.s[k + HV] = v.hi();
         }
         return b.u;
     }
@@ -74,31 +63,26 @@ struct RowCodec {
     __device__ static __forceinline__ void get(const Ring* r, int j, f32x2 (&p)[HV]) {
 #pragma unroll
         for (int k = 0; k < HV; ++k) {
-            union { Ring u; S s[2]; } b;
+            union { Ring u; float s[2]; } b;
             b.u = r[32 * k];
-            p[k] = f32x2(to(b.s[0]), to(b.s[1]));
+            p[k] = in(f32x2(b.s[0], b.s[1]), j);
         }
-        unshift(j, p);
     }
     __device__ static __forceinline__ void put(Ring* r, const f32x2 (&p)[HV], int j) {
 #pragma unroll
         for (int k = 0; k < HV; ++k) {
-            const f32x2 v = SHIFTED ? p[k] : radd(p[k], f32x2(wd(j)));
-            union { Ring u; S s[2]; } b;
-            b.s[0] = from(v.lo());
-            b.s[1] = from(v.hi());
+            const f32x2 v = out(p[k], j);
+            union { Ring u; float s[2]; } b;
+            b.s[0] = v.lo();
+            b.s[1] = v.hi();
             r[32 * k] = b.u;
         }
     }
     // what put and get make of values that stay in registers
     __device__ static __forceinline__ void round(int j, f32x2 (&p)[HV]) {
-        if constexpr (sizeof(S) != 4 || !SHIFTED) {
+        if constexpr (!SHIFTED) {
 #pragma unroll
-            for (int k = 0; k < HV; ++k) {
-                const f32x2 v = SHIFTED ? p[k] : radd(p[k], f32x2(wd(j)));
-                p[k] = f32x2(to(from(v.lo())), to(from(v.hi())));
-            }
-            unshift(j, p);
+            for (int k = 0; k < HV; ++k) p[k] = in(out(p[k], j), j);
         }
     }
 };
@@ -130,7 +114,8 @@ template <typename S, bool SHIFTED, int V, int T, bool FULL, int HINT, typename 
 __device__ __forceinline__ void march(const S* __restrict__ src, S* __restrict__ dst, const CavityView<float>& cv,
                                       int lane, int xs, int y0, int y1, int steps, const Probes& probes, long long t0,
                                       void* ring_v) {
-    using Codec = RowCodec<S, SHIFTED, V>;
+    using Codec = RowCodec<SHIFTED, V>;
+    static_assert(sizeof(S) == 4, "FP32 storage");
     using Mem = typename Codec::Mem;
     using Ring = typename Codec::Ring;
     using G = StripGeometry<V, T>;

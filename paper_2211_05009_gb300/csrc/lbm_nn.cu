@@ -275,7 +275,6 @@ __global__ void k_up2_back(const float* __restrict__ dy, int C, int h, int w, fl
     dx[i] = STORE ? v : dx[i] + v;
 }
 
-// Number of valid pixels (mask is 0/1) into cnt[0].
 // Partial sums of mask and of mask (base + out - target)_0 per block: the count n and, over n, the
 // mean density-channel error, which the loss ignores.
 constexpr int kStatBlocks = 64;
@@ -1167,7 +1166,8 @@ extern "C" int lbm_net_backward(lbm_net* n, const float* in, const float* base, 
     Graph g = make_graph(n->ch);
     const long long P = (long long)H * W;
     const int nb = 512;
-    // loss and dL/d(out) (into the dZ scratch, which backward copies before reusing it)
+    // loss and dL/d(out) into the dZ scratch, which the default back end reads in place and the others copy
+    // before they reuse it
     double* stat_part = n->parts + nb;
     k_mask_stats<<<kStatBlocks, 256, 0, n->stream>>>(mask, n->act[g.out], base, target, P, stat_part);
     k_mse<<<nb, 256, 0, n->stream>>>(n->act[g.out], base, target, mask, P, stat_part, n->d_loss, n->dz, n->parts);
