@@ -48,9 +48,11 @@ TilePlan tile_plan(int nx, int ny) {
     p.steps = kTileSteps;
     p.ow = kTileCols - 2 * p.steps;
     // Rows so that the row pairs of a step fill the warps once (10 + 2 x 3 rows, 8 pairs) or twice
-    // (24): the taller tile computes fewer nodes twice, the lower one makes more blocks.
+    // (24): the taller tile computes fewer nodes twice, the lower one makes more blocks.  The lower one
+    // up to two blocks for each of the 152 SMs (us a step, low / high: f32s 96^2 1.1 / 1.5, 192x380 with 304 low
+    // blocks 1.37 / 1.60, 288x255 with 312 1.50 / 1.61; q16s 1.6 / 2.5, 2.36 / 2.58, 2.71 / 2.58).
     const int cols = (nx + p.ow - 1) / p.ow;
-    p.oh = (long long)cols * ((ny + 9) / 10) <= 2 * 148 ? kTileLow : kTileHigh;
+    p.oh = (long long)cols * ((ny + 9) / 10) <= 2 * 152 ? kTileLow : kTileHigh;
     // a wall is never the only column or row of a tile; columns move by a copy's alignment
     p.shift_x = nx % p.ow == 1 ? 4 : 0;
     p.shift_y = ny % p.oh == 1 ? 1 : 0;
