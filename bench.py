@@ -14,8 +14,10 @@ The metric is lattice updates per second (GLUPS = nx*ny*100 per step / time).
   e2e       the same metric through the C ABI with HOST buffers: every step uploads the initial
             macroscopic field (rho, u_x, u_y; FP64, pinned) with lbm_set_moments, advances 100
             steps, reads the residual and downloads rho, u_x, u_y with lbm_moments
-  roofline  the step kernel: 18 populations x 4 bytes per node and launch / the average duration of a
-            launch (launch shape 6 advances four steps per launch, and its bound is the FP32 pipe)
+  roofline  the step kernel over the average duration of a launch, against what bounds it.  One step per
+            launch: HBM, 18 populations x 4 bytes per node.  Launch shape 6 (four steps per launch): the
+            FP32 pipe, 61 operations per node and step, against half the measured multiply-add FLOP rate;
+            its one pass over the populations per launch stands beside it as "hbm"
   cpu_baseline  the FP64 CPU oracle on a bounded sample of the same workload (first steps of
             the same 2048^2 cavity): its OpenMP build on every host core, and the plain build
             on one thread
@@ -46,6 +48,7 @@ BYTES_PER_LU = 18 * 4  # 9 populations read + 9 written, 4 bytes each
 METRIC = "D2Q9 GLUPS (fused step, lattice updates per second)"
 WORKLOAD = "square lid-driven cavity 2048x2048, Re=8000, U=0.05, FP32 arithmetic, FP32 shifted-deviation storage"
 FUSED_SHAPE, FUSED_STEPS = 6, 4  # the march: steps per launch
+OPS_PER_LU = 61  # FP32 operations of a node's moments and collision on shifted FP32 storage
 PROFILES = {False: ("k_step_f32s_2048x2048.txt", ["lbm_step_kernel.cuh"]),
             True: ("k_march_f32s_2048x2048.txt", ["lbm_march.cuh", "lbm_step_kernel.cuh"])}
 
@@ -304,6 +307,12 @@ def our_arm(args, rank, world, local_rank):
     peak, peak_kind = measured_peak()
     algo_bytes = BYTES_PER_LU * NX * NY
     achieved = algo_bytes / step_kernel_s / 1e9
+    hbm = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak, "peak_kind": peak_kind}
+    bound = hbm
+    if fused:
+        ops, ops_peak = OPS_PER_LU * FUSED_STEPS * NX * NY / step_kernel_s / 1e12, B.lbm_fma_peak(fp64=False)[0] / 2e12
+        bound = {"bound": "fp32 pipe", "achieved": ops, "peak": ops_peak, "unit": "T FP32 operations/s", "frac": ops / ops_peak,
+                 "peak_kind": "measured", "hbm": hbm}
     traffic = read_profile_traffic(cfg)
     cpu = None
     if not args.no_cpu_baseline and world == 1:
@@ -327,9 +336,8 @@ def our_arm(args, rank, world, local_rank):
         "config": {"workload": WORKLOAD, "nx": NX, "ny": NY, "Re": RE, "U": U, "storage": STORAGE,
                    "lbm_steps_per_step": CHUNK, "parallelism": f"replicas{world}",
                    "l2": "population working set 302 MB > 129 MB L2; no flush"},
-        "roofline": {"bound": "fp32 pipe" if fused else "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                     "frac": achieved / peak, "traffic": traffic,
-                     "peak_kind": peak_kind, "kernel": f"{'k_march' if fused else 'k_step'}<float, shifted> launch shape {cfg}",
+        "roofline": {**bound, "traffic": traffic,
+                     "kernel": f"{'k_march' if fused else 'k_step'}<float, shifted> launch shape {cfg}",
                      "steps_per_launch": FUSED_STEPS if fused else 1,
                      "algorithmic_bytes_per_launch": algo_bytes,
                      "avg_launch_us": step_kernel_s * 1e6},

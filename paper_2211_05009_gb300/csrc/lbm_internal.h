@@ -34,10 +34,10 @@ struct StepGeometry {
 
 // Launch shapes of the time step; all give identical populations.  0..5: one step per launch (row
 // step, lbm_step_kernel.cuh).  6: kMarchSteps plain steps per launch (lbm_march.cuh) for FP32
-// storage; steps left over run as one shorter launch, checkpoint steps one by one.  The other types
-// gain nothing from fewer passes over memory and take their default row shape there: FP64 is bound by
-// its pipe, LBM_Q16S by its code conversions, and binary16 / bfloat16 meet the FP32 pipe first
-// (binary16 4096^2: fused 178 GLUPS, row step 178; 2048^2 150 against 168).
+// storage; steps left over run as one shorter launch, checkpoint steps one by one.  The other types take
+// their default row shape there: FP64 is bound by its pipe and LBM_Q16S by its code conversions; a march
+// of binary16 was tried and not kept (converting a value at a time between steps, 178 GLUPS at 4096^2 and
+// 150 at 2048^2 where the row step ran 178 and 168).
 // 7: several steps per launch in shared-memory tiles (lbm_tile.cuh), for small grids of every type
 // but FP64, whose pipe pays for nodes computed twice.
 constexpr int kStepConfigs = 8, kRowConfigs = 6, kMarchConfig = 6, kTileConfig = 7;

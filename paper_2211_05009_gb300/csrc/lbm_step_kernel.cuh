@@ -387,7 +387,7 @@ __device__ __forceinline__ Relax<C> make_relax(C omega) {
 // is 1e-5 U off after 1000 steps of 133x77 at Re 400, this form 1.5e-7 U, increments formed per
 // direction with their momentum taken out 3.6e-7 U.)
 //
-// FP64: 53 FP64 operations (72.7 instructions with the equilibrium formed per direction): the pipe
+// FP64: 54 FP64 operations (72.7 instructions with the equilibrium formed per direction): the pipe
 // issues 2 lanes per clock and SM, so the operation count is the run time (2048^2: 7.3 GLUPS then, 10.4
 // now, 0.94 of what the pipe takes for 54.1 instructions a node at 16.8 cycles).
 // out = keep g + (omega g^eq) with the pair's omega g^eq from two fused multiply-adds.
